@@ -598,11 +598,11 @@ cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const
                                 const cplx* w, int nb, cplx* lam, cplx* phi, cplx* scratch, int* status,
                                 cudaStream_t st, const cplx* eig = nullptr);
 size_t bound_states_scratch(int m, int nb);
-// kernels_eig.cu: all eigenvalues of diag + v with squared off-diagonals east_k west_{k+1}
+// kernels_eig.cu: all eigenvalues of the axis operator (diag + v, west, east; w its quadrature weights)
 // into out[m]; *ok false when the iteration did not converge (the caller falls back to QR).
 size_t eig_scratch_entries(int m);
-cudaError_t eig_aberth(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v, cplx* scratch,
-                       cplx* out, bool* ok, cudaStream_t st);
+cudaError_t eig_aberth(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v, const cplx* w,
+                       cplx* scratch, cplx* out, bool* ok, cudaStream_t st);
 cudaError_t launch_qr_spectrum(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
                                cplx* scratch, cplx* out, int* status, cudaStream_t st);
 cudaError_t launch_weight_states(int m, int nb, const cplx* w, const cplx* phi, cplx* wphi, cudaStream_t st);

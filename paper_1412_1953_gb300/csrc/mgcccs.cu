@@ -347,7 +347,7 @@ int read_status(mgcccs_handle* h) {
 int axis_states(mgcccs_handle* h, int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
                 const cplx* w, cplx* lam, cplx* phi) {
   bool ok = false;
-  MGC_CUDA(eig_aberth(m, west, east, diag, v, h->eig_ab, h->eig_vals, &ok, h->st));
+  MGC_CUDA(eig_aberth(m, west, east, diag, v, w, h->eig_ab, h->eig_vals, &ok, h->st));
   h->launches += 4;
   if (!ok) h->eig_fallbacks += 1;
   MGC_LAUNCH(launch_bound_states(m, west, east, diag, v, w, h->nb, lam, phi, h->eig_scratch, h->status, h->st,
@@ -1714,7 +1714,8 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
   const cplx* v = axis == 0 ? h->v1c : h->v2c;
   if (method == 0) {
     bool ok = false;
-    MGC_CUDA(eig_aberth(m, west, east, diag, v, h->eig_ab, h->eig_vals, &ok, h->st));
+    const cplx* w = axis == 0 ? b.w_x : b.w_y;
+    MGC_CUDA(eig_aberth(m, west, east, diag, v, w, h->eig_ab, h->eig_vals, &ok, h->st));
     if (!ok) return MGCCCS_EBREAKDOWN;
   } else {
     MGC_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), h->st));
