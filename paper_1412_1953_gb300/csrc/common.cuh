@@ -593,10 +593,9 @@ cudaError_t launch_bpcr_setup(const StencilView& s, cplx* fac, cplx* scratch, in
 // u = A_c^{-1} f through the factors; buf holds 2 mx my complex entries
 template <class C>
 cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const C* f, C* u, cplx* buf, cudaStream_t st);
-// eig: all m eigenvalues when already computed (eig_aberth), else null (FP64 QR inside)
-cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
-                                const cplx* w, int nb, cplx* lam, cplx* phi, cplx* scratch, int* status,
-                                cudaStream_t st, const cplx* eig = nullptr);
+// eig: all m eigenvalues (eig_aberth, or launch_qr_spectrum when that did not converge)
+cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const cplx* v, const cplx* w, int nb,
+                                cplx* lam, cplx* phi, cplx* scratch, int* status, cudaStream_t st, const cplx* eig);
 size_t bound_states_scratch(int m, int nb);
 // kernels_eig.cu: all eigenvalues of the axis operator (diag + v, west, east; w its quadrature weights)
 // into out[m]; *ok false when the iteration did not converge (the caller falls back to QR).

@@ -5,12 +5,11 @@
 //    contour.
 //  * Diagonal D of H - E and omega/D per node, potentials injected at coincident nodes.
 //  * Dense inverse of the coarsest-level operator (Gauss-Jordan, partial pivoting).
-//  * Bound states of H1, H2 (Eq. (9)): all eigenvalues by root-free implicit QR on the
-//    squared off-diagonals (Pal-Walker-Kahan form) applied without conjugation to the
-//    complex-symmetric tridiagonal; the n_b with smallest real part are refined by
-//    inverse and Rayleigh-quotient iteration with a pivoted tridiagonal LU, normalised
-//    bilinearly, int phi^2 dz = 1 (Sec. 3.1, Remark 3), then two shift-and-invert steps
-//    and a bilinear Rayleigh quotient (Sec. 5.1.2, Sec. 5.2).
+//  * Bound states of H1, H2 (Eq. (9)): of all eigenvalues (kernels_eig.cu, or here the
+//    root-free implicit QR on the squared off-diagonals, Pal-Walker-Kahan form, applied
+//    without conjugation to the complex-symmetric tridiagonal) the n_b with smallest real
+//    part are refined by Rayleigh-quotient iteration and two shift-and-invert steps (Sec.
+//    5.1.2, Sec. 5.2), normalised bilinearly, int phi^2 dz = 1 (Sec. 3.1, Remark 3).
 //  * Channel potentials V^A, V^B (Sec. 4.2) and the cyclic-reduction factors of the
 //    coupled-channel systems (Eqs. (28)-(29)).
 #include <algorithm>
@@ -231,212 +230,294 @@ __device__ bool qr_rootfree_eigenvalues(int m, cplx* a, cplx* b2) {
   return true;
 }
 
-// Pivoted LU of the tridiagonal T - sigma I (T: sub `west` (row k couples to k-1),
-// diagonal `diag + v`, super `east`).  Row k of U holds u0 (col k), u1 (col k+1),
-// u2 (col k+2); mu[k] is the multiplier of step k and sw[k] says whether rows k, k+1
-// were exchanged.
-struct TriLU {
-  cplx *u0, *u1, *u2, *mu;
-  int* sw;
+// ---- refinement of the bound states: one block per state.
+//
+// A shift-and-invert step at an eigenvalue z known to rounding needs no elimination: with the
+// quadrature weights w_k (w_k east_k = w_{k+1} west_{k+1}, diag_k = -(west_k + east_k)) and the
+// flux F_k = w_k east_k (u_{k+1} - u_k), the rows of (H1 - z) u = 0 read
+//   F_k = F_{k-1} + w_k (z - v_k) u_k,   u_{k+1} = u_k + F_k / (w_k east_k),
+// and the solution of (H1 - z) x = gamma e_r is the solution uL started at the first row for
+// k <= r and the one uR started at the last row for k >= r, matched at r.  r is taken where
+// |uL uR|, proportional to the diagonal of the inverse, is largest, so neither is carried into
+// a region where it decays.  Both are linear recurrences: a thread forms the 2 x 2 transfer
+// matrix of its rows, a scan over the threads gives each its starting vector, and it then walks
+// its rows (four warps from either end).  Values carry power-of-two exponents of their own.
+constexpr int BS_THREADS = 256, BS_HALF = BS_THREADS / 2, BS_WARPS = BS_HALF / 32;
+constexpr int BS_SMEM = 200 * 1024;
+
+// Workspace of a state: 1/(w east), uL (then x), uR, and the exponents of uL and uR.
+__host__ __device__ constexpr size_t states_bytes(int m) { return (sizeof(cplx) * 3 + sizeof(int) * 2) * (size_t)m; }
+
+__device__ __forceinline__ int hi_max(int m, cplx z) {
+  return max(m, max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff));
+}
+// 2^-e for the exponent e of the high word hm, which is added to *ex (nothing for zero and beyond 2^1000).
+__device__ __forceinline__ double pow2_take(int hm, int* ex) {
+  const int e = (hm >> 20) - 1023;
+  if (hm < (1 << 20) || e > 1000) return 1.0;
+  *ex += e;
+  return __hiloint2double((1023 - e) << 20, 0);
+}
+
+// (u, F) after = [a b; c d] (u, F) before, times 2^e.
+struct Transfer2 {
+  cplx a, b, c, d;
+  int e;
 };
+__device__ __forceinline__ void rescale(Transfer2& t) {
+  const double f = pow2_take(hi_max(hi_max(hi_max(hi_max(0, t.a), t.b), t.c), t.d), &t.e);
+  t.a = cscal(f, t.a); t.b = cscal(f, t.b); t.c = cscal(f, t.c); t.d = cscal(f, t.d);
+}
+__device__ __forceinline__ void rescale(cplx& u, cplx& F, int& e) {
+  const double f = pow2_take(hi_max(hi_max(0, u), F), &e);
+  u = cscal(f, u);
+  F = cscal(f, F);
+}
+// t <- t o s (s acts first)
+__device__ __forceinline__ Transfer2 compose(const Transfer2& t, const Transfer2& s) {
+  Transfer2 r;
+  r.a = cfma(t.a, s.a, cmul(t.b, s.c));
+  r.b = cfma(t.a, s.b, cmul(t.b, s.d));
+  r.c = cfma(t.c, s.a, cmul(t.d, s.c));
+  r.d = cfma(t.c, s.b, cmul(t.d, s.d));
+  r.e = t.e + s.e;
+  rescale(r);
+  return r;
+}
+__device__ __forceinline__ cplx shfl_up_c(cplx z, int o) {
+  return cmk(__shfl_up_sync(0xffffffffu, z.x, o), __shfl_up_sync(0xffffffffu, z.y, o));
+}
+__device__ __forceinline__ Transfer2 shfl_up_t(const Transfer2& t, int o) {
+  return Transfer2{shfl_up_c(t.a, o), shfl_up_c(t.b, o), shfl_up_c(t.c, o), shfl_up_c(t.d, o),
+                   __shfl_up_sync(0xffffffffu, t.e, o)};
+}
+constexpr int HI_BIG = (1023 + 400) << 20, HI_SMALL = (1023 - 400) << 20;   // 2^400, 2^-400
+__device__ __forceinline__ bool off_range(int hm) { return hm > HI_BIG || hm < HI_SMALL; }
 
-__device__ void tri_lu(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v, cplx sigma,
-                       TriLU lu) {
-  cplx Dk = csub(cadd(diag[0], v[0]), sigma);
-  cplx U1 = (m > 1) ? east[0] : cmk(0.0, 0.0);
-  for (int k = 0; k < m - 1; ++k) {
-    cplx L = west[k + 1];
-    cplx dn = csub(cadd(diag[k + 1], v[k + 1]), sigma);
-    cplx cn = (k + 2 < m) ? east[k + 1] : cmk(0.0, 0.0);
-    if (cabs2(L) > cabs2(Dk)) {
-      // exchange: pivot row is row k+1
-      cplx mu = cdiv(Dk, L);
-      lu.u0[k] = L; lu.u1[k] = dn; lu.u2[k] = cn; lu.mu[k] = mu; lu.sw[k] = 1;
-      Dk = cfms(mu, dn, U1);
-      U1 = cneg(cmul(mu, cn));
-    } else {
-      cplx mu = (Dk.x == 0.0 && Dk.y == 0.0) ? cmk(0.0, 0.0) : cdiv(L, Dk);
-      lu.u0[k] = Dk; lu.u1[k] = U1; lu.u2[k] = cmk(0.0, 0.0); lu.mu[k] = mu; lu.sw[k] = 0;
-      Dk = cfms(mu, U1, dn);
-      U1 = cn;
+// Sums of two complex values over the block, to every thread (fixed order).
+__device__ void bs_sum2(cplx& a, cplx& b, double (*sh)[BS_THREADS / 32]) {
+  double v[4] = {a.x, a.y, b.x, b.y};
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_down_sync(0xffffffffu, v[c], o);
+    if ((threadIdx.x & 31) == 0) sh[c][threadIdx.x >> 5] = v[c];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    v[c] = sh[c][0];
+#pragma unroll
+    for (int w = 1; w < BS_THREADS / 32; ++w) v[c] += sh[c][w];
+  }
+  __syncthreads();
+  a = cmk(v[0], v[1]);
+  b = cmk(v[2], v[3]);
+}
+
+// The entry of largest key (lowest index on ties) over the block, to every thread.
+__device__ void bs_argmax(double& key, int& idx, double (*sh)[BS_THREADS / 32]) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double k2 = __shfl_xor_sync(0xffffffffu, key, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
+    if (k2 > key || (k2 == key && i2 < idx)) { key = k2; idx = i2; }
+  }
+  if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = key; sh[1][threadIdx.x >> 5] = (double)idx; }
+  __syncthreads();
+  key = sh[0][0];
+  idx = (int)sh[1][0];
+#pragma unroll
+  for (int w = 1; w < BS_THREADS / 32; ++w) {
+    const double k2 = sh[0][w];
+    const int i2 = (int)sh[1][w];
+    if (k2 > key || (k2 == key && i2 < idx)) { key = k2; idx = i2; }
+  }
+  __syncthreads();
+}
+
+// Block q: the eigenvalue with the q-th smallest real part (ties: lower index) of the m given,
+// Rayleigh-quotient iteration from it (each step a shift-and-invert step and the bilinear
+// quotient of its result), the paper's two shift-and-invert steps, and the bilinear
+// normalisation.  The quotient x^T W H1 x = sum w v x^2 - sum w east (x_{k+1} - x_k)^2 is summed
+// without the cancellation of H1 x.  Bound by the FP64 pipe of the block's one SM (a warp's FP64
+// instruction occupies its quarter of an SM for 64 cycles however few lanes need it).  1023
+// rows, three states: 45.8 ms with one thread per state walking pivoted tridiagonal LU factors
+// in global memory, 4.3 ms with the elimination run from both ends by two threads in shared
+// memory, 0.26 ms so.
+__global__ void __launch_bounds__(BS_THREADS) k_bound_states(int m, const cplx* __restrict__ west,
+                                                             const cplx* __restrict__ east,
+                                                             const cplx* __restrict__ v, const cplx* __restrict__ w,
+                                                             cplx* __restrict__ lam, cplx* __restrict__ phi,
+                                                             cplx* __restrict__ scratch, int in_smem, int* status,
+                                                             const cplx* __restrict__ eig) {
+  extern __shared__ cplx bs_work[];
+  __shared__ double sh[4][BS_THREADS / 32];
+  __shared__ Transfer2 tot[2][BS_WARPS];
+  __shared__ int no_eig;
+  const int q = blockIdx.x, t = threadIdx.x;
+  if (t == 0) no_eig = *status & MGC_ST_EIG;         // one read: another block may set it meanwhile
+  __syncthreads();
+  if (no_eig) return;
+  cplx* base = in_smem ? bs_work : scratch + (size_t)q * ((states_bytes(m) + sizeof(cplx) - 1) / sizeof(cplx));
+  cplx *ic = base, *uL = base + m, *uR = base + 2 * (size_t)m, *x = uL;
+  int *eL = reinterpret_cast<int*>(base + 3 * (size_t)m), *eR = eL + m;
+  const cplx zero = cmk(0.0, 0.0), one = cmk(1.0, 0.0);
+  // the q-th smallest real part: q + 1 passes, each for the least (value, index) beyond the last
+  double last = 0.0;
+  int li = -1;
+  for (int s = 0; s <= q; ++s) {
+    double best = -INFINITY;
+    int bi = m;
+    for (int k = t; k < m; k += BS_THREADS) {
+      const double r = eig[k].x;
+      if (li >= 0 && !(r > last || (r == last && k > li))) continue;
+      if (bi == m || -r > best) { best = -r; bi = k; }
     }
+    bs_argmax(best, bi, sh);
+    last = -best;
+    li = bi < m ? bi : 0;
   }
-  lu.u0[m - 1] = Dk;
-  lu.u1[m - 1] = cmk(0.0, 0.0);
-  lu.u2[m - 1] = cmk(0.0, 0.0);
-}
+  cplx lmb = eig[li];
+  for (int k = t; k < m; k += BS_THREADS) ic[k] = cdiv(one, cmul(w[k], east[k]));
+  const int dir = t / BS_HALF, g = t % BS_HALF, wq = g >> 5, lane = t & 31;
+  const int cn = (m + BS_HALF - 1) / BS_HALF;
+  const int g0 = min(g * cn, m), g1 = min(g0 + cn, m);   // this thread's steps, counted from its end
+  const cplx cs = cmul(w[0], west[0]);
 
-// Solve with the factors in place on b; an exactly zero pivot (the shift equals an
-// eigenvalue to the last bit) is replaced by a tiny one, the usual inverse-iteration device.
-__device__ void tri_solve(int m, TriLU lu, cplx* b, double tiny) {
-  for (int k = 0; k < m - 1; ++k) {
-    if (lu.sw[k]) { cplx t = b[k]; b[k] = b[k + 1]; b[k + 1] = t; }
-    b[k + 1] = cfms(lu.mu[k], b[k], b[k + 1]);
+  // x = the solution of (H1 - z) x = gamma e_r, x_r = 1
+  auto shift_invert = [&](cplx z) {
+    __syncthreads();
+    Transfer2 T{one, zero, zero, one, 0};
+    for (int p = g0; p < g1; ++p) {
+      const int k = dir ? m - 1 - p : p;
+      const cplx qk = cmul(w[k], csub(z, v[k])), i = ic[k];
+      if (dir == 0) {
+        T.c = cfma(qk, T.a, T.c); T.d = cfma(qk, T.b, T.d);
+        T.a = cfma(i, T.c, T.a);  T.b = cfma(i, T.d, T.b);
+      } else {
+        T.a = cfms(i, T.c, T.a);  T.b = cfms(i, T.d, T.b);
+        T.c = cfms(qk, T.a, T.c); T.d = cfms(qk, T.b, T.d);
+      }
+      if (off_range(hi_max(hi_max(0, T.a), T.b))) rescale(T);
+    }
+    rescale(T);
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const Transfer2 s = shfl_up_t(T, o);
+      if (lane >= o) T = compose(T, s);
+    }
+    if (lane == 31) tot[dir][wq] = T;
+    Transfer2 E = shfl_up_t(T, 1);
+    if (lane == 0) E = Transfer2{one, zero, zero, one, 0};
+    __syncthreads();
+    // (u, F) before the first row, carried to this thread's first step
+    cplx u = dir ? zero : one, F = dir ? one : cs;
+    int e = 0;
+    auto act = [&](const Transfer2& s) {
+      const cplx u2 = cfma(s.a, u, cmul(s.b, F)), F2 = cfma(s.c, u, cmul(s.d, F));
+      u = u2;
+      F = F2;
+      e += s.e;
+      rescale(u, F, e);
+    };
+    for (int b = 0; b < wq; ++b) act(tot[dir][b]);
+    act(E);
+    for (int p = g0; p < g1; ++p) {
+      const int k = dir ? m - 1 - p : p;
+      const cplx qk = cmul(w[k], csub(z, v[k])), i = ic[k];
+      if (dir == 0) {
+        uL[k] = u;
+        eL[k] = e;
+        F = cfma(qk, u, F);
+        u = cfma(i, F, u);
+      } else {
+        u = cfms(i, F, u);
+        uR[k] = u;
+        eR[k] = e;
+        F = cfms(qk, u, F);
+      }
+      if (off_range(hi_max(hi_max(0, u), F))) rescale(u, F, e);
+    }
+    __syncthreads();
+    // log2 |uL uR| to within one (the high words as fixed-point numbers)
+    double key = -INFINITY;
+    int r = m;
+    for (int k = t; k < m; k += BS_THREADS) {
+      const double a = cabs1(uL[k]), b = cabs1(uR[k]);
+      if (!(a > 0.0) || !(b > 0.0)) continue;
+      const double l = (double)(eL[k] + eR[k]) + 0x1p-20 * (double)(__double2hiint(a) + __double2hiint(b));
+      if (r == m || l > key) { key = l; r = k; }
+    }
+    bs_argmax(key, r, sh);
+    if (r >= m) r = 0;
+    const cplx sl = cdiv(one, uL[r]), sr = cdiv(one, uR[r]);
+    const int el = eL[r], er = eR[r];
+    __syncthreads();
+    for (int k = t; k < m; k += BS_THREADS) {
+      const cplx y = k <= r ? cmul(sl, uL[k]) : cmul(sr, uR[k]);
+      const int sh2 = k <= r ? eL[k] - el : eR[k] - er;
+      x[k] = cmk(scalbn(y.x, sh2), scalbn(y.y, sh2));
+    }
+    __syncthreads();
+  };
+  // bilinear Rayleigh quotient x^T W H1 x / x^T W x
+  auto quotient = [&]() {
+    cplx num = zero, den = zero;
+    for (int k = t; k < m; k += BS_THREADS) {
+      const cplx xk = x[k], d = csub(k + 1 < m ? x[k + 1] : zero, xk);
+      const cplx wx2 = cmul(w[k], cmul(xk, xk));
+      den = cadd(den, wx2);
+      num = cfma(v[k], wx2, num);
+      num = cfms(cmul(w[k], east[k]), cmul(d, d), num);
+      if (k == 0) num = cfms(cs, cmul(xk, xk), num);
+    }
+    bs_sum2(num, den, sh);
+    return cdiv(num, den);
+  };
+  for (int it = 0; it < 6; ++it) {
+    shift_invert(lmb);
+    const cplx ln = quotient();
+    const bool conv = cabs1(csub(ln, lmb)) <= 1e-14 * fmax(1.0, cabs1(ln));
+    lmb = ln;
+    if (conv) break;
   }
-  for (int k = m - 1; k >= 0; --k) {
-    cplx t = b[k];
-    if (k + 1 < m) t = cfms(lu.u1[k], b[k + 1], t);
-    if (k + 2 < m) t = cfms(lu.u2[k], b[k + 2], t);
-    cplx piv = lu.u0[k];
-    if (piv.x == 0.0 && piv.y == 0.0) piv = cmk(tiny, 0.0);
-    b[k] = cdiv(t, piv);
+  for (int it = 0; it < 2; ++it) {
+    shift_invert(lmb);
+    lmb = quotient();
   }
-}
-
-// Bilinear normalisation sum w x^2 = 1, then Re x > 0 at the entry of largest modulus.
-__device__ void bilinear_normalise(int m, const cplx* w, cplx* x) {
-  cplx s = cmk(0.0, 0.0);
-  for (int k = 0; k < m; ++k) s = cfma(w[k], cmul(x[k], x[k]), s);
-  cplx inv = cdiv(cmk(1.0, 0.0), csqrt_p(s));
+  // bilinear normalisation sum w x^2 = 1, then Re x > 0 at the entry of largest modulus
+  cplx s = zero, unused = zero;
+  for (int k = t; k < m; k += BS_THREADS) s = cfma(w[k], cmul(x[k], x[k]), s);
+  bs_sum2(s, unused, sh);
+  cplx inv = cdiv(one, csqrt_p(s));
   double best = -1.0;
   int kb = 0;
-  for (int k = 0; k < m; ++k) {
-    x[k] = cmul(x[k], inv);
-    double a = cabs2(x[k]);
+  for (int k = t; k < m; k += BS_THREADS) {
+    const double a = cabs2(cmul(x[k], inv));
     if (a > best) { best = a; kb = k; }
   }
-  if (x[kb].x < 0.0)
-    for (int k = 0; k < m; ++k) x[k] = cneg(x[k]);
+  bs_argmax(best, kb, sh);
+  if (cmul(x[kb], inv).x < 0.0) inv = cneg(inv);
+  bool fin = isfinite(lmb.x) && isfinite(lmb.y);
+  for (int k = t; k < m; k += BS_THREADS) {
+    const cplx y = cmul(x[k], inv);
+    phi[(size_t)q * m + k] = y;
+    fin = fin && isfinite(y.x) && isfinite(y.y);
+  }
+  if (t == 0) lam[q] = lmb;
+  if (!fin) atomicOr(status, MGC_ST_EIG);
 }
 
-__device__ void max_normalise(int m, cplx* x) {
-  double best = 0.0;
-  for (int k = 0; k < m; ++k) best = fmax(best, cabs1(x[k]));
-  if (best > 0.0) {
-    double s = 1.0 / best;
-    for (int k = 0; k < m; ++k) x[k] = cscal(s, x[k]);
-  }
+// Two states that refined onto the same eigenvalue mean the estimates were too poor.
+__global__ void k_states_distinct(int nb, const cplx* __restrict__ lam, int* status) {
+  const int a = threadIdx.x / MGC_MAX_NB, b = threadIdx.x % MGC_MAX_NB;
+  if (a < b && b < nb && cabs1(csub(lam[a], lam[b])) <= 1e-10 * fmax(1.0, cabs1(lam[a])))
+    atomicOr(status, MGC_ST_EIG);
 }
 
-__device__ cplx rayleigh(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
-                         const cplx* w, const cplx* x) {
-  cplx acc = cmk(0.0, 0.0);
-  for (int k = 0; k < m; ++k) {
-    cplx hx = cmul(cadd(diag[k], v[k]), x[k]);
-    if (k > 0) hx = cfma(west[k], x[k - 1], hx);
-    if (k + 1 < m) hx = cfma(east[k], x[k + 1], hx);
-    acc = cfma(cmul(x[k], w[k]), hx, acc);
-  }
-  return acc;
-}
-
-// bilinear Rayleigh quotient x^T W H x / x^T W x (x not normalised)
-__device__ cplx rayleigh_ratio(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
-                               const cplx* w, const cplx* x) {
-  cplx num = cmk(0.0, 0.0), den = cmk(0.0, 0.0);
-  for (int k = 0; k < m; ++k) {
-    cplx hx = cmul(cadd(diag[k], v[k]), x[k]);
-    if (k > 0) hx = cfma(west[k], x[k - 1], hx);
-    if (k + 1 < m) hx = cfma(east[k], x[k + 1], hx);
-    cplx xw = cmul(x[k], w[k]);
-    num = cfma(xw, hx, num);
-    den = cfma(xw, x[k], den);
-  }
-  return cdiv(num, den);
-}
-
-// Eigenvalues by root-free QR (thread 0), the n_b with the smallest real part; then per
-// state (thread q): inverse iteration at the eigenvalue, Rayleigh-quotient iteration,
-// bilinear normalisation, and the paper's two shift-and-invert steps.  Coinciding refined
-// eigenvalues flag a failure.
-__global__ void __launch_bounds__(32) k_bound_states(int m, const cplx* __restrict__ west,
-                                                     const cplx* __restrict__ east, const cplx* __restrict__ diag,
-                                                     const cplx* __restrict__ v, const cplx* __restrict__ w, int nb,
-                                                     cplx* __restrict__ lam, cplx* __restrict__ phi,
-                                                     cplx* __restrict__ scratch, int* status,
-                                                     const cplx* __restrict__ eig) {
-  __shared__ cplx sel[MGC_MAX_NB];
-  __shared__ cplx fin_l[MGC_MAX_NB];
-  __shared__ int ok;
-  const int q = threadIdx.x;
-  cplx* d = scratch;            // m
-  cplx* e2 = scratch + m;       // m
-  if (q == 0) {
-    if (eig) {
-      // all eigenvalues given (the Ehrlich-Aberth iteration of kernels_eig.cu)
-      for (int k = 0; k < m; ++k) {
-        d[k] = eig[k];
-        e2[k] = cmk(0.0, 0.0);
-      }
-      ok = 1;
-    } else {
-      // squared off-diagonals of the symmetric form: e_k^2 = east_k * west_{k+1}
-      for (int k = 0; k < m; ++k) {
-        d[k] = cadd(diag[k], v[k]);
-        e2[k] = (k + 1 < m) ? cmul(east[k], west[k + 1]) : cmk(0.0, 0.0);
-      }
-      ok = qr_rootfree_eigenvalues(m, d, e2) ? 1 : 0;
-    }
-    if (ok) {
-      // the nb eigenvalues with the smallest real part, ascending (ties: lower index)
-      for (int s = 0; s < nb; ++s) {
-        int kb = -1;
-        for (int k = 0; k < m; ++k) {
-          if (e2[k].x == 1.0e300) continue;            // already taken
-          if (kb < 0 || d[k].x < d[kb].x) kb = k;
-        }
-        sel[s] = d[kb];
-        e2[kb] = cmk(1.0e300, 0.0);
-      }
-    } else {
-      atomicOr(status, MGC_ST_EIG);
-    }
-  }
-  __syncthreads();
-  if (ok && q < nb) {
-    cplx* base = scratch + 2 * m + (size_t)q * 5 * m;
-    TriLU lu{base, base + m, base + 2 * m, base + 3 * m,
-             reinterpret_cast<int*>(scratch + 2 * m + (size_t)nb * 5 * m) + (size_t)q * m};
-    cplx* x = base + 4 * m;
-    double scale = 0.0;
-    for (int k = 0; k < m; ++k) scale = fmax(scale, cabs1(cadd(diag[k], v[k])));
-    const double tiny = 1e-300 + 1e-16 * scale;
-    cplx lmb = sel[q];
-    for (int k = 0; k < m; ++k) x[k] = cmk(1.0, 0.0);
-    // two inverse-iteration steps at the QR eigenvalue
-    tri_lu(m, west, east, diag, v, lmb, lu);
-    for (int it = 0; it < 2; ++it) {
-      tri_solve(m, lu, x, tiny);
-      max_normalise(m, x);
-    }
-    // Rayleigh-quotient iteration to the double-precision eigenvalue
-    for (int it = 0; it < 6; ++it) {
-      cplx ln = rayleigh_ratio(m, west, east, diag, v, w, x);
-      const bool conv = cabs1(csub(ln, lmb)) <= 1e-14 * fmax(1.0, cabs1(ln));
-      lmb = ln;
-      tri_lu(m, west, east, diag, v, lmb, lu);
-      tri_solve(m, lu, x, tiny);
-      max_normalise(m, x);
-      if (conv) break;
-    }
-    bilinear_normalise(m, w, x);
-    // two shift-and-invert refinement steps with a Rayleigh-quotient update
-    for (int it = 0; it < 2; ++it) {
-      tri_lu(m, west, east, diag, v, lmb, lu);
-      tri_solve(m, lu, x, tiny);
-      max_normalise(m, x);
-      bilinear_normalise(m, w, x);
-      lmb = rayleigh(m, west, east, diag, v, w, x);
-    }
-    bool fin = isfinite(lmb.x) && isfinite(lmb.y);
-    for (int k = 0; k < m; ++k) {
-      phi[(size_t)q * m + k] = x[k];
-      fin = fin && isfinite(x[k].x) && isfinite(x[k].y);
-    }
-    lam[q] = lmb;
-    fin_l[q] = lmb;
-    if (!fin) atomicOr(status, MGC_ST_EIG);
-  }
-  __syncthreads();
-  if (ok && q == 0) {
-    // two states that refined onto the same eigenvalue mean the estimates were too poor
-    for (int a = 0; a < nb; ++a)
-      for (int b = a + 1; b < nb; ++b)
-        if (cabs1(csub(fin_l[a], fin_l[b])) <= 1e-10 * fmax(1.0, cabs1(fin_l[a]))) atomicOr(status, MGC_ST_EIG);
-  }
-}
-
-// All eigenvalues by the FP64 root-free QR (one thread), for the spectrum entry point.
+// All eigenvalues by the FP64 root-free QR (one thread): the spectrum entry point's method 1, and
+// setup's fallback when the Ehrlich-Aberth iteration does not converge.
 __global__ void k_qr_spectrum(int m, const cplx* __restrict__ west, const cplx* __restrict__ east,
                               const cplx* __restrict__ diag, const cplx* __restrict__ v, cplx* __restrict__ scratch,
                               cplx* __restrict__ out, int* status) {
@@ -681,14 +762,22 @@ cudaError_t launch_coarse_inverse(const StencilView& s, cplx* aug, cplx* Ainv, i
 }
 
 size_t bound_states_scratch(int m, int nb) {
-  // d, e^2 + per state (u0, u1, u2, mu, x) + per state int pivots
-  return sizeof(cplx) * ((size_t)2 * m + (size_t)nb * 5 * m) + sizeof(int) * (size_t)nb * m;
+  // per state the workspace that does not fit in shared memory; at least the 2 m entries of the
+  // QR fallback
+  const size_t fac = (states_bytes(m) + sizeof(cplx) - 1) / sizeof(cplx) * sizeof(cplx) * nb;
+  return std::max(fac, sizeof(cplx) * 2 * (size_t)m);
 }
 
-cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const cplx* diag, const cplx* v,
-                                const cplx* w, int nb, cplx* lam, cplx* phi, cplx* scratch, int* status,
+cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const cplx* v, const cplx* w, int nb,
+                                cplx* lam, cplx* phi, cplx* scratch, int* status,
                                 cudaStream_t st, const cplx* eig) {
-  k_bound_states<<<1, 32, 0, st>>>(m, west, east, diag, v, w, nb, lam, phi, scratch, status, eig);
+  const int in_smem = states_bytes(m) <= BS_SMEM;
+  const size_t smem = in_smem ? states_bytes(m) : 0;
+  // one constant limit, so that setups on several host threads may repeat the call
+  cudaError_t e = cudaFuncSetAttribute(k_bound_states, cudaFuncAttributeMaxDynamicSharedMemorySize, BS_SMEM);
+  if (e != cudaSuccess) return e;
+  k_bound_states<<<nb, BS_THREADS, smem, st>>>(m, west, east, v, w, lam, phi, scratch, in_smem, status, eig);
+  k_states_distinct<<<1, MGC_MAX_NB * MGC_MAX_NB, 0, st>>>(nb, lam, status);
   return cudaGetLastError();
 }
 

@@ -349,9 +349,13 @@ int axis_states(mgcccs_handle* h, int m, const cplx* west, const cplx* east, con
   bool ok = false;
   MGC_CUDA(eig_aberth(m, west, east, diag, v, w, h->eig_ab, h->eig_vals, &ok, h->st));
   h->launches += 4;
-  if (!ok) h->eig_fallbacks += 1;
-  MGC_LAUNCH(launch_bound_states(m, west, east, diag, v, w, h->nb, lam, phi, h->eig_scratch, h->status, h->st,
-                                 ok ? h->eig_vals : nullptr));
+  if (!ok) {
+    h->eig_fallbacks += 1;
+    MGC_LAUNCH(launch_qr_spectrum(m, west, east, diag, v, h->eig_scratch, h->eig_vals, h->status, h->st));
+  }
+  MGC_LAUNCH(launch_bound_states(m, west, east, v, w, h->nb, lam, phi, h->eig_scratch, h->status, h->st,
+                                 h->eig_vals));
+  h->launches += 1;   // two kernels
   return MGCCCS_OK;
 }
 
