@@ -608,9 +608,14 @@ cudaError_t launch_weight_states(int m, int nb, const cplx* w, const cplx* phi, 
 cudaError_t launch_channel_potentials(int mx, int my, int nb, const cplx* wphi, const cplx* phi,
                                       const cplx* wvphi, const cplx* vphi, const cplx* v12,
                                       cplx* VA, cplx* VB, cudaStream_t st);
-cudaError_t launch_channel_factor_pcr(const CRSystem& S, const cplx* diag, const cplx* v, double E, const cplx* lam,
-                                      const cplx* Vc, const cplx* a, const cplx* c, cplx* scratch, int* status,
-                                      cudaStream_t st);
+// One channel's axis couplings (diag, sub, sup), axis potential v, the other axis's eigenvalues
+// lam and the channel potential Vc: the unreduced system of Eq. (28) or (29).
+struct ChannelCoef {
+  const cplx *diag, *v, *lam, *Vc, *sub, *sup;
+};
+// scratch: channel_factor_pcr_scratch of each system, one after the other
+cudaError_t launch_channel_factor_pcr(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
+                                      double E, cplx* scratch, int* status, cudaStream_t st);
 size_t channel_factor_pcr_scratch(int m, int nb);
 // kernels_adjoint.cu
 int wdot_blocks(long long n);

@@ -571,146 +571,160 @@ __global__ void __launch_bounds__(256) k_channel_potentials(int rows, int len, i
   }
 }
 
-// In-place inverse of an n x n matrix (n <= MGC_MAX_NB) by Gauss-Jordan with partial pivoting.
-__device__ bool small_inverse(int n, cplx* A /* n*n row-major, replaced by inverse */) {
-  cplx aug[MGC_MAX_NB][2 * MGC_MAX_NB];
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < 2 * n; ++c) aug[r][c] = (c < n) ? A[r * n + c] : cmk(c - n == r ? 1.0 : 0.0, 0.0);
-  for (int k = 0; k < n; ++k) {
-    int piv = k;
-    double best = cabs2(aug[k][k]);
-    for (int r = k + 1; r < n; ++r)
-      if (cabs2(aug[r][k]) > best) { best = cabs2(aug[r][k]); piv = r; }
-    if (best == 0.0) return false;
-    if (piv != k)
-      for (int c = 0; c < 2 * n; ++c) { cplx t = aug[k][c]; aug[k][c] = aug[piv][c]; aug[piv][c] = t; }
-    cplx inv = cdiv(cmk(1.0, 0.0), aug[k][k]);
-    for (int c = 0; c < 2 * n; ++c) aug[k][c] = cmul(aug[k][c], inv);
-    for (int r = 0; r < n; ++r) {
-      if (r == k) continue;
-      cplx fct = aug[r][k];
-      for (int c = 0; c < 2 * n; ++c) aug[r][c] = cfms(fct, aug[k][c], aug[r][c]);
-    }
-  }
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < n; ++c) A[r * n + c] = aug[r][n + c];
-  return true;
-}
-
-// C = A B for n x n row-major blocks.
-__device__ void small_matmul(int n, const cplx* A, const cplx* B, cplx* C) {
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < n; ++c) {
-      cplx acc = cmk(0.0, 0.0);
-      for (int k = 0; k < n; ++k) acc = cfma(A[r * n + k], B[k * n + c], acc);
-      C[r * n + c] = acc;
-    }
-}
-
-// Cyclic-reduction factors of the coupled-channel system along one axis (one block):
-// B_k = (diag_k + v_k - E) I + diag(lam) + Vc_k, A_k = a_k I, C_k = c_k I, rows padded
-// with identity to M = 2^q - 1.  `scratch` holds the current A, B, C of rows 0..M.
-// Parallel cyclic reduction factors of one coupled-channel system (Eqs. (28)-(29)):
+// Parallel cyclic reduction factors of the two coupled-channel systems (Eqs. (28)-(29)):
 // rows k = 0..m-1 of A_k x_{k-1} + B_k x_k + C_k x_{k+1} = r_k with n_b x n_b blocks
 // (A_k, C_k the 1D Laplacian couplings times the identity, B_k the channel block).
 // Level l (stride s = 2^l) eliminates every row's couplings to k +- s with the rows
 // k +- s themselves: alpha = A_k B_{k-s}^{-1}, gamma = C_k B_{k+s}^{-1},
 //   A_k <- -alpha A_{k-s},  B_k <- B_k - alpha C_{k-s} - gamma A_{k+s},  C_k <- -gamma C_{k+s};
-// after ceil(log2 m) levels no coupling is left and x_k = B_k^{-1} r_k.  One block, the
-// rows of a level in parallel, double-buffered blocks.
-__global__ void __launch_bounds__(256) k_channel_factor_pcr(CRSystem S, const cplx* __restrict__ diag,
-                                                            const cplx* __restrict__ v, double E,
-                                                            const cplx* __restrict__ lam, const cplx* __restrict__ Vc,
-                                                            const cplx* __restrict__ sub, const cplx* __restrict__ sup,
-                                                            cplx* __restrict__ scratch, int* status) {
-  const int nb = S.nb, nb2 = nb * nb, m = S.m;
-  const size_t blk = (size_t)m * nb2;
-  cplx* Ab[2] = {scratch, scratch + 3 * blk};
-  cplx* Bb[2] = {scratch + blk, scratch + 4 * blk};
-  cplx* Cb[2] = {scratch + 2 * blk, scratch + 5 * blk};
-  cplx* Binv = scratch + 6 * blk;
-  const int t0 = threadIdx.x, nt = blockDim.x;
-  for (int k = t0; k < m; k += nt) {
-    cplx* A = Ab[0] + (size_t)k * nb2;
-    cplx* B = Bb[0] + (size_t)k * nb2;
-    cplx* C = Cb[0] + (size_t)k * nb2;
-    cplx base = cadd(diag[k], v[k]);
-    base.x -= E;
-    for (int r = 0; r < nb; ++r)
-      for (int c = 0; c < nb; ++c) {
-        cplx val = Vc[((size_t)k * nb + r) * nb + c];
-        if (r == c) val = cadd(val, cadd(base, lam[r]));
-        B[r * nb + c] = val;
-        A[r * nb + c] = (r == c && k > 0) ? sub[k] : cmk(0.0, 0.0);
-        C[r * nb + c] = (r == c && k < m - 1) ? sup[k] : cmk(0.0, 0.0);
-      }
+// after ceil(log2 m) levels no coupling is left and x_k = B_k^{-1} r_k.  One launch per level
+// for both systems, one warp per row with the row's blocks in shared memory; a launch ends
+// with the inverses of the blocks it made, so the next one finds its neighbours'.  The state of
+// a system is A, B, C and B^{-1} of every row, double-buffered: 8 m n_b^2 entries.
+// Bound by the latency of the inverse's pivot chain.  Two systems of 1023 rows, n_b = 3: 6.6 ms
+// as one block per system, 0.34 ms so.
+constexpr int CF_WARPS = 4;
+
+// The systems of both channels and what their first level is made from.
+struct ChannelSetup {
+  CRSystem S;
+  const cplx *diag, *v, *lam, *Vc, *sub, *sup;
+  cplx* scratch;                 // 8 m nb^2
+};
+
+// In-place inverse of the nb x nb matrix M of this warp by Gauss-Jordan elimination with
+// partial pivoting on [M | I] in aug (row pitch 2 nb); false on a zero pivot.
+__device__ bool warp_inverse(int nb, const cplx* M, cplx* aug, cplx* out) {
+  const int lane = threadIdx.x & 31, w2 = 2 * nb;
+  for (int e = lane; e < nb * w2; e += 32) {
+    const int r = e / w2, c = e - r * w2;
+    aug[e] = c < nb ? M[r * nb + c] : cmk(c - nb == r ? 1.0 : 0.0, 0.0);
   }
-  __syncthreads();
-  cplx T1[MGC_MAX_NB * MGC_MAX_NB], T2[MGC_MAX_NB * MGC_MAX_NB], al[MGC_MAX_NB * MGC_MAX_NB],
-      ga[MGC_MAX_NB * MGC_MAX_NB];
-  int cur = 0;
-  for (int l = 0; l < S.pq; ++l) {
-    const int s = 1 << l;
-    const cplx* A = Ab[cur];
-    const cplx* B = Bb[cur];
-    const cplx* C = Cb[cur];
-    for (int k = t0; k < m; k += nt) {
-      for (int r = 0; r < nb2; ++r) T1[r] = B[(size_t)k * nb2 + r];
-      if (!small_inverse(nb, T1)) {
-        atomicOr(status, MGC_ST_PIVOT);
-        for (int r = 0; r < nb2; ++r) T1[r] = cmk(0.0, 0.0);
-      }
-      for (int r = 0; r < nb2; ++r) Binv[(size_t)k * nb2 + r] = T1[r];
+  __syncwarp();
+  for (int k = 0; k < nb; ++k) {
+    int piv = k;
+    double best = cabs2(aug[k * w2 + k]);
+    for (int r = k + 1; r < nb; ++r) {
+      const double a = cabs2(aug[r * w2 + k]);
+      if (a > best) { best = a; piv = r; }
     }
-    __syncthreads();
-    cplx* A2 = Ab[cur ^ 1];
-    cplx* B2 = Bb[cur ^ 1];
-    cplx* C2 = Cb[cur ^ 1];
-    for (int k = t0; k < m; k += nt) {
-      const bool lo = k - s >= 0, hi = k + s < m;
-      if (lo) small_matmul(nb, A + (size_t)k * nb2, Binv + (size_t)(k - s) * nb2, al);
-      else for (int r = 0; r < nb2; ++r) al[r] = cmk(0.0, 0.0);
-      if (hi) small_matmul(nb, C + (size_t)k * nb2, Binv + (size_t)(k + s) * nb2, ga);
-      else for (int r = 0; r < nb2; ++r) ga[r] = cmk(0.0, 0.0);
-      cplx* pa = S.pa + ((size_t)l * m + k) * nb2;
-      cplx* pg = S.pg + ((size_t)l * m + k) * nb2;
-      for (int r = 0; r < nb2; ++r) {
-        pa[r] = al[r];
-        pg[r] = ga[r];
-        B2[(size_t)k * nb2 + r] = B[(size_t)k * nb2 + r];
-        A2[(size_t)k * nb2 + r] = cmk(0.0, 0.0);
-        C2[(size_t)k * nb2 + r] = cmk(0.0, 0.0);
-      }
-      if (lo) {
-        small_matmul(nb, al, C + (size_t)(k - s) * nb2, T1);
-        small_matmul(nb, al, A + (size_t)(k - s) * nb2, T2);
-        for (int r = 0; r < nb2; ++r) {
-          B2[(size_t)k * nb2 + r] = csub(B2[(size_t)k * nb2 + r], T1[r]);
-          A2[(size_t)k * nb2 + r] = cneg(T2[r]);
-        }
-      }
-      if (hi) {
-        small_matmul(nb, ga, A + (size_t)(k + s) * nb2, T1);
-        small_matmul(nb, ga, C + (size_t)(k + s) * nb2, T2);
-        for (int r = 0; r < nb2; ++r) {
-          B2[(size_t)k * nb2 + r] = csub(B2[(size_t)k * nb2 + r], T1[r]);
-          C2[(size_t)k * nb2 + r] = cneg(T2[r]);
-        }
-      }
+    if (best == 0.0) return false;                       // the same for every lane
+    __syncwarp();
+    if (piv != k && lane < w2) {
+      const cplx t = aug[k * w2 + lane];
+      aug[k * w2 + lane] = aug[piv * w2 + lane];
+      aug[piv * w2 + lane] = t;
     }
-    __syncthreads();
-    cur ^= 1;
+    __syncwarp();
+    const cplx inv = cdiv(cmk(1.0, 0.0), aug[k * w2 + k]);
+    __syncwarp();
+    if (lane < w2) aug[k * w2 + lane] = cmul(aug[k * w2 + lane], inv);
+    // the multipliers of this lane's entries, read before column k is cleared
+    cplx f[(2 * MGC_MAX_NB * MGC_MAX_NB + 31) / 32];
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < (2 * MGC_MAX_NB * MGC_MAX_NB + 31) / 32; ++q) {
+      const int e = lane + 32 * q;
+      if (e < nb * w2) f[q] = aug[e / w2 * w2 + k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < (2 * MGC_MAX_NB * MGC_MAX_NB + 31) / 32; ++q) {
+      const int e = lane + 32 * q;
+      if (e < nb * w2 && e / w2 != k) aug[e] = cfms(f[q], aug[k * w2 + e % w2], aug[e]);
+    }
+    __syncwarp();
   }
-  for (int k = t0; k < m; k += nt) {
-    for (int r = 0; r < nb2; ++r) T1[r] = Bb[cur][(size_t)k * nb2 + r];
-    if (!small_inverse(nb, T1)) {
-      atomicOr(status, MGC_ST_PIVOT);
-      for (int r = 0; r < nb2; ++r) T1[r] = cmk(0.0, 0.0);
-    }
-    for (int r = 0; r < nb2; ++r) S.pbinv[(size_t)k * nb2 + r] = T1[r];
-  }
+  for (int e = lane; e < nb * nb; e += 32) out[e] = aug[e / nb * w2 + nb + e % nb];
+  return true;
 }
 
+// Entry (r, c) of X Y for nb x nb row-major blocks.
+__device__ __forceinline__ cplx block_dot(int nb, const cplx* X, const cplx* Y, int r, int c) {
+  cplx acc = cmk(0.0, 0.0);
+  for (int k = 0; k < nb; ++k) acc = cfma(X[r * nb + k], Y[k * nb + c], acc);
+  return acc;
+}
+
+// Level l >= 0 of the reduction, or with l = -1 its start: the blocks of the unreduced rows.
+__global__ void __launch_bounds__(32 * CF_WARPS) k_channel_factor(ChannelSetup ca, ChannelSetup cb, double E, int l,
+                                                                  int* status) {
+  extern __shared__ cplx cf_sh[];
+  const ChannelSetup& P = blockIdx.y == 0 ? ca : cb;
+  const CRSystem& S = P.S;
+  const int nb = S.nb, nb2 = nb * nb, m = S.m;
+  const int lane = threadIdx.x & 31, k = blockIdx.x * CF_WARPS + (threadIdx.x >> 5);
+  if (k >= m || l >= S.pq) return;                         // whole warps leave; no block barrier below
+  cplx* sh = cf_sh + (size_t)(threadIdx.x >> 5) * 12 * nb2;   // ten blocks, then [B | I]
+  const size_t blk = (size_t)m * nb2, row = (size_t)k * nb2;
+  const int cur = (l + 2) & 1;                             // level l reads buffer cur, the start writes buffer 0
+  const cplx* in = P.scratch + cur * 4 * blk;
+  cplx* out = P.scratch + (l < 0 ? 0 : (cur ^ 1) * 4 * blk);
+  cplx* Bn = sh + 9 * nb2;
+  if (l < 0) {
+    cplx base = cadd(P.diag[k], P.v[k]);
+    base.x -= E;
+    for (int e = lane; e < nb2; e += 32) {
+      const int r = e / nb, c = e - r * nb;
+      cplx val = P.Vc[row + e];
+      if (r == c) val = cadd(val, cadd(base, P.lam[r]));
+      Bn[e] = val;
+      out[row + e] = (r == c && k > 0) ? P.sub[k] : cmk(0.0, 0.0);
+      out[blk + row + e] = val;
+      out[2 * blk + row + e] = (r == c && k < m - 1) ? P.sup[k] : cmk(0.0, 0.0);
+    }
+  } else {
+    const int s = 1 << l;
+    const bool lo = k - s >= 0, hi = k + s < m;
+    const size_t rl = row - (lo ? (size_t)s * nb2 : 0), rh = row + (hi ? (size_t)s * nb2 : 0);
+    // own A, C; the neighbours' B^{-1}, A, C (the row itself where a neighbour is missing)
+    cplx *A = sh, *C = sh + nb2, *Il = sh + 2 * nb2, *Al = sh + 3 * nb2, *Cl = sh + 4 * nb2, *Ih = sh + 5 * nb2,
+         *Ah = sh + 6 * nb2, *Ch = sh + 7 * nb2, *al = sh + 8 * nb2, *ga = sh + 10 * nb2;   // ga: in [B | I] until then
+    for (int e = lane; e < nb2; e += 32) {
+      A[e] = in[row + e];
+      C[e] = in[2 * blk + row + e];
+      Il[e] = in[3 * blk + rl + e];
+      Al[e] = in[rl + e];
+      Cl[e] = in[2 * blk + rl + e];
+      Ih[e] = in[3 * blk + rh + e];
+      Ah[e] = in[rh + e];
+      Ch[e] = in[2 * blk + rh + e];
+    }
+    __syncwarp();
+    cplx* pa = S.pa + ((size_t)l * m + k) * nb2;
+    cplx* pg = S.pg + ((size_t)l * m + k) * nb2;
+    for (int e = lane; e < nb2; e += 32) {
+      const int r = e / nb, c = e - r * nb;
+      al[e] = lo ? block_dot(nb, A, Il, r, c) : cmk(0.0, 0.0);
+      ga[e] = hi ? block_dot(nb, C, Ih, r, c) : cmk(0.0, 0.0);
+      pa[e] = al[e];
+      pg[e] = ga[e];
+    }
+    __syncwarp();
+    for (int e = lane; e < nb2; e += 32) {
+      const int r = e / nb, c = e - r * nb;
+      cplx b = in[blk + row + e], a2 = cmk(0.0, 0.0), c2 = a2;
+      if (lo) {
+        b = csub(b, block_dot(nb, al, Cl, r, c));
+        a2 = cneg(block_dot(nb, al, Al, r, c));
+      }
+      if (hi) {
+        b = csub(b, block_dot(nb, ga, Ah, r, c));
+        c2 = cneg(block_dot(nb, ga, Ch, r, c));
+      }
+      Bn[e] = b;
+      out[row + e] = a2;
+      out[blk + row + e] = b;
+      out[2 * blk + row + e] = c2;
+    }
+  }
+  __syncwarp();
+  cplx* dst = l == S.pq - 1 ? S.pbinv + row : out + 3 * blk + row;
+  if (!warp_inverse(nb, Bn, sh + 10 * nb2, dst)) {
+    if (lane == 0) atomicOr(status, MGC_ST_PIVOT);
+    for (int e = lane; e < nb2; e += 32) dst[e] = cmk(0.0, 0.0);
+  }
+}
 
 }  // namespace
 
@@ -811,12 +825,16 @@ int pcr_levels(int m) {
   return q;
 }
 
-size_t channel_factor_pcr_scratch(int m, int nb) { return (size_t)7 * m * nb * nb; }
+size_t channel_factor_pcr_scratch(int m, int nb) { return (size_t)8 * m * nb * nb; }
 
-cudaError_t launch_channel_factor_pcr(const CRSystem& S, const cplx* diag, const cplx* v, double E, const cplx* lam,
-                                      const cplx* Vc, const cplx* a, const cplx* c, cplx* scratch, int* status,
-                                      cudaStream_t st) {
-  k_channel_factor_pcr<<<1, 256, 0, st>>>(S, diag, v, E, lam, Vc, a, c, scratch, status);
+cudaError_t launch_channel_factor_pcr(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
+                                      double E, cplx* scratch, int* status, cudaStream_t st) {
+  const int nb = A.nb, mm = std::max(A.m, B.m), pq = std::max(A.pq, B.pq);
+  cplx* scrB = scratch + channel_factor_pcr_scratch(A.m, nb);
+  const ChannelSetup a{A, ca.diag, ca.v, ca.lam, ca.Vc, ca.sub, ca.sup, scratch};
+  const ChannelSetup b{B, cb.diag, cb.v, cb.lam, cb.Vc, cb.sub, cb.sup, scrB};
+  const dim3 grid((mm + CF_WARPS - 1) / CF_WARPS, 2);
+  const size_t smem = (size_t)CF_WARPS * 12 * nb * nb * sizeof(cplx);
+  for (int l = -1; l < pq; ++l) k_channel_factor<<<grid, 32 * CF_WARPS, smem, st>>>(a, b, E, l, status);
   return cudaGetLastError();
 }
-

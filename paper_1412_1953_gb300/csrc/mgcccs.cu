@@ -207,10 +207,8 @@ void layout(mgcccs_handle* h, Carver& cv) {
       S.pg = cv.take<cplx>((size_t)S.pq * S.m * nb2);
       S.pbinv = cv.take<cplx>((size_t)S.m * nb2);
     }
-    {
-      const int mmax = h->crA.m > h->crB.m ? h->crA.m : h->crB.m;
-      h->cr_scratch = cv.take<cplx>(channel_factor_pcr_scratch(mmax, nb));
-    }
+    h->cr_scratch =
+        cv.take<cplx>(channel_factor_pcr_scratch(h->crA.m, nb) + channel_factor_pcr_scratch(h->crB.m, nb));
     size_t es = bound_states_scratch(mx > my ? mx : my, nb);
     h->eig_scratch = cv.take<cplx>((es + sizeof(cplx) - 1) / sizeof(cplx));
     CCView& cc = h->cc;
@@ -440,10 +438,10 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
     MGC_LAUNCH(launch_channel_potentials(b.mx, b.my, nb, h->wphi, h->phi, h->wvphi, h->vphi, v12, h->VA, h->VB,
                                          st));
     // channel A runs along y with the x bound states; channel B along x with the y ones
-    MGC_LAUNCH(launch_channel_factor_pcr(h->crA, b.diag_y, v2, p.E, h->lam, h->VA, b.west_y, b.east_y,
-                                         h->cr_scratch, h->status, st));
-    MGC_LAUNCH(launch_channel_factor_pcr(h->crB, b.diag_x, v1, p.E, h->mu, h->VB, b.west_x, b.east_x,
-                                         h->cr_scratch, h->status, st));
+    const ChannelCoef ca{b.diag_y, v2, h->lam, h->VA, b.west_y, b.east_y};
+    const ChannelCoef cb{b.diag_x, v1, h->mu, h->VB, b.west_x, b.east_x};
+    MGC_LAUNCH(launch_channel_factor_pcr(h->crA, h->crB, ca, cb, p.E, h->cr_scratch, h->status, st));
+    h->launches += std::max(h->crA.pq, h->crB.pq);   // one kernel per level after the first
   }
   int rc0 = read_status(h);
   if (rc0 || !h->mixed) return rc0;
