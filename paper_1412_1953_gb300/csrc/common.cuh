@@ -590,6 +590,11 @@ bool bpcr_fits(int mx, int my);
 size_t bpcr_factor_entries(int mx, int my);                  // complex entries of the factors
 size_t bpcr_scratch_entries(int mx, int my);                 // complex entries of setup scratch
 cudaError_t launch_bpcr_setup(const StencilView& s, cplx* fac, cplx* scratch, int* status, cudaStream_t st);
+// the dense inverse of a coarsest operator of at most MGC_MAX_COARSE nodes by the same reduction;
+// *worst (cleared by the caller) receives the bits of max |A A^{-1} - I|
+size_t block_inverse_scratch(int mx, int my);
+cudaError_t launch_block_inverse(const StencilView& s, cplx* scratch, cplx* Ainv, int* status,
+                                 unsigned long long* worst, cudaStream_t st);
 // u = A_c^{-1} f through the factors; buf holds 2 mx my complex entries
 template <class C>
 cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const C* f, C* u, cplx* buf, cudaStream_t st);

@@ -176,7 +176,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
     h->bp_buf = cv.take<cplx>((size_t)2 * h->nc);
   } else {
     h->Ainv = cv.take<cplx>((size_t)h->nc * h->nc);
-    h->aug = cv.take<cplx>(coarse_inverse_scratch(h->nc));
+    h->aug = cv.take<cplx>(std::max(coarse_inverse_scratch(h->nc), block_inverse_scratch(c.mx, c.my)));
     h->bp_fac = h->bp_scr = h->bp_buf = nullptr;
   }
   {
@@ -281,7 +281,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
   }
   h->norm_part = cv.take<double>(h->norm_nparts);
   h->norm_out = cv.take<double>(4);
-  h->status = cv.take<int>(4);
+  h->status = cv.take<int>(8);   // error bits, three flags, then the dense inverse's check (below)
   h->hu = cv.take<cplx>((size_t)mx * my);
   h->hf = cv.take<cplx>((size_t)mx * my);
   h->wdot_part = cv.take<cplx>(wdot_blocks((long long)mx * my));
@@ -339,6 +339,24 @@ int read_status(mgcccs_handle* h) {
   return MGCCCS_OK;
 }
 
+// The block-wise dense inverse exchanges rows within a block only: where it met a zero pivot or
+// its residual max |A A^{-1} - I| exceeds what a well-conditioned coarsest operator leaves
+// (below 1e-12 on every grid of the tests), Gauss-Jordan elimination with partial pivoting over
+// all rows takes its place.
+constexpr double MGC_INVERSE_RESIDUAL = 1e-11;
+int coarse_inverse_check(mgcccs_handle* h) {
+  if (h->coarse_bp) return MGCCCS_OK;
+  struct {
+    int pivot, pad;
+    double worst;
+  } c;
+  MGC_CUDA(cudaMemcpyAsync(&c, h->status + 4, sizeof(c), cudaMemcpyDeviceToHost, h->st));
+  MGC_CUDA(cudaStreamSynchronize(h->st));
+  if (c.pivot == 0 && c.worst <= MGC_INVERSE_RESIDUAL) return MGCCCS_OK;
+  MGC_LAUNCH(launch_coarse_inverse(h->lv[h->L - 1].sv, h->aug, h->Ainv, h->status, h->st));
+  return MGCCCS_OK;
+}
+
 // Bound states of one axis (Eq. (9)): all eigenvalues by the Ehrlich-Aberth iteration
 // (parallel; the one-thread FP64 QR when it does not converge), then selection and
 // refinement in k_bound_states.
@@ -361,7 +379,7 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
              const cplx* phi_in = nullptr, const cplx* mu_in = nullptr, const cplx* vphi_in = nullptr) {
   const mgcccs_params& p = h->p;
   cudaStream_t st = h->st;
-  MGC_CUDA(cudaMemsetAsync(h->status, 0, 4 * sizeof(int), st));
+  MGC_CUDA(cudaMemsetAsync(h->status, 0, 8 * sizeof(int), st));
   MGC_CUDA(cudaMemcpyAsync(h->v1c, v1, sizeof(cplx) * h->lv[0].mx, cudaMemcpyDeviceToDevice, st));
   MGC_CUDA(cudaMemcpyAsync(h->v2c, v2, sizeof(cplx) * h->lv[0].my, cudaMemcpyDeviceToDevice, st));
   h->eig_fallbacks = 0;
@@ -400,7 +418,9 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
   if (h->coarse_bp) {
     MGC_LAUNCH(launch_bpcr_setup(h->lv[h->L - 1].sv, h->bp_fac, h->bp_scr, h->status, st));
   } else {
-    MGC_LAUNCH(launch_coarse_inverse(h->lv[h->L - 1].sv, h->aug, h->Ainv, h->status, st));
+    // its zero pivots go to status[4], its largest residual to status[6..7] (read at the end)
+    MGC_LAUNCH(launch_block_inverse(h->lv[h->L - 1].sv, h->aug, h->Ainv, h->status + 4,
+                                    reinterpret_cast<unsigned long long*>(h->status + 6), st));
   }
   if (h->nb > 0) {
     const LevelBufs& b = h->lv[0];
@@ -443,7 +463,9 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
     MGC_LAUNCH(launch_channel_factor_pcr(h->crA, h->crB, ca, cb, p.E, h->cr_scratch, h->status, st));
     h->launches += std::max(h->crA.pq, h->crB.pq);   // one kernel per level after the first
   }
-  int rc0 = read_status(h);
+  int rc0 = coarse_inverse_check(h);
+  if (rc0) return rc0;
+  rc0 = read_status(h);
   if (rc0 || !h->mixed) return rc0;
   // complex64 copies of every level's operator and of the bound states
   for (int l = 0; l < h->L; ++l) {
