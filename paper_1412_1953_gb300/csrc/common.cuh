@@ -527,45 +527,61 @@ struct CCViewT {
   C* Py_part;              // [nty][nb][mx]
   cplx* Px;                // [nb][my]
   cplx* Py;                // [nb][mx]
-  cplx* c;                 // [nb][nb]  c[a][b] = int int phi_a vphi_b r
   cplx* eA;                // [nb][my]
   cplx* eB;                // [nb][mx]
   const C* eAc;            // eA, eB in the element precision (the same arrays for complex128)
   const C* eBc;
-  const cplx* wvphi64;     // [nb][my] FP64 weighted states for the coupling coefficients
 };
 typedef CCViewT<cplx> CCView;
 typedef CCViewT<float2> CCView32;
 
-// One coupled-channel system (Eqs. (28)-(29)) with its parallel-cyclic-reduction factors.
+// One coupled-channel system (Eqs. (28)-(29)) with its cyclic-reduction factors.
 struct CRSystem {
   int m, nb;
-  // right-hand side r[a][k] = P[a][k] - sum_l coef(a, l) basis[l][k] with the conventions of
-  // Eqs. (25)-(26): channel A (chan 0) l > a, coef = c[a][l], basis = vphi (along y);
-  // channel B (chan 1) l >= a, coef = c[l][a], basis = phi (along x)
+  // right-hand side r[a][k] = P[a][k] - sum_l d(a, l) basis[l][k], d(a, l) = sum_k wst[l][k] P[a][k],
+  // with the conventions of Eqs. (25)-(26): channel A (chan 0) l > a, d = c_al of Eq. (27),
+  // basis = vphi (along y); channel B (chan 1) l >= a, d = c_la, basis = phi (along x)
   int chan;
   const cplx* P;           // [nb][m] projections P^x (channel A) or P^y (channel B)
-  const cplx* cmat;        // [nb][nb] c
+  const cplx* wst;         // [nb][m] weighted states along the system's axis
   const cplx* basis;       // [nb][m]
   cplx* e;                 // [nb][m] solution
   float2* e32;             // [nb][m] solution rounded to complex64 (mixed precision), or null
-  // parallel cyclic reduction: pq = ceil(log2 m) levels; level l with stride s = 2^l
-  // updates every row k by x_k -= pa_k x_{k-s} + pg_k x_{k+s}; then x_k = pbinv_k x_k.
-  // Rows are 0..m-1; terms outside them are absent.
-  int pq;
-  cplx* pa;                // [pq][m][nb*nb]
-  cplx* pg;                // [pq][m][nb*nb]
-  cplx* pbinv;             // [m][nb*nb]
+  // R = 2^p rows per CTA, k = rank R + i; ns = floor(m / R) separators (rows with i = R - 1).
+  // pack, per CTA (cr_pack_entries): for each level l < p and each row kept at it (i + 1 = 2s j,
+  // s = 2^l) alpha, gamma; the gamma of the previous CTA's separator at each level; and for each
+  // row eliminated (i < R - 1) B^{-1} A, B^{-1} C, B^{-1} of its level.  sinv: the dense inverse of
+  // the separators' system, [ns nb][ns nb].
+  int p, ns;
+  cplx* pack;
+  cplx* sinv;
+  // setup only: the factors of the parallel reduction of the separators, [levels][ns][2 nb^2], then
+  // their last B^{-1}, [ns][nb^2]
+  cplx* sfac;
 };
-int pcr_levels(int m);
+constexpr int CR_CLUSTER = 16;       // CTAs per system (a non-portable cluster size)
+// log2 of the rows per CTA: the least power of two that 16 CTAs cover m rows with
+__host__ __device__ constexpr int cr_log_rows(int m) {
+  int p = 0;
+  while ((CR_CLUSTER << p) < m) ++p;
+  return p;
+}
+__host__ __device__ constexpr size_t cr_pack_entries(int R, int p, int nb) {
+  return (size_t)nb * nb * (5 * (size_t)(R - 1) + p);
+}
+// Whether a CTA's factors fit in shared memory beside its rows.
+__host__ __device__ constexpr bool cr_pack_in_smem(int m, int nb) {
+  const int p = cr_log_rows(m);
+  return 16 * (cr_pack_entries(1 << p, p, nb) + ((size_t)nb << p)) <= 200 * 1024;
+}
 int cc_tiles_x(int mx);
 int cc_tiles_y(int my);
 template <class C>
 cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f,
                                     cudaStream_t st);
 template <class C>
-cudaError_t launch_cc_rhs(const CCViewT<C>& c, cudaStream_t st);
-cudaError_t channel_solve_prepare(int nb, int m_max);
+cudaError_t launch_reduce_projections(const CCViewT<C>& c, cudaStream_t st);
+cudaError_t channel_solve_prepare(int nb, int mA, int mB);
 cudaError_t launch_channel_solve(const CRSystem& A, const CRSystem& B, cudaStream_t st);
 template <class C>
 cudaError_t launch_cccs_correct(const CCViewT<C>& c, C* u, cudaStream_t st);
@@ -618,10 +634,12 @@ cudaError_t launch_channel_potentials(int mx, int my, int nb, const cplx* wphi, 
 struct ChannelCoef {
   const cplx *diag, *v, *lam, *Vc, *sub, *sup;
 };
-// scratch: channel_factor_pcr_scratch of each system, one after the other
-cudaError_t launch_channel_factor_pcr(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
+// scratch: channel_factor_scratch of each system, one after the other
+cudaError_t launch_channel_factor(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
                                       double E, cplx* scratch, int* status, cudaStream_t st);
-size_t channel_factor_pcr_scratch(int m, int nb);
+size_t channel_factor_scratch(int m, int nb);
+size_t channel_separator_entries(int ns, int nb);               // of CRSystem::sfac
+int channel_factor_launches(const CRSystem& A, const CRSystem& B);
 // kernels_adjoint.cu
 int wdot_blocks(long long n);
 cudaError_t launch_weighted_dot(int mx, int my, const cplx* wx, const cplx* wy, const cplx* a, const cplx* b,

@@ -10,7 +10,8 @@
 //
 // The projections are fused into the residual pass and reduced deterministically:
 // per 32 x 32 tile, sums along x and along y through a shared-memory tile give
-// per-tile partials, which a second kernel sums in a fixed order.
+// per-tile partials, which a second kernel sums in a fixed order; the channel solves form
+// the coefficients and right-hand sides from the sums as they start.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -116,38 +117,26 @@ __global__ void __launch_bounds__(256) k_reduce_partials(int nb, int mx, int my,
   }
 }
 
-// c[a][b] = sum_j w_y(j) vphi_b(j) P^x_a(j): one block per (a, b).
-__global__ void __launch_bounds__(256) k_cc_coef(int nb, int my, const cplx* __restrict__ wvphi,
-                                                 const cplx* __restrict__ Px, cplx* __restrict__ cmat) {
-  mgc_pdl_enter();
-  __shared__ double sh[2][8];
-  const int a = blockIdx.x / nb, b = blockIdx.x % nb;
-  cplx acc = cmk(0.0, 0.0);
-  for (int j = threadIdx.x; j < my; j += 256) acc = cfma(__ldg(wvphi + b * my + j), __ldg(Px + a * my + j), acc);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.x += __shfl_down_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
-  }
-  if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = acc.x; sh[1][threadIdx.x >> 5] = acc.y; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    cplx tot = cmk(0.0, 0.0);
-    for (int w = 0; w < 8; ++w) tot = cadd(tot, cmk(sh[0][w], sh[1][w]));
-    cmat[a * nb + b] = tot;
-  }
-}
-
-// Coupled-channel solves (Eqs. (28)-(29)) by parallel cyclic reduction with setup-time
-// factors: each system is solved by one thread-block cluster of CR_CLUSTER CTAs (cluster
-// 0: channel A along y, cluster 1: channel B along x); every level is one pass over the
-// (row, component) pairs split across the cluster.  Levels are separated by split
-// cluster barriers: every thread arrives (release) after its stores, loads the read-only
-// factor rows of its first item of the next level, and only then waits (acquire), so
-// the factor loads overlap the barrier.  Arrive and wait sit outside all data-dependent
-// branches, so each warp executes them convergently.  Sums are formed as independent
-// length-nb dot products, which keeps the dependent FP64 chain short.
-constexpr int CR_CLUSTER = 16;           // non-portable size: allowed per kernel at setup
+// Coupled-channel solves (Eqs. (28)-(29)) by cyclic reduction with setup-time factors: each
+// system is solved by one thread-block cluster of CR_CLUSTER CTAs (cluster 0: channel A along y,
+// cluster 1: channel B along x).  CTA `rank` owns the R = 2^p block rows [rank R, rank R + R) in
+// its shared memory.  Level l < p (stride s = 2^l) eliminates every other remaining row,
+// r_k -= alpha_k r_{k-s} + gamma_k r_{k+s} for the rows with k + 1 a multiple of 2s, until each
+// CTA is left with its last row, the separator.  Only a separator's gamma term reaches into the
+// next CTA, and nobody reads a separator meanwhile, so the next CTA sums those terms and the
+// levels need block barriers only.  The separators (at most 16) are solved by the dense inverse
+// of their system, every CTA gathering all their right-hand sides after one cluster barrier and
+// forming the two it borders on; the eliminated rows follow in reverse order, x_k = B_k^{-1} r_k
+// - alpha_k x_{k-s} - gamma_k x_{k+s}, again within the CTA.
+// What bounds it is the latency of ~2 p small steps: a warp-wide FP64 instruction occupies its
+// quarter of an SM for 64 cycles however few lanes need it, so LP lanes share the products of an
+// item (a row's component), and the factors are copied to shared memory while the preceding
+// kernel drains (large systems read them from L2).  Against parallel cyclic reduction over the
+// cluster (every row updated at each of log2 m levels, a cluster barrier between them) with the
+// coupling coefficients in a kernel of their own: 26.0 against 28.0 + 6.7 us for 1023 rows and
+// n_b = 3, 16.2 against 18.1 + 4.1 us for 127 rows (cold L2); for 2047 rows and n_b = 6, where
+// that took 11 m row updates, a step of the mixed-precision solve is 73 us shorter (50.3 to
+// 44.6 ms a solve of 78 steps).
 constexpr int CR_THREADS = 256;
 
 __device__ __forceinline__ void cluster_arrive() {
@@ -156,109 +145,215 @@ __device__ __forceinline__ void cluster_arrive() {
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
-
-template <int NB>
-__device__ __forceinline__ void load_row(cplx (&d)[NB], const cplx* __restrict__ src) {
-#pragma unroll
-  for (int p = 0; p < NB; ++p) d[p] = __ldg(src + p);
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
 
-template <int NB>
-__device__ __forceinline__ cplx dot_row(const cplx (&a)[NB], const cplx* x) {
-  cplx s = cmul(a[0], x[0]);
+// Sum over the LP lanes of an item, to all of them.
+template <int LP>
+__device__ __forceinline__ cplx item_sum(cplx v) {
 #pragma unroll
-  for (int p = 1; p < NB; ++p) s = cfma(a[p], x[p], s);
-  return s;
+  for (int o = 1; o < LP; o *= 2) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+  }
+  return v;
 }
 
-// Level l (stride s = 2^l) updates every row, x_k <- x_k - pa_k x_{k-s} - pg_k x_{k+s}
-// (X and Y alternate); after ceil(log2 m) levels x_k = pbinv_k x_k.  Against block cyclic
-// reduction (2 log2 m dependent levels on half the rows) this halves the dependent levels
-// for log2(m)/2 times the arithmetic, which 16-CTA clusters absorb: 37 us against 57 us
-// per CCCS at 1023 rows, n_b = 3.
-// Rows per CTA when one 16-CTA cluster holds the m block rows of a system.
-__host__ __device__ __forceinline__ int cr_rows(int m) { return (m + CR_CLUSTER - 1) / CR_CLUSTER; }
+// -(fa xl + fg xh) (+ fb r) of one component, its NB-term rows shared by LP lanes; a null x drops
+// its term.
+template <int NB, int LP, int NBLK>
+__device__ __forceinline__ cplx item_dot(const cplx* fa, const cplx* fg, const cplx* fb, const cplx* xl,
+                                         const cplx* xh, const cplx* r, int part) {
+  cplx acc = cmk(0.0, 0.0);
+#pragma unroll
+  for (int t = 0; t < (NBLK * NB + LP - 1) / LP; ++t) {
+    const int idx = t * LP + part, blk = idx / NB, q = idx - blk * NB;
+    if (NBLK == 3 && blk == 2) {
+      if (r) acc = cfma(fb[q], r[q], acc);
+    } else if (blk < 2) {
+      const cplx* f = blk == 0 ? fa : fg;
+      const cplx* x = blk == 0 ? xl : xh;
+      if (x) acc = cfms(f[q], x[q], acc);
+    }
+  }
+  return item_sum<LP>(acc);
+}
 
-// One system per 16-CTA cluster.  CTA `rank` owns block rows [rank R, rank R + R) and keeps
-// their current right-hand sides in its shared memory (two buffers, one per parity of the
-// level); a level reads rows k - s and k + s from the shared memory of the CTAs that own
-// them (distributed shared memory), and the split cluster barrier between levels orders
-// those reads against the next level's writes.  The factor rows of the next level are
-// fetched between the barrier's arrive and wait.
+// What a CTA works on: rows [k0, k0 + R) of m, the rows in X, the previous separator's share in
+// V, the separators' solutions xL (previous) and xO (own), null where there is none.
+struct ChannelRows {
+  int m, k0, R, p, rank;
+  cplx *X, *V;
+  const cplx *xL, *xO;
+};
+
+// Level l of the elimination.
+template <int NB, int LP>
+__device__ void channel_down(const ChannelRows& c, const cplx* F, int l) {
+  constexpr int nb2 = NB * NB, PASS = CR_THREADS / LP;
+  const int s = 1 << l, nk = c.R >> (l + 1), nit = (nk + (c.rank > 0 ? 1 : 0)) * NB, part = threadIdx.x % LP;
+  const cplx* fw = F + (size_t)(c.R - (c.R >> l)) * 2 * nb2;
+  const cplx* vf = F + (size_t)(c.R - 1) * 2 * nb2 + (size_t)l * nb2;
+  for (int p0 = 0; p0 < nit; p0 += PASS) {
+    const int it = p0 + threadIdx.x / LP, j = it / NB, comp = it - j * NB;
+    const int i = j < nk ? 2 * s * (j + 1) - 1 : -1;
+    const bool on = it < nit && c.k0 + i < c.m;
+    const cplx* f = j < nk ? fw + (size_t)j * 2 * nb2 + comp * NB : vf - nb2 + comp * NB;
+    const cplx* xl = on && j < nk ? c.X + (i - s) * NB : nullptr;
+    const cplx* xh = on && i + s < c.R && c.k0 + i + s < c.m ? c.X + (i + s) * NB : nullptr;
+    const cplx a = item_dot<NB, LP, 2>(f, f + nb2, nullptr, xl, xh, nullptr, part);
+    if (on && part == 0) {
+      cplx* t = j < nk ? c.X + i * NB + comp : c.V + comp;
+      *t = cadd(*t, a);
+    }
+  }
+}
+
+// The rows eliminated at level l, from their neighbours' solutions.  A pass takes whole rows and
+// writes after a barrier: an update in place reads all components of its row.
+template <int NB, int LP>
+__device__ void channel_up(const ChannelRows& c, const cplx* F, int l) {
+  constexpr int nb2 = NB * NB, PASS = CR_THREADS / LP / NB * NB;
+  const int s = 1 << l, nit = (c.R >> (l + 1)) * NB, part = threadIdx.x % LP, it0 = threadIdx.x / LP;
+  const cplx* bk = F + ((size_t)(c.R - 1) * 2 + c.p) * nb2;
+  for (int p0 = 0; p0 < nit; p0 += PASS) {
+    const int it = p0 + it0, j = it / NB, comp = it - j * NB, i = s - 1 + 2 * s * j;
+    const bool on = it0 < PASS && it < nit && c.k0 + i < c.m;
+    const cplx* f = bk + (size_t)(on ? i : 0) * 3 * nb2 + comp * NB;
+    const cplx* xl = !on ? nullptr : (j == 0 ? c.xL : c.X + (i - s) * NB);
+    const cplx* xh = !on ? nullptr : (i + s == c.R - 1 ? c.xO : (c.k0 + i + s < c.m ? c.X + (i + s) * NB : nullptr));
+    const cplx v = item_dot<NB, LP, 3>(f, f + nb2, f + 2 * nb2, xl, xh, on ? c.X + i * NB : nullptr, part);
+    __syncthreads();
+    if (on && part == 0) c.X[i * NB + comp] = v;
+  }
+}
+
 template <int NB>
 __global__ void __cluster_dims__(CR_CLUSTER, 1, 1) __launch_bounds__(CR_THREADS)
-k_channel_solve_pcr(CRSystem SA, CRSystem SB) {
-  mgc_pdl_enter();
-  extern __shared__ cplx cr_x[];   // [2][R * NB]
-  cg::cluster_group cl = cg::this_cluster();
-  const int sys = blockIdx.x / CR_CLUSTER;
-  const int rank = (int)cl.block_rank();
-  const CRSystem S = sys == 0 ? SA : SB;
+k_channel_solve(CRSystem SA, CRSystem SB) {
+  extern __shared__ cplx cr_sh[];        // X [R][NB], then the factors when they fit
   constexpr int nb2 = NB * NB;
-  const int m = S.m, pq = S.pq;
-  const int R = cr_rows(m), nloc = R * NB, k0 = rank * R;
-  cplx* X = cr_x;
-  cplx* Y = cr_x + nloc;
-  // the channel right-hand sides with the uniqueness conventions (Eqs. (25)-(26))
-  for (int e = threadIdx.x; e < nloc; e += CR_THREADS) {
-    const int k = k0 + e / NB, comp = e % NB;
-    cplx v = cmk(0.0, 0.0);
-    if (k < m) {
-      v = S.P[comp * m + k];
-      if (S.chan == 0) {
-        for (int l = comp + 1; l < NB; ++l) v = cfms(S.cmat[comp * NB + l], __ldg(S.basis + l * m + k), v);   // b_al
-      } else {
-        for (int l = comp; l < NB; ++l) v = cfms(S.cmat[l * NB + comp], __ldg(S.basis + l * m + k), v);       // a_bl
-      }
+  __shared__ cplx cpart[nb2], csum[nb2], V[NB], xs[2][NB], rs[CR_CLUSTER * NB];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+  const CRSystem S = blockIdx.x < CR_CLUSTER ? SA : SB;
+  const int m = S.m, p = S.p, R = 1 << p, ns = S.ns, k0 = rank * R;
+  cplx* const X = cr_sh;
+  const size_t len = cr_pack_entries(R, p, NB);
+  const cplx* F = S.pack + rank * len;
+  const bool in_smem = cr_pack_in_smem(m, NB);
+  if (k0 < m) {
+    // the factors were written at setup: fetch them ahead of the wait for the projections
+    if (in_smem) {
+      for (size_t e = tid; e < len; e += CR_THREADS) copy_async16(X + R * NB + e, F + e);
+    } else if (tid == 0) {
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(F), "r"((unsigned)(len * sizeof(cplx)))
+                   : "memory");
     }
-    X[e] = v;
+  }
+  mgc_pdl_enter();
+
+  // the projections of this CTA's rows, and their share of the coupling coefficients
+  // csum[a][l] = sum_k wst_l(k) P_a(k) that the conventions of Eqs. (25)-(26) use: c_al of Eq.
+  // (27), l > a, in channel A, c_la, l >= a, in channel B
+  for (int e = tid; e < R * NB; e += CR_THREADS) {
+    const int comp = e >> p, k = k0 + (e & (R - 1));
+    X[(k - k0) * NB + comp] = k < m ? S.P[comp * m + k] : cmk(0.0, 0.0);
+  }
+  if (tid < NB) V[tid] = cmk(0.0, 0.0);
+  __syncthreads();
+  {
+    constexpr int CL = NB <= 3 ? 16 : NB <= 5 ? 8 : 4;   // lanes a coefficient: one warp a quarter
+    const int l0 = S.chan == 0 ? 1 : 0, part = tid % CL;
+    for (int q0 = 0; q0 < nb2; q0 += CR_THREADS / CL) {
+      // coefficient q of the triangle, counted row by row
+      int q = q0 + tid / CL, a = 0;
+      while (a < NB && q >= NB - l0 - a) { q -= max(0, NB - l0 - a); ++a; }
+      const int l = a + l0 + q;
+      const bool on = a < NB && l < NB;
+      cplx acc = cmk(0.0, 0.0);
+      if (on)
+        for (int k = k0 + part; k < min(k0 + R, m); k += CL)
+          acc = cfma(__ldg(S.wst + l * m + k), X[(k - k0) * NB + a], acc);
+      acc = item_sum<CL>(acc);
+      if (on && part == 0) cpart[a * NB + l] = acc;
+    }
   }
   cluster_arrive();
-  const int e0 = threadIdx.x, kf = k0 + e0 / NB;
-  const bool first_ok = e0 < nloc && kf < m;
-  cplx fa[NB], fb[NB];
-  for (int l = 0; l < pq; ++l) {
-    const int s = 1 << l;
-    const cplx* pa = S.pa + (size_t)l * m * nb2;
-    const cplx* pg = S.pg + (size_t)l * m * nb2;
-    if (first_ok) {
-      const size_t fo = (size_t)kf * nb2 + (e0 % NB) * NB;
-      load_row<NB>(fa, pa + fo);
-      load_row<NB>(fb, pg + fo);
+  cluster_wait();
+  {
+    const int q = tid / 4;
+    cplx acc = cmk(0.0, 0.0);
+    if (q < nb2 && q % NB >= q / NB + (S.chan == 0 ? 1 : 0)) {
+#pragma unroll
+      for (int c = 0; c < CR_CLUSTER / 4; ++c)
+        acc = cadd(acc, *cl.map_shared_rank(cpart + q, (tid % 4) * (CR_CLUSTER / 4) + c));
     }
-    cluster_wait();
-    for (int e = e0; e < nloc; e += CR_THREADS) {
-      const int k = k0 + e / NB, comp = e % NB;
-      if (k >= m) break;
-      if (e != e0) {
-        const size_t fo = (size_t)k * nb2 + comp * NB;
-        load_row<NB>(fa, pa + fo);
-        load_row<NB>(fb, pg + fo);
-      }
-      cplx acc = X[e];
-      if (k - s >= 0) {
-        const int q = (k - s) / R;
-        acc = csub(acc, dot_row<NB>(fa, cl.map_shared_rank(X + (k - s - q * R) * NB, q)));
-      }
-      if (k + s < m) {
-        const int q = (k + s) / R;
-        acc = csub(acc, dot_row<NB>(fb, cl.map_shared_rank(X + (k + s - q * R) * NB, q)));
-      }
-      Y[e] = acc;
-    }
-    cluster_arrive();
-    cplx* t = X; X = Y; Y = t;
+    acc = item_sum<4>(acc);
+    if (q < nb2 && tid % 4 == 0) csum[q] = acc;
   }
-  if (first_ok) load_row<NB>(fa, S.pbinv + (size_t)kf * nb2 + (e0 % NB) * NB);
-  cluster_wait();   // every CTA is past its last remote read: each now reads only its own rows
-  for (int e = e0; e < nloc; e += CR_THREADS) {
-    const int k = k0 + e / NB, comp = e % NB;
-    if (k >= m) break;
-    if (e != e0) load_row<NB>(fa, S.pbinv + (size_t)k * nb2 + comp * NB);
-    const cplx v = dot_row<NB>(fa, X + (e / NB) * NB);
+  __syncthreads();
+  for (int e = tid; e < R * NB; e += CR_THREADS) {
+    const int comp = e >> p, k = k0 + (e & (R - 1));
+    if (k >= m) continue;
+    cplx v = X[(k - k0) * NB + comp];
+    for (int l = comp + (S.chan == 0 ? 1 : 0); l < NB; ++l)
+      v = cfms(csum[comp * NB + l], __ldg(S.basis + l * m + k), v);
+    X[(k - k0) * NB + comp] = v;
+  }
+  if (in_smem) {
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    F = X + R * NB;
+  }
+  __syncthreads();
+
+  const ChannelRows c{m, k0, R, p, rank, X, V, rank > 0 ? xs[0] : nullptr, rank < ns ? xs[1] : nullptr};
+  for (int l = 0; l < p; ++l) {
+    // four lanes an item while that still leaves one warp a quarter
+    if (((R >> (l + 1)) + 1) * NB <= 32) channel_down<NB, 4>(c, F, l);
+    else channel_down<NB, 2>(c, F, l);
+    __syncthreads();
+  }
+  cluster_arrive();
+  cluster_wait();
+  for (int e = tid; e < ns * NB; e += CR_THREADS) {
+    const int q = e / NB, comp = e - q * NB;
+    cplx v = *cl.map_shared_rank(X + (R - 1) * NB + comp, q);
+    if (q + 1 < CR_CLUSTER) v = cadd(v, *cl.map_shared_rank(V + comp, q + 1));
+    rs[e] = v;
+  }
+  __syncthreads();
+  cluster_arrive();                      // past this CTA's last remote read
+  {
+    constexpr int GL = 16;               // lanes an output
+    for (int o0 = 0; o0 < 2 * NB; o0 += CR_THREADS / GL) {
+      const int o = o0 + tid / GL, q = rank - 1 + o / NB, part = tid % GL;
+      const bool on = o < 2 * NB && q >= 0 && q < ns;
+      cplx acc = cmk(0.0, 0.0);
+      if (on) {
+        const cplx* g = S.sinv + (size_t)(q * NB + o % NB) * ns * NB;
+        for (int e = part; e < ns * NB; e += GL) acc = cfma(__ldg(g + e), rs[e], acc);
+      }
+      acc = item_sum<GL>(acc);
+      if (on && part == 0) xs[o / NB][o % NB] = acc;
+    }
+  }
+  __syncthreads();
+  for (int l = p - 1; l >= 0; --l) {
+    if ((R >> (l + 1)) * NB <= 32) channel_up<NB, 4>(c, F, l);
+    else channel_up<NB, 2>(c, F, l);
+    __syncthreads();
+  }
+  for (int e = tid; e < R * NB; e += CR_THREADS) {
+    const int comp = e >> p, i = e & (R - 1), k = k0 + i;
+    if (k >= m) continue;
+    const cplx v = i == R - 1 ? xs[1][comp] : X[i * NB + comp];
     S.e[comp * m + k] = v;
     if (S.e32) S.e32[comp * m + k] = make_float2((float)v.x, (float)v.y);
   }
+  cluster_wait();
 }
 
 // u += sum_m phi_m(x) e^A_m(y) + sum_l e^B_l(x) vphi_l(y) (Eq. (30)).  A thread takes one
@@ -337,33 +432,39 @@ cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& 
 }
 
 template <class C>
-cudaError_t launch_cc_rhs(const CCViewT<C>& c, cudaStream_t st) {
+cudaError_t launch_reduce_projections(const CCViewT<C>& c, cudaStream_t st) {
   int tot = c.nb * (c.mx + c.my);
-  cudaError_t e = mgc_launch(k_reduce_partials<C>, dim3((8 * tot + 255) / 256), dim3(256), 0, st, c.nb, c.mx, c.my,
-                             cc_tiles_x(c.mx), cc_tiles_y(c.my), c.Px_part, c.Py_part, c.Px, c.Py);
-  if (e != cudaSuccess) return e;
-  return mgc_launch(k_cc_coef, dim3(c.nb * c.nb), dim3(256), 0, st, c.nb, c.my, c.wvphi64, c.Px, c.c);
+  return mgc_launch(k_reduce_partials<C>, dim3((8 * tot + 255) / 256), dim3(256), 0, st, c.nb, c.mx, c.my,
+                    cc_tiles_x(c.mx), cc_tiles_y(c.my), c.Px_part, c.Py_part, c.Px, c.Py);
 }
+
+namespace {
+size_t channel_smem(int m, int nb) {
+  const int p = cr_log_rows(m);
+  return sizeof(cplx) * (((size_t)nb << p) + (cr_pack_in_smem(m, nb) ? cr_pack_entries(1 << p, p, nb) : 0));
+}
+}  // namespace
 
 // Clusters of more than 8 CTAs must be allowed per kernel (once, before any launch or
 // capture); called by setup.
-// Raises (never lowers) the kernel's dynamic shared-memory limit to what m_max rows need,
+// Raises (never lowers) the kernel's dynamic shared-memory limit to what the systems need,
 // so every handle set up so far can still launch.
-cudaError_t channel_solve_prepare(int nb, int m_max) {
+cudaError_t channel_solve_prepare(int nb, int mA, int mB) {
   static std::mutex mu;
   static int granted[MGC_MAX_NB + 1] = {0};
   if (nb < 1 || nb > MGC_MAX_NB) return cudaErrorInvalidValue;
-  const int smem = 2 * cr_rows(m_max) * nb * (int)sizeof(cplx);
+  const size_t a = channel_smem(mA, nb), b = channel_smem(mB, nb);
+  const int smem = (int)(a > b ? a : b);
   std::lock_guard<std::mutex> lock(mu);
   if (granted[nb] > 0 && smem <= granted[nb]) return cudaSuccess;
   const int want = smem > 48 * 1024 ? smem : 48 * 1024;
   cudaError_t e = cudaErrorInvalidValue;
   switch (nb) {
-#define MGC_PREP(K)                                                                                        \
-  case K:                                                                                                  \
-    e = cudaFuncSetAttribute(k_channel_solve_pcr<K>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); \
+#define MGC_PREP(K)                                                                                      \
+  case K:                                                                                                \
+    e = cudaFuncSetAttribute(k_channel_solve<K>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);     \
     if (e == cudaSuccess)                                                                                \
-      e = cudaFuncSetAttribute(k_channel_solve_pcr<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, want); \
+      e = cudaFuncSetAttribute(k_channel_solve<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, want);   \
     break;
     MGC_PREP(1) MGC_PREP(2) MGC_PREP(3) MGC_PREP(4) MGC_PREP(5) MGC_PREP(6) MGC_PREP(7) MGC_PREP(8)
 #undef MGC_PREP
@@ -373,20 +474,14 @@ cudaError_t channel_solve_prepare(int nb, int m_max) {
 }
 
 cudaError_t launch_channel_solve(const CRSystem& A, const CRSystem& B, cudaStream_t st) {
-  const int mm = A.m > B.m ? A.m : B.m;
-  const size_t smem = 2 * (size_t)cr_rows(mm) * A.nb * sizeof(cplx);
+  const size_t a = channel_smem(A.m, A.nb), b = channel_smem(B.m, B.nb), smem = a > b ? a : b;
   switch (A.nb) {
-    case 1: return mgc_launch(k_channel_solve_pcr<1>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 2: return mgc_launch(k_channel_solve_pcr<2>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 3: return mgc_launch(k_channel_solve_pcr<3>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 4: return mgc_launch(k_channel_solve_pcr<4>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 5: return mgc_launch(k_channel_solve_pcr<5>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 6: return mgc_launch(k_channel_solve_pcr<6>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 7: return mgc_launch(k_channel_solve_pcr<7>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
-    case 8: return mgc_launch(k_channel_solve_pcr<8>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
+#define MGC_SOLVE(K) \
+  case K: return mgc_launch(k_channel_solve<K>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);
+    MGC_SOLVE(1) MGC_SOLVE(2) MGC_SOLVE(3) MGC_SOLVE(4) MGC_SOLVE(5) MGC_SOLVE(6) MGC_SOLVE(7) MGC_SOLVE(8)
+#undef MGC_SOLVE
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <class C>
@@ -407,7 +502,7 @@ cudaError_t launch_cccs_correct(const CCViewT<C>& c, C* u, cudaStream_t st) {
 #define MGC_INSTANTIATE(C)                                                                                  \
   template cudaError_t launch_residual_project<C>(const StencilViewT<C>&, const CCViewT<C>&, const C*,     \
                                                   const C*, cudaStream_t);                                \
-  template cudaError_t launch_cc_rhs<C>(const CCViewT<C>&, cudaStream_t);                                 \
+  template cudaError_t launch_reduce_projections<C>(const CCViewT<C>&, cudaStream_t);                     \
   template cudaError_t launch_cccs_correct<C>(const CCViewT<C>&, C*, cudaStream_t);
 MGC_INSTANTIATE(double2)
 MGC_INSTANTIATE(float2)

@@ -577,12 +577,15 @@ __global__ void __launch_bounds__(256) k_channel_potentials(int rows, int len, i
 // Level l (stride s = 2^l) eliminates every row's couplings to k +- s with the rows
 // k +- s themselves: alpha = A_k B_{k-s}^{-1}, gamma = C_k B_{k+s}^{-1},
 //   A_k <- -alpha A_{k-s},  B_k <- B_k - alpha C_{k-s} - gamma A_{k+s},  C_k <- -gamma C_{k+s};
-// after ceil(log2 m) levels no coupling is left and x_k = B_k^{-1} r_k.  One launch per level
+// after ceil(log2 m) levels no coupling is left and x_k = B_k^{-1} r_k.  The first p levels
+// eliminate every other remaining row: the eliminated row leaves B_k^{-1}, B_k^{-1} A_k and
+// B_k^{-1} C_k of its level for the back substitution and takes no part in the later levels,
+// which then couple the separators (the last row of every 2^p) only.  One launch per level
 // for both systems, one warp per row with the row's blocks in shared memory; a launch ends
 // with the inverses of the blocks it made, so the next one finds its neighbours'.  The state of
 // a system is A, B, C and B^{-1} of every row, double-buffered: 8 m n_b^2 entries.
 // Bound by the latency of the inverse's pivot chain.  Two systems of 1023 rows, n_b = 3: 6.6 ms
-// as one block per system, 0.34 ms so.
+// as one block per system that updated every row at every level, 0.18 ms so.
 constexpr int CF_WARPS = 4;
 
 // The systems of both channels and what their first level is made from.
@@ -646,6 +649,13 @@ __device__ __forceinline__ cplx block_dot(int nb, const cplx* X, const cplx* Y, 
   return acc;
 }
 
+// Reduction levels of the separators' system.
+__host__ __device__ constexpr int sep_levels(int ns) {
+  int q = 0;
+  while ((1 << q) < ns) ++q;
+  return q;
+}
+
 // Level l >= 0 of the reduction, or with l = -1 its start: the blocks of the unreduced rows.
 __global__ void __launch_bounds__(32 * CF_WARPS) k_channel_factor(ChannelSetup ca, ChannelSetup cb, double E, int l,
                                                                   int* status) {
@@ -654,7 +664,9 @@ __global__ void __launch_bounds__(32 * CF_WARPS) k_channel_factor(ChannelSetup c
   const CRSystem& S = P.S;
   const int nb = S.nb, nb2 = nb * nb, m = S.m;
   const int lane = threadIdx.x & 31, k = blockIdx.x * CF_WARPS + (threadIdx.x >> 5);
-  if (k >= m || l >= S.pq) return;                         // whole warps leave; no block barrier below
+  // whole warps leave; no block barrier below
+  const int R = 1 << S.p, rank = k / R, i = k % R, pq = S.p + sep_levels(S.ns);
+  if (k >= m || l >= pq || (l > 0 && (k + 1) % (1 << min(l, S.p)) != 0)) return;
   cplx* sh = cf_sh + (size_t)(threadIdx.x >> 5) * 12 * nb2;   // ten blocks, then [B | I]
   const size_t blk = (size_t)m * nb2, row = (size_t)k * nb2;
   const int cur = (l + 2) & 1;                             // level l reads buffer cur, the start writes buffer 0
@@ -691,14 +703,30 @@ __global__ void __launch_bounds__(32 * CF_WARPS) k_channel_factor(ChannelSetup c
       Ch[e] = in[2 * blk + rh + e];
     }
     __syncwarp();
-    cplx* pa = S.pa + ((size_t)l * m + k) * nb2;
-    cplx* pg = S.pg + ((size_t)l * m + k) * nb2;
+    cplx* pack = S.pack + rank * cr_pack_entries(R, S.p, nb);
+    if (l < S.p && ((k + 1) >> l) % 2 != 0) {
+      const cplx* Bi = in + 3 * blk + row;
+      cplx* d = pack + ((size_t)(R - 1) * 2 + S.p + (size_t)i * 3) * nb2;
+      for (int e = lane; e < nb2; e += 32) {
+        const int r = e / nb, c = e - r * nb;
+        d[e] = block_dot(nb, Bi, A, r, c);
+        d[nb2 + e] = block_dot(nb, Bi, C, r, c);
+        d[2 * nb2 + e] = Bi[e];
+      }
+      return;
+    }
+    // where alpha, gamma go, and a separator's gamma also to the next CTA
+    cplx* pa = l < S.p ? pack + ((size_t)(R - (R >> l)) + (i + 1) / (2 * s) - 1) * 2 * nb2
+                       : S.sfac + ((size_t)(l - S.p) * S.ns + rank) * 2 * nb2;
+    cplx* pv = l < S.p && i == R - 1 && k + 1 < m
+                   ? pack + cr_pack_entries(R, S.p, nb) + ((size_t)(R - 1) * 2 + l) * nb2 : nullptr;
     for (int e = lane; e < nb2; e += 32) {
       const int r = e / nb, c = e - r * nb;
       al[e] = lo ? block_dot(nb, A, Il, r, c) : cmk(0.0, 0.0);
       ga[e] = hi ? block_dot(nb, C, Ih, r, c) : cmk(0.0, 0.0);
       pa[e] = al[e];
-      pg[e] = ga[e];
+      pa[nb2 + e] = ga[e];
+      if (pv) pv[e] = ga[e];
     }
     __syncwarp();
     for (int e = lane; e < nb2; e += 32) {
@@ -719,10 +747,46 @@ __global__ void __launch_bounds__(32 * CF_WARPS) k_channel_factor(ChannelSetup c
     }
   }
   __syncwarp();
-  cplx* dst = l == S.pq - 1 ? S.pbinv + row : out + 3 * blk + row;
+  // the last level's inverses (of the only level when the separators are not coupled)
+  cplx* dst = l == pq - 1 && (k + 1) % R == 0 ? S.sfac + ((size_t)(pq - S.p) * S.ns * 2 + rank) * nb2
+                                              : out + 3 * blk + row;
   if (!warp_inverse(nb, Bn, sh + 10 * nb2, dst)) {
     if (lane == 0) atomicOr(status, MGC_ST_PIVOT);
     for (int e = lane; e < nb2; e += 32) dst[e] = cmk(0.0, 0.0);
+  }
+}
+
+// Column blockIdx.x of the inverse of the separators' system: their parallel cyclic reduction
+// applied to a unit vector, one thread per (separator, component).
+__global__ void __launch_bounds__(CR_CLUSTER * MGC_MAX_NB) k_separator_inverse(CRSystem SA, CRSystem SB) {
+  __shared__ cplx x[2][CR_CLUSTER * MGC_MAX_NB];
+  const CRSystem& S = blockIdx.y == 0 ? SA : SB;
+  const int nb = S.nb, nb2 = nb * nb, n = S.ns * nb, col = blockIdx.x, e = threadIdx.x;
+  if (col >= n) return;
+  const int q = e / nb, c = e - q * nb;
+  if (e < n) x[0][e] = cmk(e == col ? 1.0 : 0.0, 0.0);
+  __syncthreads();
+  int cur = 0;
+  const int levels = sep_levels(S.ns);
+  for (int l = 0; l < levels; ++l) {
+    const int s = 1 << l;
+    if (e < n) {
+      const cplx* f = S.sfac + ((size_t)l * S.ns + q) * 2 * nb2 + c * nb;
+      cplx v = x[cur][e];
+      for (int t = 0; t < nb; ++t) {
+        if (q - s >= 0) v = cfms(f[t], x[cur][(q - s) * nb + t], v);
+        if (q + s < S.ns) v = cfms(f[nb2 + t], x[cur][(q + s) * nb + t], v);
+      }
+      x[cur ^ 1][e] = v;
+    }
+    __syncthreads();
+    cur ^= 1;
+  }
+  if (e < n) {
+    const cplx* f = S.sfac + ((size_t)levels * S.ns * 2 + q) * nb2 + c * nb;
+    cplx v = cmk(0.0, 0.0);
+    for (int t = 0; t < nb; ++t) v = cfma(f[t], x[cur][q * nb + t], v);
+    S.sinv[(size_t)e * n + col] = v;
   }
 }
 
@@ -819,22 +883,24 @@ cudaError_t launch_channel_potentials(int mx, int my, int nb, const cplx* wphi, 
   return cudaGetLastError();
 }
 
-int pcr_levels(int m) {
-  int q = 0;
-  while ((1 << q) < m) ++q;
-  return q;
+size_t channel_separator_entries(int ns, int nb) { return ((size_t)sep_levels(ns) * 2 + 1) * ns * nb * nb; }
+
+int channel_factor_launches(const CRSystem& A, const CRSystem& B) {
+  return 2 + std::max(A.p + sep_levels(A.ns), B.p + sep_levels(B.ns));   // the start, the levels, the separators
 }
 
-size_t channel_factor_pcr_scratch(int m, int nb) { return (size_t)8 * m * nb * nb; }
+size_t channel_factor_scratch(int m, int nb) { return (size_t)8 * m * nb * nb; }
 
-cudaError_t launch_channel_factor_pcr(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
+cudaError_t launch_channel_factor(const CRSystem& A, const CRSystem& B, const ChannelCoef& ca, const ChannelCoef& cb,
                                       double E, cplx* scratch, int* status, cudaStream_t st) {
-  const int nb = A.nb, mm = std::max(A.m, B.m), pq = std::max(A.pq, B.pq);
-  cplx* scrB = scratch + channel_factor_pcr_scratch(A.m, nb);
+  const int nb = A.nb, mm = std::max(A.m, B.m);
+  const int levels = channel_factor_launches(A, B) - 2;
+  cplx* scrB = scratch + channel_factor_scratch(A.m, nb);
   const ChannelSetup a{A, ca.diag, ca.v, ca.lam, ca.Vc, ca.sub, ca.sup, scratch};
   const ChannelSetup b{B, cb.diag, cb.v, cb.lam, cb.Vc, cb.sub, cb.sup, scrB};
   const dim3 grid((mm + CF_WARPS - 1) / CF_WARPS, 2);
   const size_t smem = (size_t)CF_WARPS * 12 * nb * nb * sizeof(cplx);
-  for (int l = -1; l < pq; ++l) k_channel_factor<<<grid, 32 * CF_WARPS, smem, st>>>(a, b, E, l, status);
+  for (int l = -1; l < levels; ++l) k_channel_factor<<<grid, 32 * CF_WARPS, smem, st>>>(a, b, E, l, status);
+  k_separator_inverse<<<dim3(CR_CLUSTER * nb, 2), CR_CLUSTER * nb, 0, st>>>(A, B);
   return cudaGetLastError();
 }

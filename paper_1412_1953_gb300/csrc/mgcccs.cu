@@ -202,29 +202,28 @@ void layout(mgcccs_handle* h, Carver& cv) {
       S.m = c == 0 ? my : mx;
       S.nb = nb;
       const size_t nb2 = (size_t)nb * nb;
-      S.pq = pcr_levels(S.m);
-      S.pa = cv.take<cplx>((size_t)S.pq * S.m * nb2);
-      S.pg = cv.take<cplx>((size_t)S.pq * S.m * nb2);
-      S.pbinv = cv.take<cplx>((size_t)S.m * nb2);
+      S.p = cr_log_rows(S.m);
+      S.ns = S.m >> S.p;
+      S.pack = cv.take<cplx>(CR_CLUSTER * cr_pack_entries(1 << S.p, S.p, nb));
+      S.sinv = cv.take<cplx>((size_t)S.ns * S.ns * nb2);
+      S.sfac = cv.take<cplx>(channel_separator_entries(S.ns, nb));
     }
     h->cr_scratch =
-        cv.take<cplx>(channel_factor_pcr_scratch(h->crA.m, nb) + channel_factor_pcr_scratch(h->crB.m, nb));
+        cv.take<cplx>(channel_factor_scratch(h->crA.m, nb) + channel_factor_scratch(h->crB.m, nb));
     size_t es = bound_states_scratch(mx > my ? mx : my, nb);
     h->eig_scratch = cv.take<cplx>((es + sizeof(cplx) - 1) / sizeof(cplx));
     CCView& cc = h->cc;
     cc.mx = mx; cc.my = my; cc.nb = nb;
     cc.wphi = h->wphi; cc.wvphi = h->wvphi; cc.phi = h->phi; cc.vphi = h->vphi;
-    cc.wvphi64 = h->wvphi;
     cc.Px_part = cv.take<cplx>((size_t)cc_tiles_x(mx) * nb * my);
     cc.Py_part = cv.take<cplx>((size_t)cc_tiles_y(my) * nb * mx);
     cc.Px = cv.take<cplx>((size_t)nb * my);
     cc.Py = cv.take<cplx>((size_t)nb * mx);
-    cc.c = cv.take<cplx>((size_t)nb * nb);
     cc.eA = cv.take<cplx>((size_t)nb * my);
     cc.eB = cv.take<cplx>((size_t)nb * mx);
     cc.eAc = cc.eA; cc.eBc = cc.eB;
-    h->crA.chan = 0; h->crA.P = cc.Px; h->crA.cmat = cc.c; h->crA.basis = h->vphi;
-    h->crB.chan = 1; h->crB.P = cc.Py; h->crB.cmat = cc.c; h->crB.basis = h->phi;
+    h->crA.chan = 0; h->crA.P = cc.Px; h->crA.wst = h->wvphi; h->crA.basis = h->vphi;
+    h->crB.chan = 1; h->crB.P = cc.Py; h->crB.wst = h->wphi; h->crB.basis = h->phi;
     h->crA.e = cc.eA; h->crA.e32 = nullptr;
     h->crB.e = cc.eB; h->crB.e32 = nullptr;
     if (p.precision == 1) {
@@ -237,13 +236,12 @@ void layout(mgcccs_handle* h, Carver& cv) {
       c3.wphi = h->wphi32; c3.wvphi = h->wvphi32; c3.phi = h->phi32; c3.vphi = h->vphi32;
       c3.Px_part = cv.take<float2>((size_t)cc_tiles_x(mx) * nb * my);
       c3.Py_part = cv.take<float2>((size_t)cc_tiles_y(my) * nb * mx);
-      c3.Px = cc.Px; c3.Py = cc.Py; c3.c = cc.c; c3.eA = cc.eA; c3.eB = cc.eB;
+      c3.Px = cc.Px; c3.Py = cc.Py; c3.eA = cc.eA; c3.eB = cc.eB;
       float2* eA32 = cv.take<float2>((size_t)nb * my);
       float2* eB32 = cv.take<float2>((size_t)nb * mx);
       c3.eAc = eA32; c3.eBc = eB32;
       h->crA.e32 = eA32;
       h->crB.e32 = eB32;
-      c3.wvphi64 = h->wvphi;
     }
   }
   StencilView s0{};
@@ -425,7 +423,7 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
   if (h->nb > 0) {
     const LevelBufs& b = h->lv[0];
     const int nb = h->nb;
-    MGC_CUDA(channel_solve_prepare(nb, h->crA.m > h->crB.m ? h->crA.m : h->crB.m));
+    MGC_CUDA(channel_solve_prepare(nb, h->crA.m, h->crB.m));
     if (lam_in) {
       // states supplied by the caller (a previous setup on the same grid and V1, V2)
       MGC_CUDA(cudaMemcpyAsync(h->lam, lam_in, sizeof(cplx) * nb, cudaMemcpyHostToDevice, st));
@@ -460,8 +458,8 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
     // channel A runs along y with the x bound states; channel B along x with the y ones
     const ChannelCoef ca{b.diag_y, v2, h->lam, h->VA, b.west_y, b.east_y};
     const ChannelCoef cb{b.diag_x, v1, h->mu, h->VB, b.west_x, b.east_x};
-    MGC_LAUNCH(launch_channel_factor_pcr(h->crA, h->crB, ca, cb, p.E, h->cr_scratch, h->status, st));
-    h->launches += std::max(h->crA.pq, h->crB.pq);   // one kernel per level after the first
+    MGC_LAUNCH(launch_channel_factor(h->crA, h->crB, ca, cb, p.E, h->cr_scratch, h->status, st));
+    h->launches += channel_factor_launches(h->crA, h->crB) - 1;
   }
   int rc0 = coarse_inverse_check(h);
   if (rc0) return rc0;
@@ -620,8 +618,7 @@ int cccs_fine(mgcccs_handle* h, C* u, const C* f) {
   cudaStream_t st = h->st;
   const CCViewT<C>& cc = cc_view<C>(h);
   MGC_LAUNCH(launch_residual_project(*level_io<C>(h, 0).sv, cc, (const C*)u, f, st));
-  MGC_LAUNCH(launch_cc_rhs(cc, st));
-  h->launches += 1;   // launch_cc_rhs issues two kernels
+  MGC_LAUNCH(launch_reduce_projections(cc, st));
   MGC_LAUNCH(launch_channel_solve(h->crA, h->crB, st));
   MGC_LAUNCH(launch_cccs_correct(cc, u, st));
   return MGCCCS_OK;

@@ -69,12 +69,15 @@ def test_bound_state_residuals(nx, ny, levels, nb):
             assert np.abs(np.sort(l.real) - ev.real).max() <= 1e-11 * scale
 
 
-# every block size, rows short of and beyond a multiple of the rows per block
-@pytest.mark.parametrize("nx,ny,nb", [(16, 24, 1), (24, 16, 2), (40, 24, 4), (64, 72, 5), (48, 64, 7), (72, 40, 8)])
+# every block size, rows short of and beyond a multiple of the rows per block, and (from 128 rows
+# on, by n_b) one to four elimination levels with different counts on the two axes
+@pytest.mark.parametrize("nx,ny,nb", [(16, 24, 1), (24, 16, 2), (40, 24, 4), (64, 72, 5), (48, 64, 7), (72, 40, 8),
+                                      (4, 4, 2), (152, 248, 8), (496, 208, 4), (368, 496, 6)])
 def test_channel_factors(nx, ny, nb):
     prob = _problem(nx, ny)
-    so = O.Solver(O.params_from_problem(prob, levels=3, n_b=nb), prob.v1, prob.v2, prob.v12)
-    sg = M.Solver(M.params_for(prob, levels=3, n_b=nb), prob.v1, prob.v2, prob.v12)
+    levels = 1 if nx < 8 else 4 if nx > 128 else 3
+    so = O.Solver(O.params_from_problem(prob, levels=levels, n_b=nb), prob.v1, prob.v2, prob.v12)
+    sg = M.Solver(M.params_for(prob, levels=levels, n_b=nb), prob.v1, prob.v2, prob.v12)
     g = np.random.default_rng(nb)
     u = g.standard_normal(prob.f.shape) + 1j * g.standard_normal(prob.f.shape)
     ud = torch.as_tensor(u).to("cuda")
