@@ -457,12 +457,15 @@ cudaError_t launch_round_copy(long long n, const cplx* a, float2* b, cudaStream_
 cudaError_t launch_promote(long long n, const float2* x, cplx* y, cudaStream_t st);
 
 // kernels_krylov.cu
+cudaError_t krylov_prepare();                 // before the first launch of a handle
 // grid of the grid-stride Krylov kernels: per_sm blocks of 256 threads per SM at most
 int krylov_blocks(long long n, int per_sm);
-int multidot_blocks(long long n, int k);
+template <class C>
+int multidot_blocks(long long n, int k);   // C the element type of the vectors
 template <class C>
 cudaError_t launch_multidot(long long n, int k, const C* V, long long ld, const C* w, cplx* partial,
                             int nblk, const int* gate, cudaStream_t st);
+int multiaxpy_blocks(long long n);                 // of a complex128 update
 cudaError_t launch_reduce_dots(int nblk, int k, const cplx* partial, cplx* out, cplx* acc_into, cudaStream_t st);
 template <class C>
 cudaError_t launch_multiaxpy(long long n, int k, const C* V, long long ld, const cplx* coef, double sgn,

@@ -1,0 +1,60 @@
+// Sums of FP64 products on the integer pipes.
+//
+// This part issues a warp's FP64 instruction over 64 cycles of its quarter of an SM, a 32 x 32 ->
+// 64-bit integer multiply-add over 4 and other integer operations over 2 (measured: 1.7, 32.6 and
+// 66 lane operations per clock and SM).  A complex FP64 multiply-add is 4 FP64 instructions, 256
+// cycles; below it is 12 integer multiply-adds and, for an operand not converted before, about 26
+// integer operations, 48 and 52 cycles that overlap.
+//
+// A double x = +-m 2^(e - 1075) (m the 53-bit significand, e the biased exponent) becomes, for a
+// common exponent E >= e, the integer +-((16 m) >> (E - e)) of at most 57 bits, that is x to within
+// 2^(E - 1079): four bits more than a double of the largest magnitude keeps, so an operand that
+// shares E with one up to 16 times as large is still exact to its last bit.  It is held as two
+// limbs h 2^29 + l of its sign (|h| < 2^28, |l| < 2^29).  In a product (h h' 2^58 + (h l' + l h')
+// 2^29 + l l') the last term, below 2^-56 of the largest product and of either sign, is dropped;
+// the sums of the others are exact in 64 bits for FX_TERMS complex terms, and are then rounded to
+// a double once.  Against FP64 multiply-adds, which round each partial sum to 2^-53 of itself, the
+// error stays below that of the same sum (measured at each kernel).
+//
+// Largest exponents outside FX_MIN..FX_MAX (nothing but zeros and subnormals, huge, infinite or
+// NaN operands) take the FP64 instructions; fx_ok tells.
+#pragma once
+#include "common.cuh"
+
+constexpr int FX_MIN = 600, FX_MAX = 1446;       // biased exponents; a product's scale stays normal
+constexpr int FX_TERMS = 8;                      // complex terms between two roundings
+
+__device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool fx_ok(int E) { return (unsigned)(E - FX_MIN) <= (unsigned)(FX_MAX - FX_MIN); }
+
+struct FxLimbs {
+  int h, l;
+};
+// x, of exponent e, for the common exponent E >= e: the significand left-justified in 64 bits, its 57 bits
+// from position 7 + E - e on, and the sign multiplied in (on the other integer pipe).
+__device__ __forceinline__ FxLimbs fx_limbs(double x, int e, int E) {
+  const int hi = __double2hiint(x), s = (hi >> 31) | 1;
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned a1 = __funnelshift_l(lo, ((unsigned)hi & 0xfffffu) | 0x100000u, 11), a0 = lo << 11;
+  const int t = min(E + 7 - e, 63);
+  const unsigned long long m = (unsigned long long)a1 << 32 | a0;
+  const int h = (int)__funnelshift_rc(a1, 0u, t - 3), l = (int)((unsigned)(m >> t) & 0x1fffffffu);
+  return FxLimbs{h * s, l * s};
+}
+__device__ __forceinline__ FxLimbs fx_neg(FxLimbs a) { return FxLimbs{-a.h, -a.l}; }
+
+// The two exact partial sums of sum a b.
+struct FxSum {
+  long long hh, mid;
+};
+__device__ __forceinline__ void fx_mac(FxSum& s, FxLimbs a, FxLimbs b) {
+  s.hh += (long long)a.h * b.h;
+  s.mid += (long long)a.h * b.l;
+  s.mid += (long long)a.l * b.h;
+}
+// acc + the sum of products with exponents that add up to E2, rounded; the sum is cleared.
+__device__ __forceinline__ double fx_flush(FxSum& s, int E2, double acc) {
+  const long long t = s.hh + ((s.mid + (1LL << 28)) >> 29);
+  s.hh = s.mid = 0;
+  return fma((double)t, __hiloint2double((E2 - 2100 + 1023) << 20, 0), acc);
+}

@@ -6,7 +6,7 @@
 // device, so the host only reads one residual estimate per step.
 //
 // Basis vectors are stored contiguously: V_i = V + i * ld.
-#include "common.cuh"
+#include "fixed.cuh"
 
 namespace {
 
@@ -63,6 +63,327 @@ __global__ void __launch_bounds__(NT) k_multidot(long long n, const C* __restric
   cplx tot = block_sum_c<NT>(acc, sh);
   if (threadIdx.x == 0) partial[(size_t)i * gridDim.x + blockIdx.x] = tot;
 }
+
+// ---- complex128 Gram-Schmidt on the integer pipes (fixed.cuh).  With FP64 instructions the pair
+// runs at the FP64 pipe's rate, a third of the HBM bandwidth.
+
+// Asynchronous 16-byte copy to shared memory (_if: zeros when !ok), and the wait for all but the last
+// N groups of them.  A lane reads back only what it copied, so no barrier is involved.
+__device__ __forceinline__ void copy16(cplx* dst, const cplx* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy16_if(cplx* dst, const cplx* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// The multi-dot: a block takes DG vectors, so that w is converted once for all of them, and a
+// warp DU x 32 consecutive points at a time, the last 32 of them with FP64 instructions, which
+// otherwise idle.  The exponents of w and of each vector are the largest met so far (a warp's
+// own); a larger one first rounds the sums held so far.  The sequence of chunks (w, then each
+// vector, of one tile after another) is fetched DS - 1 chunks ahead.  About 90 instructions a
+// product and the 16 warps that 128 registers allow bound it.  1023^2, 12 vectors (12 and 1
+// of 16.7 MB read): 88.0 us with FP64 multiply-adds, 63 with 64-bit shifts of masked keys in the
+// conversion, 58 before the FP64 share, 53.7 us now, 3.7 TB/s.
+constexpr int DG = 4, DU = 4, DS = 4;
+
+__global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const cplx* __restrict__ V, long long ld,
+                                                       const cplx* __restrict__ w, cplx* __restrict__ partial,
+                                                       const int* __restrict__ gate) {
+  mgc_pdl_enter();
+  extern __shared__ cplx gs_sh[];                      // [warp][DS][DU][32], then the block sums
+  const int i0 = blockIdx.y * DG, nv = min(DG, k - i0), tid = threadIdx.x, lane = tid & 31;
+  if (gate && *gate == 0) {
+    if (tid < nv) partial[(size_t)(i0 + tid) * gridDim.x + blockIdx.x] = cmk(0.0, 0.0);
+    return;
+  }
+  cplx* const ring = gs_sh + (size_t)(tid >> 5) * DS * DU * 32 + lane;
+  const long long step = (long long)gridDim.x * NT * DU;
+  long long p0 = (long long)blockIdx.x * NT * DU + (tid >> 5) * 32 * DU;   // the warp's tile
+  // the next chunk to fetch: vector fi (0: w, i: vector i0 + i - 1) of the tile at fp
+  const cplx* const Vg = V + (size_t)i0 * ld;
+  const cplx* fv = w;
+  long long fp = p0;
+  int fi = 0, fs = 0;
+  auto fetch = [&]() {
+    if (fp < n) {
+      const cplx* src = fv + fp + lane;
+      if (fp + 32 * DU <= n) {
+#pragma unroll
+        for (int u = 0; u < DU; ++u) copy16(ring + (fs * DU + u) * 32, src + 32 * u);
+      } else {
+#pragma unroll
+        for (int u = 0; u < DU; ++u) copy16_if(ring + (fs * DU + u) * 32, src + 32 * u, fp + lane + 32 * u < n);
+      }
+      fv = fi == 0 ? Vg : fv + ld;
+      if (++fi > nv) {
+        fi = 0;
+        fv = w;
+        fp += step;
+      }
+    }
+    fs = (fs + 1) % DS;
+    copy_commit();
+  };
+  int rs = 0;
+  int ex[DU], ey[DU];                                  // exponents of the chunk taken last
+  auto take = [&](cplx (&v)[DU]) {                     // the oldest chunk; returns its largest exponent
+    copy_wait<DS - 2>();
+    int e = 0;
+#pragma unroll
+    for (int u = 0; u < DU; ++u) {
+      v[u] = ring[(rs * DU + u) * 32];
+      ex[u] = fx_exp(v[u].x);
+      ey[u] = fx_exp(v[u].y);
+      e = max(max(e, ex[u]), ey[u]);
+    }
+    rs = (rs + 1) % DS;
+    fetch();
+    return (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  };
+  cplx sum[DG];
+  FxSum re[DG], im[DG];
+  int E[DG], Ew = 0;
+#pragma unroll
+  for (int i = 0; i < DG; ++i) {
+    sum[i] = cmk(0.0, 0.0);
+    re[i] = im[i] = FxSum{0, 0};
+    E[i] = 0;
+  }
+  auto flush = [&](int i) {
+    if (!fx_ok(Ew) || !fx_ok(E[i])) return;            // nothing was summed at these exponents
+    sum[i].x = fx_flush(re[i], Ew + E[i], sum[i].x);
+    sum[i].y = fx_flush(im[i], Ew + E[i], sum[i].y);
+  };
+#pragma unroll
+  for (int c = 0; c < DS - 1; ++c) fetch();
+  int held = 0;                                        // terms in the sums
+  for (; p0 < n; p0 += step) {
+    cplx v[DU];
+    const int et = take(v);
+    if (et > Ew || held + DU - 1 > FX_TERMS) {
+#pragma unroll
+      for (int i = 0; i < DG; ++i) flush(i);
+      held = 0;
+      Ew = max(Ew, et);
+    }
+    held += DU - 1;
+    FxLimbs wx[DU - 1], wy[DU - 1];
+    const cplx wl = v[DU - 1];
+#pragma unroll
+    for (int u = 0; u < DU - 1; ++u) {
+      wx[u] = fx_limbs(v[u].x, ex[u], Ew);
+      wy[u] = fx_limbs(v[u].y, ey[u], Ew);
+    }
+#pragma unroll
+    for (int i = 0; i < DG; ++i) {
+      if (i >= nv) break;
+      const int ei = take(v);
+      if (ei > E[i]) {
+        flush(i);
+        E[i] = ei;
+      }
+      if (fx_ok(Ew) && fx_ok(E[i])) {
+#pragma unroll
+        for (int u = 0; u < DU - 1; ++u) {
+          const FxLimbs ax = fx_limbs(v[u].x, ex[u], E[i]), ay = fx_limbs(v[u].y, ey[u], E[i]);
+          fx_mac(re[i], ax, wx[u]);
+          fx_mac(re[i], ay, wy[u]);
+          fx_mac(im[i], ax, wy[u]);
+          fx_mac(im[i], fx_neg(ay), wx[u]);
+        }
+        const cplx a = v[DU - 1];
+        sum[i].x = fma(a.x, wl.x, fma(a.y, wl.y, sum[i].x));
+        sum[i].y = fma(a.x, wl.y, fma(-a.y, wl.x, sum[i].y));
+      } else {
+#pragma unroll
+        for (int u = 0; u < DU; ++u) {
+          const long long p = p0 + lane + 32 * u;
+          const cplx b = p < n ? __ldg(w + p) : cmk(0.0, 0.0);
+          sum[i].x = fma(v[u].x, b.x, fma(v[u].y, b.y, sum[i].x));
+          sum[i].y = fma(v[u].x, b.y, fma(-v[u].y, b.x, sum[i].y));
+        }
+      }
+    }
+  }
+  copy_wait<0>();
+  __syncthreads();
+  double (*sh)[NT] = reinterpret_cast<double (*)[NT]>(gs_sh);
+#pragma unroll
+  for (int i = 0; i < DG; ++i) {
+    flush(i);
+    sh[2 * i][tid] = sum[i].x;
+    sh[2 * i + 1][tid] = sum[i].y;
+  }
+  __syncthreads();
+  // warp q sums component q over the block's threads (fixed order)
+  const int q = tid >> 5;
+  static_assert(2 * DG == NT / 32, "one warp per component");
+  double tot = sh[q][lane];
+#pragma unroll
+  for (int t = 1; t < NT / 32; ++t) tot += sh[q][lane + 32 * t];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+  if (lane == 0 && (q >> 1) < nv) {
+    double* out = reinterpret_cast<double*>(partial + (size_t)(i0 + (q >> 1)) * gridDim.x + blockIdx.x);
+    const bool self = Vg + (q >> 1) * ld == w;         // w itself: |w|^2, exactly real
+    out[q & 1] = self && (q & 1) ? 0.0 : tot;
+  }
+}
+constexpr int MULTIDOT_SMEM = NT * DS * DU * (int)sizeof(cplx);
+static_assert(MULTIDOT_SMEM >= 2 * DG * NT * (int)sizeof(double), "the block sums reuse the ring");
+
+// The update w += sgn sum_i coef[i] V_i.  The coefficients are converted once per block, each
+// with its own exponent; a warp's sums over the vectors share the exponent of the largest product
+// met so far (at first that of the largest coefficient and the first vector).  A warp takes
+// UU x 32 points at a time and fetches the chunks (w, then each vector) ahead, as above.
+// 1023^2, 11 vectors: 90.1 us with FP64 multiply-adds, 49.5 us now (UU = 4; 58 with UU = 2, which
+// is the faster at 255^2: 7.6 against 11.4 us, few tiles a warp), 4.4 TB/s.
+constexpr int UF = 16;                                 // chunks in flight x points a lane
+
+template <int UU>
+__global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long n, int k, const cplx* __restrict__ V, long long ld,
+                                                        const cplx* __restrict__ coef, double sgn,
+                                                        cplx* __restrict__ w, double* __restrict__ norm_part,
+                                                        const int* __restrict__ gate, const int* __restrict__ dk) {
+  mgc_pdl_enter();
+  constexpr int AS = UF / UU;
+  extern __shared__ cplx gs_sh[];                      // [warp][AS][UU][32]
+  __shared__ cplx sc[64];
+  __shared__ int4 sl[64];                              // limbs of re and im
+  __shared__ int se[64];
+  __shared__ int smax;
+  __shared__ double sh[NT / 32];
+  if (gate && *gate == 0) return;
+  if (dk) k = min(k, *dk);
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) smax = 0;
+  __syncthreads();
+  for (int i = tid; i < k; i += NT) {
+    const cplx q = cscal(sgn, coef[i]);
+    const int ex = fx_exp(q.x), ey = fx_exp(q.y), e = max(ex, ey);
+    const FxLimbs x = fx_limbs(q.x, ex, e), y = fx_limbs(q.y, ey, e);
+    sc[i] = q;
+    sl[i] = make_int4(x.h, x.l, y.h, y.l);
+    se[i] = e;
+    atomicMax(&smax, e);
+  }
+  __syncthreads();
+  cplx* const ring = gs_sh + (size_t)(tid >> 5) * AS * UU * 32 + lane;
+  const long long step = (long long)gridDim.x * NT * UU;
+  long long p0 = (long long)blockIdx.x * NT * UU + (tid >> 5) * 32 * UU;
+  const cplx* fv = w;
+  long long fp = p0;
+  int fi = 0, fs = 0, rs = 0;
+  auto fetch = [&]() {
+    if (fp < n) {
+      const cplx* src = fv + fp + lane;
+      if (fp + 32 * UU <= n) {
+#pragma unroll
+        for (int u = 0; u < UU; ++u) copy16(ring + (fs * UU + u) * 32, src + 32 * u);
+      } else {
+#pragma unroll
+        for (int u = 0; u < UU; ++u) copy16_if(ring + (fs * UU + u) * 32, src + 32 * u, fp + lane + 32 * u < n);
+      }
+      fv = fi == 0 ? V : fv + ld;
+      if (++fi > k) {
+        fi = 0;
+        fv = w;
+        fp += step;
+      }
+    }
+    fs = (fs + 1) % AS;
+    copy_commit();
+  };
+  auto take = [&](cplx (&v)[UU]) {
+    copy_wait<AS - 2>();
+#pragma unroll
+    for (int u = 0; u < UU; ++u) v[u] = ring[(rs * UU + u) * 32];
+    rs = (rs + 1) % AS;
+    fetch();
+  };
+#pragma unroll
+  for (int c = 0; c < AS - 1; ++c) fetch();
+  double n2 = 0.0;
+  for (; p0 < n; p0 += step) {
+    cplx acc[UU];
+    FxSum re[UU], im[UU];
+    take(acc);
+#pragma unroll
+    for (int u = 0; u < UU; ++u) re[u] = im[u] = FxSum{0, 0};
+    int E2 = 0, held = 0;
+    auto flush = [&]() {
+      if (held == 0) return;
+#pragma unroll
+      for (int u = 0; u < UU; ++u) {
+        acc[u].x = fx_flush(re[u], E2, acc[u].x);
+        acc[u].y = fx_flush(im[u], E2, acc[u].y);
+      }
+      held = 0;
+    };
+    for (int i = 0; i < k; ++i) {
+      cplx v[UU];
+      take(v);
+      int ex[UU], ey[UU], e = 0;
+#pragma unroll
+      for (int u = 0; u < UU; ++u) {
+        ex[u] = fx_exp(v[u].x);
+        ey[u] = fx_exp(v[u].y);
+        e = max(max(e, ex[u]), ey[u]);
+      }
+      const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)e), ec = se[i];
+      if (fx_ok(ev) && fx_ok(ec)) {
+        if (ev + ec > E2 || held == FX_TERMS) {
+          flush();
+          // the first time: room for the largest coefficient
+          E2 = max(E2, i == 0 && fx_ok(smax) ? ev + smax : ev + ec);
+        }
+        ++held;
+        const int4 c = sl[i];
+        const FxLimbs cx{c.x, c.y}, cy{c.z, c.w}, my = fx_neg(cy);
+        const int E = E2 - ec;
+#pragma unroll
+        for (int u = 0; u < UU; ++u) {
+          const FxLimbs x = fx_limbs(v[u].x, ex[u], E), y = fx_limbs(v[u].y, ey[u], E);
+          fx_mac(re[u], x, cx);
+          fx_mac(re[u], y, my);
+          fx_mac(im[u], y, cx);
+          fx_mac(im[u], x, cy);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < UU; ++u) acc[u] = cfma(sc[i], v[u], acc[u]);
+      }
+    }
+    flush();
+#pragma unroll
+    for (int u = 0; u < UU; ++u)
+      if (p0 + lane + 32 * u < n) {
+        w[p0 + lane + 32 * u] = acc[u];
+        if (norm_part) n2 += cabs2(acc[u]);
+      }
+  }
+  copy_wait<0>();
+  if (norm_part) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n2 += __shfl_down_sync(0xffffffffu, n2, o);
+    if (lane == 0) sh[tid >> 5] = n2;
+    __syncthreads();
+    if (tid == 0) {
+      double tot = 0.0;
+      for (int q = 0; q < NT / 32; ++q) tot += sh[q];
+      norm_part[blockIdx.x] = tot;
+    }
+  }
+}
+constexpr int MULTIAXPY_SMEM = NT * UF * (int)sizeof(cplx);
 
 // out[i] = sum_b partial[i][b] (fixed order); acc_into[i] += out[i] when given.
 __global__ void __launch_bounds__(NT) k_reduce_dots(int nblk, const cplx* __restrict__ partial,
@@ -399,16 +720,40 @@ __global__ void k_zero_c(int n, cplx* __restrict__ a) {
 
 }  // namespace
 
+// The dynamic shared memory of the complex128 pair, allowed once per handle setup.
+cudaError_t krylov_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(k_multidot_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, MULTIDOT_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_multiaxpy_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MULTIAXPY_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_multiaxpy_fx<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, MULTIAXPY_SMEM);
+  return e;
+}
+
 int krylov_blocks(long long n, int per_sm) {
   const long long b = (n + NT - 1) / NT, cap = (long long)per_sm * mgc_sm_count();
+  return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
+}
+
+// Four points a lane once they fill the resident blocks several times over, else two.
+static bool axpy_wide(long long n) { return n >= 4LL * 2 * mgc_sm_count() * NT; }
+int multiaxpy_blocks(long long n) {
+  const long long b = (n + NT * 2 - 1) / (NT * 2), cap = (axpy_wide(n) ? 2LL : 3LL) * mgc_sm_count();
   return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
 }
 
 // Blocks per vector of a k-vector multi-dot: about one full wave (8 blocks per SM) over
 // all k vectors, so that each thread folds many elements before its share of the block
 // reduction; never more than krylov_blocks(n), never fewer than 64.
+template <class C>
 int multidot_blocks(long long n, int k) {
   const int cap = krylov_blocks(n, 4);
+  if constexpr (sizeof(C) == sizeof(cplx)) {
+    // two resident blocks per SM over the groups of DG vectors
+    const long long tiles = (n + NT * DU - 1) / (NT * DU), fill = 2LL * mgc_sm_count() / ((k + DG - 1) / DG);
+    const long long b = tiles < fill ? tiles : fill;
+    return (int)(b < 1 ? 1 : b < cap ? b : cap);
+  }
   int b = 8 * mgc_sm_count() / (k < 1 ? 1 : k);
   if (b < 64) b = 64;
   return b < cap ? b : cap;
@@ -417,7 +762,11 @@ int multidot_blocks(long long n, int k) {
 template <class C>
 cudaError_t launch_multidot(long long n, int k, const C* V, long long ld, const C* w, cplx* partial,
                             int nblk, const int* gate, cudaStream_t st) {
-  return mgc_launch(k_multidot<C>, dim3(nblk, k), dim3(NT), 0, st, n, V, ld, w, partial, gate);
+  if constexpr (sizeof(C) == sizeof(cplx))
+    return mgc_launch(k_multidot_fx, dim3(nblk, (k + DG - 1) / DG), dim3(NT), MULTIDOT_SMEM, st, n, k, V, ld, w,
+                      partial, gate);
+  else
+    return mgc_launch(k_multidot<C>, dim3(nblk, k), dim3(NT), 0, st, n, V, ld, w, partial, gate);
 }
 
 cudaError_t launch_reduce_dots(int nblk, int k, const cplx* partial, cplx* out, cplx* acc_into, cudaStream_t st) {
@@ -427,12 +776,19 @@ cudaError_t launch_reduce_dots(int nblk, int k, const cplx* partial, cplx* out, 
 template <class C>
 cudaError_t launch_multiaxpy(long long n, int k, const C* V, long long ld, const cplx* coef, double sgn,
                              C* w, double* norm_part, int nblk, const int* gate, cudaStream_t st, const int* dk) {
-  if constexpr (sizeof(C) == sizeof(float2)) {
+  if constexpr (sizeof(C) == sizeof(cplx)) {
+    if (axpy_wide(n))
+      return mgc_launch(k_multiaxpy_fx<4>, dim3(nblk), dim3(NT), MULTIAXPY_SMEM, st, n, k, V, ld, coef, sgn, w, norm_part,
+                        gate, dk);
+    return mgc_launch(k_multiaxpy_fx<2>, dim3(nblk), dim3(NT), MULTIAXPY_SMEM, st, n, k, V, ld, coef, sgn, w, norm_part,
+                      gate, dk);
+  } else {
     if (pairs_ok(V, w, ld)) {
       return mgc_launch(k_multiaxpy_c64, dim3(nblk), dim3(NT), 0, st, n, k, V, ld, coef, sgn, w, norm_part, gate, dk);
     }
   }
-  return mgc_launch(k_multiaxpy<C>, dim3(nblk), dim3(NT), 0, st, n, k, V, ld, coef, sgn, w, norm_part, gate, dk);
+  if constexpr (sizeof(C) == sizeof(float2))
+    return mgc_launch(k_multiaxpy<C>, dim3(nblk), dim3(NT), 0, st, n, k, V, ld, coef, sgn, w, norm_part, gate, dk);
 }
 
 template <class C>
@@ -442,6 +798,7 @@ cudaError_t launch_scale_by_norm(long long n, const C* w, C* out, const double* 
 }
 
 #define MGC_INSTANTIATE(C)                                                                                  \
+  template int multidot_blocks<C>(long long, int);                                                          \
   template cudaError_t launch_multidot<C>(long long, int, const C*, long long, const C*, cplx*, int,        \
                                          const int*, cudaStream_t);                                       \
   template cudaError_t launch_multiaxpy<C>(long long, int, const C*, long long, const cplx*, double, C*,   \

@@ -251,9 +251,9 @@ void layout(mgcccs_handle* h, Carver& cv) {
   h->norm_nparts = nparts > n2b ? nparts : n2b;
   const long long N = (long long)mx * my;
   h->km = p.krylov_restart;
-  // complex128 Krylov kernels are FP64-bound at 4 blocks per SM; the complex64 update is
-  // bound by memory latency and gets 6, which its register count allows
-  h->kr_nblk = krylov_blocks(N, p.precision == 1 ? 6 : 4);
+  // blocks of the Gram-Schmidt update: for complex64, which is bound by memory latency, the six
+  // per SM that its register count allows
+  h->kr_nblk = p.precision == 1 ? krylov_blocks(N, 6) : multiaxpy_blocks(N);
   h->kld = (N + 31) / 32 * 32;
   if (h->km > 0) {
     const int m = h->km;
@@ -272,7 +272,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
     h->g = cv.take<cplx>(m + 1);
     h->y = cv.take<cplx>(m);
     h->hc = cv.take<cplx>(m + 1);
-    h->dotpart = cv.take<cplx>((size_t)(m + 1) * h->kr_nblk);
+    h->dotpart = cv.take<cplx>((size_t)(m + 1) * krylov_blocks(N, 4));   // multidot_blocks at most
     h->gate = cv.take<int>(4);
     h->ctl = cv.take<SolveCtl>(1);
     if (h->kr_nblk > h->norm_nparts) h->norm_nparts = h->kr_nblk;
@@ -377,6 +377,7 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
              const cplx* phi_in = nullptr, const cplx* mu_in = nullptr, const cplx* vphi_in = nullptr) {
   const mgcccs_params& p = h->p;
   cudaStream_t st = h->st;
+  MGC_CUDA(krylov_prepare());
   MGC_CUDA(cudaMemsetAsync(h->status, 0, 8 * sizeof(int), st));
   MGC_CUDA(cudaMemcpyAsync(h->v1c, v1, sizeof(cplx) * h->lv[0].mx, cudaMemcpyDeviceToDevice, st));
   MGC_CUDA(cudaMemcpyAsync(h->v2c, v2, sizeof(cplx) * h->lv[0].my, cudaMemcpyDeviceToDevice, st));
@@ -761,7 +762,7 @@ int issue_arnoldi_step(mgcccs_handle* h, int j) {
   // Gram-Schmidt, first pass: H(0:j, j) = V^H w ; w -= V H(0:j, j).  w is column j+1 of V,
   // so the multi-dot over columns 0..j+1 also yields |w|^2 (for the reorthogonalisation
   // test), left in H(j+1, j) until the Givens rotation writes that entry.
-  const int nbd = multidot_blocks(N, j + 2);
+  const int nbd = multidot_blocks<C>(N, j + 2);
   MGC_LAUNCH(launch_multidot(N, j + 2, (const C*)V, ld, (const C*)w, h->dotpart, nbd, (const int*)nullptr, st));
   MGC_LAUNCH(launch_reduce_dots(nbd, j + 2, h->dotpart, col, nullptr, st));
   const double* w_norm2 = reinterpret_cast<const double*>(col + j + 1);
@@ -1598,7 +1599,7 @@ int mgcccs_gs_dots(mgcccs_t h, const mgcccs_c128* V, long long ld, int k, const 
   if (!h || !V || !w || !out || h->km < 1 || k < 1 || k > h->km + 1) return MGCCCS_EINVAL;
   const long long N = (long long)h->lv[0].mx * h->lv[0].my;
   if (ld < N) return MGCCCS_EINVAL;
-  const int nbd = multidot_blocks(N, k);
+  const int nbd = multidot_blocks<cplx>(N, k);
   MGC_LAUNCH(launch_multidot(N, k, reinterpret_cast<const cplx*>(V), ld, reinterpret_cast<const cplx*>(w),
                              h->dotpart, nbd, (const int*)nullptr, h->st));
   MGC_LAUNCH(launch_reduce_dots(nbd, k, h->dotpart, reinterpret_cast<cplx*>(out), nullptr, h->st));
@@ -1612,8 +1613,8 @@ int mgcccs_gs_update(mgcccs_t h, const mgcccs_c128* V, long long ld, int k, cons
   const long long N = (long long)h->lv[0].mx * h->lv[0].my;
   if (ld < N) return MGCCCS_EINVAL;
   MGC_LAUNCH(launch_multiaxpy(N, k, reinterpret_cast<const cplx*>(V), ld, reinterpret_cast<const cplx*>(coef),
-                              -1.0, reinterpret_cast<cplx*>(w), (double*)nullptr, h->kr_nblk, (const int*)nullptr,
-                              h->st));
+                              -1.0, reinterpret_cast<cplx*>(w), (double*)nullptr, multiaxpy_blocks(N),
+                              (const int*)nullptr, h->st));
   return MGCCCS_OK;
 }
 
@@ -1623,7 +1624,7 @@ int mgcccs_gs_dots_c64(mgcccs_t h, const mgcccs_c64* V, long long ld, int k, con
   if (!h || !V || !w || !out || h->km < 1 || k < 1 || k > h->km + 1) return MGCCCS_EINVAL;
   const long long N = (long long)h->lv[0].mx * h->lv[0].my;
   if (ld < N) return MGCCCS_EINVAL;
-  const int nbd = multidot_blocks(N, k);
+  const int nbd = multidot_blocks<float2>(N, k);
   MGC_LAUNCH(launch_multidot(N, k, reinterpret_cast<const float2*>(V), ld, reinterpret_cast<const float2*>(w),
                              h->dotpart, nbd, (const int*)nullptr, h->st));
   MGC_LAUNCH(launch_reduce_dots(nbd, k, h->dotpart, reinterpret_cast<cplx*>(out), nullptr, h->st));
