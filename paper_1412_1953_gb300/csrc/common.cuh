@@ -578,7 +578,8 @@ __host__ __device__ constexpr bool cr_pack_in_smem(int m, int nb) {
   return 16 * (cr_pack_entries(1 << p, p, nb) + ((size_t)nb << p)) <= 200 * 1024;
 }
 int cc_tiles_x(int mx);
-int cc_tiles_y(int my);
+int cc_tile_rows(int mx, int my);   // rows per warp of a CCCS tile (8 warps): 1, 2 or 4
+int cc_tiles_y(int mx, int my);
 template <class C>
 cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f,
                                     cudaStream_t st);

@@ -52,6 +52,25 @@ __device__ __forceinline__ void fx_mac(FxSum& s, FxLimbs a, FxLimbs b) {
   s.mid += (long long)a.h * b.l;
   s.mid += (long long)a.l * b.h;
 }
+// Carry the middle sum into the upper one, so that FX_TERMS more terms fit (the upper sum itself
+// holds 4 FX_TERMS terms).
+__device__ __forceinline__ void fx_carry(FxSum& s) {
+  s.hh += (s.mid + (1LL << 28)) >> 29;
+  s.mid = 0;
+}
+// (re, im) += a b for complex a = (ax, ay), b = (bx, by).
+__device__ __forceinline__ void fx_cmac(FxSum& re, FxSum& im, int4 a, int4 b) {
+  const FxLimbs ax{a.x, a.y}, ay{a.z, a.w}, bx{b.x, b.y}, by{b.z, b.w};
+  fx_mac(re, ax, bx);
+  fx_mac(re, fx_neg(ay), by);
+  fx_mac(im, ax, by);
+  fx_mac(im, ay, bx);
+}
+__device__ __forceinline__ int fx_exp(cplx z) { return max(fx_exp(z.x), fx_exp(z.y)); }
+__device__ __forceinline__ int4 fx_limbs(cplx z, int E) {
+  const FxLimbs x = fx_limbs(z.x, fx_exp(z.x), E), y = fx_limbs(z.y, fx_exp(z.y), E);
+  return make_int4(x.h, x.l, y.h, y.l);
+}
 // acc + the sum of products with exponents that add up to E2, rounded; the sum is cleared.
 __device__ __forceinline__ double fx_flush(FxSum& s, int E2, double acc) {
   const long long t = s.hh + ((s.mid + (1LL << 28)) >> 29);

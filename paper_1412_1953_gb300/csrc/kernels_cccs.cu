@@ -16,16 +16,14 @@
 
 #include <mutex>
 
-#include "common.cuh"
+#include "fixed.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace {
 
 constexpr int TX = 32;        // tile width (one warp per row)
-constexpr int WY = 8;         // warps per block
-constexpr int SY = 4;         // rows per warp
-constexpr int TY = WY * SY;   // tile height
+constexpr int WY = 8;         // warps per block; a tile has SY rows per warp, SY = 1, 2 or 4
 
 template <class C>
 __device__ __forceinline__ C ldz(const C* __restrict__ a, int p, bool ok) {
@@ -40,15 +38,15 @@ __device__ __forceinline__ C residual_at(const StencilViewT<C>& s, const C* __re
                                        ldz(u, p - s.mx, j > 0), ldz(u, p + s.mx, j + 1 < s.my), __ldg(f + p));
 }
 
-// One 32 x 32 tile per block: each thread computes the residual at four nodes into a
+// One tile of 32 x 8 SY nodes per block: each thread computes the residual at SY nodes into a
 // padded shared tile; then, with the tile transposed through shared memory, one thread
 // per (row, state) sums P^x over the tile's 32 columns and one thread per (column,
-// state) sums P^y over its 32 rows.  Each residual costs 4 n_b FP64 FMAs of projection
-// work and no shuffle reductions.
-template <int NB, class C>
+// state) sums P^y over its rows, without shuffle reductions.
+template <int NB, int SY, class C>
 __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s, CCViewT<C> c, const C* __restrict__ u,
                                                               const C* __restrict__ f) {
   mgc_pdl_enter();
+  constexpr int TY = SY * WY;
   __shared__ C R[TY][TX + 1];
   const int lane = threadIdx.x;
   const int wy = threadIdx.y;
@@ -66,10 +64,10 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
   });
   __syncthreads();
   const int t = wy * TX + lane;
-  for (int w = t; w < 2 * TX * NB; w += TX * WY) {
-    if (w < TX * NB) {
+  for (int w = t; w < (TX + TY) * NB; w += TX * WY) {
+    if (w < TY * NB) {
       // P^x partial: row `row`, state m, over the tile's columns
-      const int m = w / TX, row = w % TX;
+      const int m = w / TY, row = w % TY;
       const int ncol = min(TX, s.mx - i0);
       const C* wp = c.wphi + (size_t)m * s.mx + i0;
       C acc = CT<C>::make(0.0, 0.0);
@@ -77,7 +75,7 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
       if (j0 + row < s.my) c.Px_part[((size_t)blockIdx.x * NB + m) * s.my + j0 + row] = acc;
     } else {
       // P^y partial: column `col`, state l, over the tile's rows
-      const int w2 = w - TX * NB;
+      const int w2 = w - TY * NB;
       const int l = w2 / TX, col = w2 % TX;
       const int nrow = min(TY, s.my - j0);
       const C* wv = c.wvphi + (size_t)l * s.my + j0;
@@ -85,6 +83,93 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
       for (int rr = 0; rr < nrow; ++rr) acc = cfma(__ldg(wv + rr), R[rr][col], acc);
       if (i0 + col < s.mx) c.Py_part[((size_t)blockIdx.y * NB + l) * s.mx + i0 + col] = acc;
     }
+  }
+}
+
+// The same in complex128 with the projections on the integer pipes (fixed.cuh): the tile's
+// residuals share one exponent, and so do each state's weighted values over the tile's columns
+// (rows).  A residual's 2 n_b complex products then cost 24 n_b integer multiply-adds, 96 n_b
+// cycles of a quarter of an SM, against 8 n_b FP64 instructions, 512 n_b cycles, and run beside
+// the FP64 instructions of the other blocks' residuals, which bound the kernel.  1023^2, n_b = 3:
+// 76.6 us with FP64 multiply-adds, 41.2 us so; 127^2: 19.2 us in tiles of 32 rows (16 blocks), 7.4
+// us in tiles of 8 (cold L2).
+template <int NB, int SY>
+__global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilView s, CCView c, const cplx* __restrict__ u,
+                                                                 const cplx* __restrict__ f) {
+  mgc_pdl_enter();
+  constexpr int TY = SY * WY;
+  __shared__ int4 R[TY][TX + 1];                         // limbs, or the values themselves
+  __shared__ int4 wl[NB][TX], wr[NB][TY];
+  __shared__ int ewl[NB], ewr[NB], eR, bad;
+  const int lane = threadIdx.x, wy = threadIdx.y, t = wy * TX + lane;
+  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, i = i0 + lane;
+  if (t == 0) eR = bad = 0;
+  __syncthreads();
+  cplx r[SY];
+  dispatch_kinds(s, i0, min(i0 + TX, s.mx), j0, min(j0 + TY, s.my), [&](auto kx, auto ky, auto ir, auto dg) {
+#pragma unroll
+    for (int q = 0; q < SY; ++q) {
+      const int j = j0 + q * WY + wy;
+      r[q] = (i < s.mx && j < s.my)
+                 ? residual_at<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
+                       s, u, f, i, j)
+                 : cmk(0.0, 0.0);
+    }
+  });
+  int e = 0;
+#pragma unroll
+  for (int q = 0; q < SY; ++q) e = max(e, fx_exp(r[q]));
+  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (lane == 0) atomicMax(&eR, e);
+  for (int p = wy; p < 2 * NB; p += WY) {                // a warp converts one state's values of the tile
+    const int m = p >> 1, n = p & 1 ? TY : TX, k = (p & 1 ? j0 : i0) + lane, len = p & 1 ? s.my : s.mx;
+    const cplx w = lane < n && k < len ? __ldg((p & 1 ? c.wvphi : c.wphi) + (size_t)m * len + k) : cmk(0.0, 0.0);
+    const int ew = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(w));
+    if (lane < n) (p & 1 ? wr[m] : wl[m])[lane] = fx_limbs(w, ew);
+    if (lane == 0) {
+      (p & 1 ? ewr : ewl)[m] = ew;
+      if (!fx_ok(ew)) bad = 1;
+    }
+  }
+  __syncthreads();
+  const int E = eR;
+  const bool ok = fx_ok(E) && !bad;
+#pragma unroll
+  for (int q = 0; q < SY; ++q) {
+    int4 v;
+    if (ok) v = fx_limbs(r[q], E);
+    else v = make_int4(__double2loint(r[q].x), __double2hiint(r[q].x), __double2loint(r[q].y), __double2hiint(r[q].y));
+    R[q * WY + wy][lane] = v;
+  }
+  __syncthreads();
+  for (int w = t; w < (TX + TY) * NB; w += TX * WY) {
+    const bool px = w < TY * NB;                         // P^x: a row's columns; P^y: a column's rows
+    const int w2 = px ? w : w - TY * NB, m = px ? w2 / TY : w2 / TX, at = px ? w2 % TY : w2 % TX;
+    const int n = px ? TX : TY;
+    cplx acc = cmk(0.0, 0.0);
+    if (ok) {
+      const int4* x = px ? &R[at][0] : &R[0][at];
+      const int4* y = px ? wl[m] : wr[m];
+      const int stride = px ? 1 : TX + 1;
+      FxSum re{0, 0}, im{0, 0};
+      for (int k0 = 0; k0 < n; k0 += FX_TERMS) {
+#pragma unroll
+        for (int k = 0; k < FX_TERMS; ++k) fx_cmac(re, im, y[k0 + k], x[(k0 + k) * stride]);
+        fx_carry(re);
+        fx_carry(im);
+      }
+      const int E2 = E + (px ? ewl[m] : ewr[m]);
+      acc = cmk(fx_flush(re, E2, 0.0), fx_flush(im, E2, 0.0));
+    } else {
+      const int cnt = px ? min(TX, s.mx - i0) : min(TY, s.my - j0);
+      const cplx* y = px ? c.wphi + (size_t)m * s.mx + i0 : c.wvphi + (size_t)m * s.my + j0;
+      for (int k = 0; k < cnt; ++k) {
+        const int4 v = px ? R[at][k] : R[k][at];
+        acc = cfma(__ldg(y + k), cmk(__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)), acc);
+      }
+    }
+    if (px && j0 + at < s.my) c.Px_part[((size_t)blockIdx.x * NB + m) * s.my + j0 + at] = acc;
+    if (!px && i0 + at < s.mx) c.Py_part[((size_t)blockIdx.y * NB + m) * s.mx + i0 + at] = acc;
   }
 }
 
@@ -356,15 +441,12 @@ k_channel_solve(CRSystem SA, CRSystem SB) {
   cluster_wait();
 }
 
-// u += sum_m phi_m(x) e^A_m(y) + sum_l e^B_l(x) vphi_l(y) (Eq. (30)).  A thread takes one
-// column i and cc_rows<C>() consecutive rows: phi_m(i) and e^B_l(i) stay in registers
+// u += sum_m phi_m(x) e^A_m(y) + sum_l e^B_l(x) vphi_l(y) (Eq. (30)), complex64.  A thread takes one
+// column i and CC_ROWS consecutive rows: phi_m(i) and e^B_l(i) stay in registers
 // across its rows (per node only the warp-uniform e^A_m(j), vphi_l(j) are loaded), and the
-// loads of its values of u are issued together, so a complex64 warp has 8 x 256 bytes of u
-// in flight (the complex64 pass is bound by how much of u is in flight).  Same sums in the
-// same order per node.  Rows per thread: 8 for complex64 (memory-bound), 4 for complex128
-// (FP64-bound, where the register cost of more rows would only lower occupancy).
-template <class C>
-__host__ __device__ constexpr int cc_rows() { return sizeof(C) == sizeof(float2) ? 8 : 4; }
+// loads of its values of u are issued together, so a warp has 8 x 256 bytes of u
+// in flight (the pass is bound by how much of u is in flight).
+constexpr int CC_ROWS = 8;
 
 template <int NB, class C>
 __global__ void __launch_bounds__(256) k_cccs_correct(int mx, int my, const C* __restrict__ phi,
@@ -372,7 +454,6 @@ __global__ void __launch_bounds__(256) k_cccs_correct(int mx, int my, const C* _
                                                       const C* __restrict__ eB, C* __restrict__ u) {
   mgc_pdl_enter();
   const int i = blockIdx.x * 32 + threadIdx.x;
-  constexpr int CC_ROWS = cc_rows<C>();
   const int j0 = (blockIdx.y * 8 + threadIdx.y) * CC_ROWS;
   if (i >= mx || j0 >= my) return;
   C a[NB], b[NB];
@@ -398,22 +479,135 @@ __global__ void __launch_bounds__(256) k_cccs_correct(int mx, int my, const C* _
   }
 }
 
+// The same in complex128 on the integer pipes (fixed.cuh).  A block of 32 columns by 8 RT rows
+// converts the values it needs of phi_m, e^B_l (columns) and e^A_m, vphi_l (rows), each with its
+// exponent over the block, and aligns the 2 n_b products to the largest of their exponents by
+// shifting e^A and vphi on conversion; a node then takes 24 n_b integer multiply-adds and four
+// FP64 instructions (two conversions, two additions) against 8 n_b FP64 instructions.
+// 1023^2, n_b = 3: 45.0 us with FP64 multiply-adds, 17.4 us so; 127^2: 9.6 and, with RT = 1, 4.5 us
+// (cold L2).
+template <int NB, int RT>
+__global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const cplx* __restrict__ phi,
+                                                         const cplx* __restrict__ vphi, const cplx* __restrict__ eA,
+                                                         const cplx* __restrict__ eB, cplx* __restrict__ u) {
+  mgc_pdl_enter();
+  constexpr int TYC = 8 * RT;
+  __shared__ int4 col[2 * NB][32], row[2 * NB][TYC];     // [phi | e^B], [e^A | vphi]
+  __shared__ int ec[2 * NB], er[2 * NB];
+  const int lane = threadIdx.x, wy = threadIdx.y;
+  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * TYC, i = i0 + lane, jt = j0 + wy * RT;
+  cplx v[RT];
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+    if (i < mx && jt + r < my) v[r] = u[(size_t)(jt + r) * mx + i];
+  auto value = [&](int p, int side) {                    // product p's factor at this lane's column (row)
+    const int m = p < NB ? p : p - NB, k = (side ? j0 : i0) + lane, len = side ? my : mx;
+    const cplx* a = p < NB ? (side ? eA : phi) : (side ? vphi : eB);
+    return k < len && (!side || lane < TYC) ? __ldg(a + (size_t)m * len + k) : cmk(0.0, 0.0);
+  };
+  for (int p = wy; p < 4 * NB; p += 8) {
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(value(p >> 1, p & 1)));
+    if (lane == 0) (p & 1 ? er : ec)[p >> 1] = e;
+  }
+  __syncthreads();
+  int E2 = 0;
+  bool ok = true;
+#pragma unroll
+  for (int p = 0; p < 2 * NB; ++p) {
+    E2 = max(E2, ec[p] + er[p]);
+    ok = ok && fx_ok(ec[p]) && fx_ok(er[p]);
+  }
+  if (!ok) {
+    if (i >= mx) return;
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+      const int j = jt + r;
+      if (j >= my) break;
+      cplx w = v[r];
+      for (int m = 0; m < NB; ++m) w = cfma(__ldg(phi + m * mx + i), __ldg(eA + m * my + j), w);
+      for (int l = 0; l < NB; ++l) w = cfma(__ldg(eB + l * mx + i), __ldg(vphi + l * my + j), w);
+      u[(size_t)j * mx + i] = w;
+    }
+    return;
+  }
+  for (int p = wy; p < 4 * NB; p += 8) {
+    const int q = p >> 1;
+    if (p & 1) {
+      if (lane < TYC) row[q][lane] = fx_limbs(value(q, 1), E2 - ec[q]);
+    } else {
+      col[q][lane] = fx_limbs(value(q, 0), ec[q]);
+    }
+  }
+  __syncthreads();
+  if (i >= mx) return;
+  int4 a[2 * NB];
+#pragma unroll
+  for (int p = 0; p < 2 * NB; ++p) a[p] = col[p][lane];
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+    if (jt + r >= my) break;
+    FxSum re{0, 0}, im{0, 0};
+#pragma unroll
+    for (int p = 0; p < 2 * NB; ++p) {
+      fx_cmac(re, im, a[p], row[p][wy * RT + r]);
+      if (p + 1 == FX_TERMS) {
+        fx_carry(re);
+        fx_carry(im);
+      }
+    }
+    u[(size_t)(jt + r) * mx + i] = cmk(fx_flush(re, E2, v[r].x), fx_flush(im, E2, v[r].y));
+  }
+}
+
+template <int NB, int SY, class C>
+cudaError_t rp_launch(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f, cudaStream_t st) {
+  dim3 g(cc_tiles_x(s.mx), cc_tiles_y(s.mx, s.my));
+  if constexpr (sizeof(C) == sizeof(cplx))
+    return mgc_launch(k_residual_project_fx<NB, SY>, g, dim3(TX, WY), 0, st, s, c, u, f);
+  else
+    return mgc_launch(k_residual_project<NB, SY, C>, g, dim3(TX, WY), 0, st, s, c, u, f);
+}
 template <int NB, class C>
 cudaError_t rp_launch(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f, cudaStream_t st) {
-  dim3 g(cc_tiles_x(s.mx), cc_tiles_y(s.my));
-  return mgc_launch(k_residual_project<NB, C>, g, dim3(TX, WY), 0, st, s, c, u, f);
+  switch (cc_tile_rows(s.mx, s.my)) {
+    case 1: return rp_launch<NB, 1, C>(s, c, u, f, st);
+    case 2: return rp_launch<NB, 2, C>(s, c, u, f, st);
+    default: return rp_launch<NB, 4, C>(s, c, u, f, st);
+  }
 }
 
 template <int NB, class C>
 cudaError_t corr_launch(const CCViewT<C>& c, C* u, cudaStream_t st) {
-  dim3 g((c.mx + 31) / 32, (c.my + 8 * cc_rows<C>() - 1) / (8 * cc_rows<C>()));
-  return mgc_launch(k_cccs_correct<NB, C>, g, dim3(32, 8), 0, st, c.mx, c.my, c.phi, c.vphi, c.eAc, c.eBc, u);
+  if constexpr (sizeof(C) == sizeof(cplx)) {
+    auto go = [&](auto kern, int rt) {
+      return mgc_launch(kern, dim3((c.mx + 31) / 32, (c.my + 8 * rt - 1) / (8 * rt)), dim3(32, 8), 0, st, c.mx, c.my,
+                        c.phi, c.vphi, c.eAc, c.eBc, u);
+    };
+    switch (cc_tile_rows(c.mx, c.my)) {
+      case 1: return go(k_cccs_correct_fx<NB, 1>, 1);
+      case 2: return go(k_cccs_correct_fx<NB, 2>, 2);
+      default: return go(k_cccs_correct_fx<NB, 4>, 4);
+    }
+  } else {
+    dim3 g((c.mx + 31) / 32, (c.my + 8 * CC_ROWS - 1) / (8 * CC_ROWS));
+    return mgc_launch(k_cccs_correct<NB, C>, g, dim3(32, 8), 0, st, c.mx, c.my, c.phi, c.vphi, c.eAc, c.eBc, u);
+  }
 }
 
 }  // namespace
 
 int cc_tiles_x(int mx) { return (mx + TX - 1) / TX; }
-int cc_tiles_y(int my) { return (my + TY - 1) / TY; }
+// Rows per warp of a tile: four, but on grids that then have fewer than two blocks per SM (up to
+// some 550 nodes an axis) two or one.
+int cc_tile_rows(int mx, int my) {
+  for (int sy = 4; sy > 1; sy /= 2)
+    if ((long long)cc_tiles_x(mx) * ((my + WY * sy - 1) / (WY * sy)) >= 2LL * mgc_sm_count()) return sy;
+  return 1;
+}
+int cc_tiles_y(int mx, int my) {
+  const int ty = WY * cc_tile_rows(mx, my);
+  return (my + ty - 1) / ty;
+}
 
 template <class C>
 cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f,
@@ -435,7 +629,7 @@ template <class C>
 cudaError_t launch_reduce_projections(const CCViewT<C>& c, cudaStream_t st) {
   int tot = c.nb * (c.mx + c.my);
   return mgc_launch(k_reduce_partials<C>, dim3((8 * tot + 255) / 256), dim3(256), 0, st, c.nb, c.mx, c.my,
-                    cc_tiles_x(c.mx), cc_tiles_y(c.my), c.Px_part, c.Py_part, c.Px, c.Py);
+                    cc_tiles_x(c.mx), cc_tiles_y(c.mx, c.my), c.Px_part, c.Py_part, c.Px, c.Py);
 }
 
 namespace {

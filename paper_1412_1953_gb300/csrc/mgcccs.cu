@@ -216,7 +216,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
     cc.mx = mx; cc.my = my; cc.nb = nb;
     cc.wphi = h->wphi; cc.wvphi = h->wvphi; cc.phi = h->phi; cc.vphi = h->vphi;
     cc.Px_part = cv.take<cplx>((size_t)cc_tiles_x(mx) * nb * my);
-    cc.Py_part = cv.take<cplx>((size_t)cc_tiles_y(my) * nb * mx);
+    cc.Py_part = cv.take<cplx>((size_t)cc_tiles_y(mx, my) * nb * mx);
     cc.Px = cv.take<cplx>((size_t)nb * my);
     cc.Py = cv.take<cplx>((size_t)nb * mx);
     cc.eA = cv.take<cplx>((size_t)nb * my);
@@ -235,7 +235,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
       c3.mx = mx; c3.my = my; c3.nb = nb;
       c3.wphi = h->wphi32; c3.wvphi = h->wvphi32; c3.phi = h->phi32; c3.vphi = h->vphi32;
       c3.Px_part = cv.take<float2>((size_t)cc_tiles_x(mx) * nb * my);
-      c3.Py_part = cv.take<float2>((size_t)cc_tiles_y(my) * nb * mx);
+      c3.Py_part = cv.take<float2>((size_t)cc_tiles_y(mx, my) * nb * mx);
       c3.Px = cc.Px; c3.Py = cc.Py; c3.eA = cc.eA; c3.eB = cc.eB;
       float2* eA32 = cv.take<float2>((size_t)nb * my);
       float2* eB32 = cv.take<float2>((size_t)nb * mx);

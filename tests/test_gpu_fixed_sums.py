@@ -116,3 +116,26 @@ def test_non_finite_entries_stay_where_they_belong():
     nanw[3] = np.nan
     h, w1 = _run(sv, V, 3, nanw)
     assert not np.any(np.isfinite(h)) and not np.any(np.isfinite(w1))
+
+
+# tiles of 8, 16 and 32 rows (by the number of blocks), ragged last tiles, sums that carry (more
+# than 8 products a node), sources scaled into the range of the FP64 instructions and back
+@pytest.mark.parametrize("nx,ny,levels,nb", [(16, 24, 3, 1), (64, 136, 4, 8), (416, 432, 4, 5), (608, 592, 5, 3)])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 60, 2.0 ** -460])
+def test_cccs_tiles(nx, ny, levels, nb, scale):
+    from oracle import mgcccs_oracle as O
+    L = 30.0 * nx / 128 if nx < 128 else 30.0
+    prob = inputs.temkin_poet(nx, L=L, R0=2 * L / 3, theta=math.pi / 6, E=0.5, seed=4, ny=ny)
+    so = O.Solver(O.params_from_problem(prob, levels=levels, n_b=nb), prob.v1, prob.v2, prob.v12)
+    sg = M.Solver(M.params_for(prob, levels=levels, n_b=nb), prob.v1, prob.v2, prob.v12)
+    g = np.random.default_rng(nx)
+    u = g.standard_normal(prob.f.shape) + 1j * g.standard_normal(prob.f.shape)
+    ref = so.cccs(u, prob.f)                           # linear in (u, f): a power of two scales exactly
+    ud = torch.as_tensor(u * scale).to("cuda")
+    sg.cccs(ud, torch.as_tensor(prob.f * scale).to("cuda"))
+    # the bound of the oracle parity tests at these sizes
+    assert np.abs(ud.cpu().numpy() / scale - ref).max() <= 1e-9 * np.abs(ref).max()
+    ud = torch.as_tensor(u).to("cuda")
+    ud[3, 5] = complex(np.nan, 0.0)
+    sg.cccs(ud, torch.as_tensor(prob.f).to("cuda"))
+    assert not bool(torch.isfinite(torch.view_as_real(ud)).any())    # a NaN reaches every node
