@@ -3,18 +3,21 @@
 // This part issues a warp's FP64 instruction over 64 cycles of its quarter of an SM, a 32 x 32 ->
 // 64-bit integer multiply-add over 4 and other integer operations over 2 (measured: 1.7, 32.6 and
 // 66 lane operations per clock and SM).  A complex FP64 multiply-add is 4 FP64 instructions, 256
-// cycles; below it is 12 integer multiply-adds and, for an operand not converted before, about 26
-// integer operations, 48 and 52 cycles that overlap.
+// cycles; below it is 12 integer multiply-adds and, for an operand not converted before, about 32
+// integer operations, 48 and 64 cycles that overlap.
 //
 // A double x = +-m 2^(e - 1075) (m the 53-bit significand, e the biased exponent) becomes, for a
-// common exponent E >= e, the integer +-((16 m) >> (E - e)) of at most 57 bits, that is x to within
-// 2^(E - 1079): four bits more than a double of the largest magnitude keeps, so an operand that
-// shares E with one up to 16 times as large is still exact to its last bit.  It is held as two
-// limbs h 2^29 + l of its sign (|h| < 2^28, |l| < 2^29).  In a product (h h' 2^58 + (h l' + l h')
-// 2^29 + l l') the last term, below 2^-56 of the largest product and of either sign, is dropped;
-// the sums of the others are exact in 64 bits for FX_TERMS complex terms, and are then rounded to
-// a double once.  Against FP64 multiply-adds, which round each partial sum to 2^-53 of itself, the
-// error stays below that of the same sum (measured at each kernel).
+// common exponent E >= e, the integer nearest to +-16 m 2^(e - E) of at most 57 bits, that is x to
+// within 2^(E - 1080): four bits more than a double of the largest magnitude keeps, so an operand
+// that shares E with one up to 16 times as large is still exact to its last bit.  It is held as two
+// limbs h 2^29 + l (|h| <= 2^28, |l| <= 2^28).  In a product (h h' 2^58 + (h l' + l h')
+// 2^29 + l l') the last term, below 2^-56 of the largest product, is dropped; the sums of the others
+// are exact in 64 bits for FX_TERMS complex terms, and are then rounded to a double once.  What is
+// dropped must have no mean, or a long sum that cancels keeps it, so low limbs lie about zero and
+// conversions round without a preference.  (With low limbs of the operands' signs and cut conversions, a dot product of
+// 1023^2 skewed, nearly cancelling terms was 1e-17 to 1e-16 |v| |w| off its 64-bit value, and 2e-19
+// with FP64 multiply-adds.)  Against these, which round each partial sum to 2^-53 of itself, the
+// error then stays within that of the same sum (measured at each kernel).
 //
 // Largest exponents outside FX_MIN..FX_MAX (nothing but zeros and subnormals, huge, infinite or
 // NaN operands) take the FP64 instructions; fx_ok tells.
@@ -31,14 +34,17 @@ struct FxLimbs {
   int h, l;
 };
 // x, of exponent e, for the common exponent E >= e: the significand left-justified in 64 bits, its 57 bits
-// from position 7 + E - e on, and the sign multiplied in (on the other integer pipe).
-__device__ __forceinline__ FxLimbs fx_limbs(double x, int e, int E) {
+// from position 7 + E - e on rounded, split at 2^29 with l in [-2^28, 2^28), and the sign multiplied in (on
+// the other integer pipe).  Ties, one in 2^d of the values that lose d bits, go away from zero, or
+// towards it with down = 1: long sums alternate it by lane, so that ties leave no mean either.
+__device__ __forceinline__ FxLimbs fx_limbs(double x, int e, int E, int down = 0) {
   const int hi = __double2hiint(x), s = (hi >> 31) | 1;
   const unsigned lo = (unsigned)__double2loint(x);
   const unsigned a1 = __funnelshift_l(lo, ((unsigned)hi & 0xfffffu) | 0x100000u, 11), a0 = lo << 11;
-  const int t = min(E + 7 - e, 63);
-  const unsigned long long m = (unsigned long long)a1 << 32 | a0;
-  const int h = (int)__funnelshift_rc(a1, 0u, t - 3), l = (int)((unsigned)(m >> t) & 0x1fffffffu);
+  unsigned long long r;                                  // with a bit more, for rounding; 0 for E - e > 57
+  asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(((unsigned long long)a1 << 32 | a0) - down), "r"(E + 6 - e));
+  r += (1u << 29) + 1;
+  const int h = (int)(r >> 30), l = (int)(((unsigned)r & 0x3fffffffu) >> 1) - (1 << 28);
   return FxLimbs{h * s, l * s};
 }
 __device__ __forceinline__ FxLimbs fx_neg(FxLimbs a) { return FxLimbs{-a.h, -a.l}; }
@@ -67,8 +73,8 @@ __device__ __forceinline__ void fx_cmac(FxSum& re, FxSum& im, int4 a, int4 b) {
   fx_mac(im, ay, bx);
 }
 __device__ __forceinline__ int fx_exp(cplx z) { return max(fx_exp(z.x), fx_exp(z.y)); }
-__device__ __forceinline__ int4 fx_limbs(cplx z, int E) {
-  const FxLimbs x = fx_limbs(z.x, fx_exp(z.x), E), y = fx_limbs(z.y, fx_exp(z.y), E);
+__device__ __forceinline__ int4 fx_limbs(cplx z, int E, int down = 0) {
+  const FxLimbs x = fx_limbs(z.x, fx_exp(z.x), E, down), y = fx_limbs(z.y, fx_exp(z.y), E, down);
   return make_int4(x.h, x.l, y.h, y.l);
 }
 // acc + the sum of products with exponents that add up to E2, rounded; the sum is cleared.

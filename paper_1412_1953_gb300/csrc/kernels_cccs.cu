@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
     const int m = p >> 1, n = p & 1 ? TY : TX, k = (p & 1 ? j0 : i0) + lane, len = p & 1 ? s.my : s.mx;
     const cplx w = lane < n && k < len ? __ldg((p & 1 ? c.wvphi : c.wphi) + (size_t)m * len + k) : cmk(0.0, 0.0);
     const int ew = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(w));
-    if (lane < n) (p & 1 ? wr[m] : wl[m])[lane] = fx_limbs(w, ew);
+    if (lane < n) (p & 1 ? wr[m] : wl[m])[lane] = fx_limbs(w, ew, lane & 1);
     if (lane == 0) {
       (p & 1 ? ewr : ewl)[m] = ew;
       if (!fx_ok(ew)) bad = 1;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
 #pragma unroll
   for (int q = 0; q < SY; ++q) {
     int4 v;
-    if (ok) v = fx_limbs(r[q], E);
+    if (ok) v = fx_limbs(r[q], E, (lane + q * WY + wy) & 1);
     else v = make_int4(__double2loint(r[q].x), __double2hiint(r[q].x), __double2loint(r[q].y), __double2hiint(r[q].y));
     R[q * WY + wy][lane] = v;
   }

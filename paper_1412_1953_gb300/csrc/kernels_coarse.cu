@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(32 * BP_KQ) k_bp_level_fx(int nr, int m, int s
     // alpha and gamma are subtracted
     const int r2 = t / (BP_KQ * BP_KC), k2 = t - r2 * BP_KQ * BP_KC;
     const cplx x = bs[r2][k2];
-    bl[r2][k2] = fx_limbs(r2 == 1 ? x : cneg(x), E2 - ef[r2]);
+    bl[r2][k2] = fx_limbs(r2 == 1 ? x : cneg(x), E2 - ef[r2], k2 & 1);
   }
   __syncthreads();
   cplx acc = cmk(0.0, 0.0);

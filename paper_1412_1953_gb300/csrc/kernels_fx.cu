@@ -356,7 +356,7 @@ cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t 
 
 // Limbs of one value on the host (as fx_limbs).
 static void host_limbs(double x, int E, int* h, int* l) {
-  const double m = std::floor(std::ldexp(std::fabs(x), 1079 - E));
+  const double m = std::floor(std::ldexp(std::fabs(x), 1079 - E) + 0.5);
   const long long M = (long long)m;
   const int sg = x < 0 ? -1 : 1;
   *h = sg * (int)(M >> 29);

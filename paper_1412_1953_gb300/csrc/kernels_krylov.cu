@@ -91,7 +91,8 @@ __device__ __forceinline__ void copy_wait() {
 // vector, of one tile after another) is fetched DS - 1 chunks ahead.  About 90 instructions a
 // product and the 16 warps that 128 registers allow bound it.  1023^2, 12 vectors (12 and 1
 // of 16.7 MB read): 88.0 us with FP64 multiply-adds, 63 with 64-bit shifts of masked keys in the
-// conversion, 58 before the FP64 share, 53.7 us now, 3.7 TB/s.
+// conversion, 58 before the FP64 share, 53.7 with it, 56.9 us with conversions that leave no mean
+// (fixed.cuh; ties alternate by lane: 4 us of a pair), 3.5 TB/s.
 constexpr int DG = 4, DU = 4, DS = 4;
 
 __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const cplx* __restrict__ V, long long ld,
@@ -179,8 +180,8 @@ __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const
     const cplx wl = v[DU - 1];
 #pragma unroll
     for (int u = 0; u < DU - 1; ++u) {
-      wx[u] = fx_limbs(v[u].x, ex[u], Ew);
-      wy[u] = fx_limbs(v[u].y, ey[u], Ew);
+      wx[u] = fx_limbs(v[u].x, ex[u], Ew, lane & 1);
+      wy[u] = fx_limbs(v[u].y, ey[u], Ew, lane & 1);
     }
 #pragma unroll
     for (int i = 0; i < DG; ++i) {
@@ -193,7 +194,8 @@ __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const
       if (fx_ok(Ew) && fx_ok(E[i])) {
 #pragma unroll
         for (int u = 0; u < DU - 1; ++u) {
-          const FxLimbs ax = fx_limbs(v[u].x, ex[u], E[i]), ay = fx_limbs(v[u].y, ey[u], E[i]);
+          const FxLimbs ax = fx_limbs(v[u].x, ex[u], E[i], lane & 1);
+          const FxLimbs ay = fx_limbs(v[u].y, ey[u], E[i], lane & 1);
           fx_mac(re[i], ax, wx[u]);
           fx_mac(re[i], ay, wy[u]);
           fx_mac(im[i], ax, wy[u]);
@@ -244,7 +246,7 @@ static_assert(MULTIDOT_SMEM >= 2 * DG * NT * (int)sizeof(double), "the block sum
 // with its own exponent; a warp's sums over the vectors share the exponent of the largest product
 // met so far (at first that of the largest coefficient and the first vector).  A warp takes
 // UU x 32 points at a time and fetches the chunks (w, then each vector) ahead, as above.
-// 1023^2, 11 vectors: 90.1 us with FP64 multiply-adds, 49.5 us now (UU = 4; 58 with UU = 2, which
+// 1023^2, 11 vectors: 90.1 us with FP64 multiply-adds, 50.0 us now (UU = 4; 58 with UU = 2, which
 // is the faster at 255^2: 7.6 against 11.4 us, few tiles a warp), 4.4 TB/s.
 constexpr int UF = 16;                                 // chunks in flight x points a lane
 
