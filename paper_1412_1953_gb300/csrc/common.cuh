@@ -556,6 +556,7 @@ struct CRSystem {
   // row eliminated (i < R - 1) B^{-1} A, B^{-1} C, B^{-1} of its level.  sinv: the dense inverse of
   // the separators' system, [ns nb][ns nb].
   int p, ns;
+  int shared_gpu;          // 1: other solves run beside this one (cr_pack_in_smem)
   cplx* pack;
   cplx* sinv;
   // setup only: the factors of the parallel reduction of the separators, [levels][ns][2 nb^2], then
@@ -572,10 +573,14 @@ __host__ __device__ constexpr int cr_log_rows(int m) {
 __host__ __device__ constexpr size_t cr_pack_entries(int R, int p, int nb) {
   return (size_t)nb * nb * (5 * (size_t)(R - 1) + p);
 }
-// Whether a CTA's factors fit in shared memory beside its rows.
-__host__ __device__ constexpr bool cr_pack_in_smem(int m, int nb) {
+// Whether a CTA copies its factors to shared memory beside its rows: where they fit, and where the
+// solve has the GPU to itself.  Then the copy takes 2 us (127 rows) to 4 us (1023) off the
+// preconditioner (226.4 -> 222.5 us at 1024^2).  In a batch other solves fill that latency, and what
+// the shared memory takes from the kernels beside it costs more: 64 solves on 256^2 to 1024^2 grids
+// make 125.8 solves/s with copies, 129.7 from L2.
+__host__ __device__ constexpr bool cr_pack_in_smem(int m, int nb, bool shared_gpu) {
   const int p = cr_log_rows(m);
-  return 16 * (cr_pack_entries(1 << p, p, nb) + ((size_t)nb << p)) <= 200 * 1024;
+  return !shared_gpu && 16 * (cr_pack_entries(1 << p, p, nb) + ((size_t)nb << p)) <= 200 * 1024;
 }
 int cc_tiles_x(int mx);
 int cc_tile_rows(int mx, int my);   // rows per warp of a CCCS tile (8 warps): 1, 2 or 4

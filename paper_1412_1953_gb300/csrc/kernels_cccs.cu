@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(256) k_reduce_partials(int nb, int mx, int my,
 // What bounds it is the latency of ~2 p small steps: a warp-wide FP64 instruction occupies its
 // quarter of an SM for 64 cycles however few lanes need it, so LP lanes share the products of an
 // item (a row's component), and the factors are copied to shared memory while the preceding
-// kernel drains (large systems read them from L2).  Against parallel cyclic reduction over the
-// cluster (every row updated at each of log2 m levels, a cluster barrier between them) with the
+// kernel drains (large systems, and batches, read them from L2: cr_pack_in_smem).  Against
+// parallel cyclic reduction over the cluster (every row updated at each of log2 m levels, a cluster barrier between them) with the
 // coupling coefficients in a kernel of their own: 26.0 against 28.0 + 6.7 us for 1023 rows and
 // n_b = 3, 16.2 against 18.1 + 4.1 us for 127 rows (cold L2); for 2047 rows and n_b = 6, where
 // that took 11 m row updates, a step of the mixed-precision solve is 73 us shorter (50.3 to
@@ -379,7 +379,7 @@ k_channel_solve(CRSystem SA, CRSystem SB) {
   cplx* const X = cr_sh;
   const size_t len = cr_pack_entries(R, p, NB);
   const cplx* F = S.pack + rank * len;
-  const bool in_smem = cr_pack_in_smem(m, NB);
+  const bool in_smem = cr_pack_in_smem(m, NB, S.shared_gpu);
   if (k0 < m) {
     // the factors were written at setup: fetch them ahead of the wait for the projections
     if (in_smem) {
@@ -696,9 +696,10 @@ cudaError_t launch_reduce_projections(const CCViewT<C>& c, cudaStream_t st) {
 }
 
 namespace {
-size_t channel_smem(int m, int nb) {
+size_t channel_smem(int m, int nb, bool shared_gpu) {
   const int p = cr_log_rows(m);
-  return sizeof(cplx) * (((size_t)nb << p) + (cr_pack_in_smem(m, nb) ? cr_pack_entries(1 << p, p, nb) : 0));
+  return sizeof(cplx) *
+         (((size_t)nb << p) + (cr_pack_in_smem(m, nb, shared_gpu) ? cr_pack_entries(1 << p, p, nb) : 0));
 }
 }  // namespace
 
@@ -710,7 +711,7 @@ cudaError_t channel_solve_prepare(int nb, int mA, int mB) {
   static std::mutex mu;
   static int granted[MGC_MAX_NB + 1] = {0};
   if (nb < 1 || nb > MGC_MAX_NB) return cudaErrorInvalidValue;
-  const size_t a = channel_smem(mA, nb), b = channel_smem(mB, nb);
+  const size_t a = channel_smem(mA, nb, false), b = channel_smem(mB, nb, false);
   const int smem = (int)(a > b ? a : b);
   std::lock_guard<std::mutex> lock(mu);
   if (granted[nb] > 0 && smem <= granted[nb]) return cudaSuccess;
@@ -731,7 +732,8 @@ cudaError_t channel_solve_prepare(int nb, int mA, int mB) {
 }
 
 cudaError_t launch_channel_solve(const CRSystem& A, const CRSystem& B, cudaStream_t st) {
-  const size_t a = channel_smem(A.m, A.nb), b = channel_smem(B.m, B.nb), smem = a > b ? a : b;
+  const size_t a = channel_smem(A.m, A.nb, A.shared_gpu), b = channel_smem(B.m, B.nb, B.shared_gpu);
+  const size_t smem = a > b ? a : b;
   switch (A.nb) {
 #define MGC_SOLVE(K) \
   case K: return mgc_launch(k_channel_solve<K>, dim3(2 * CR_CLUSTER), dim3(CR_THREADS), smem, st, A, B);

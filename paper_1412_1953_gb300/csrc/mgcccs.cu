@@ -1882,7 +1882,10 @@ int mgcccs_batch_create(mgcccs_batch_t* out, mgcccs_t* handles, int count, mgccc
   b->u = us;
   b->st = reinterpret_cast<cudaStream_t>(stream);
   b->exec = nullptr;
+  // the handles' own solves, before and after, have the GPU to themselves
+  for (mgcccs_handle* h : hs) h->crA.shared_gpu = h->crB.shared_gpu = count > 1;
   int rc = instantiate_solves(hs.data(), us.data(), fs.data(), count, &b->exec);
+  for (mgcccs_handle* h : hs) h->crA.shared_gpu = h->crB.shared_gpu = 0;
   if (rc) {
     delete b;
     return rc;
