@@ -305,7 +305,7 @@ int mgcccs_get_bound_states(mgcccs_t h, mgcccs_c128* lambda, mgcccs_c128* phi,
 int mgcccs_norm2_noalloc(const mgcccs_c128* v, size_t n, double* norm2, void* stream);
 
 /* ---- FP64 throughput probe (a measurement utility; the paper has no counterpart) ----
- * The complex128 kernels are bound by the FP64 pipe.  mgcccs_fp64_probe launches
+ * The rate of FP64 instructions, by which the one-step complex128 kernels are bound.  It launches
  * `blocks` blocks of 256 threads on `stream` (cudaStream_t as void*; NULL = legacy
  * default stream), each thread running MGCCCS_PROBE_CHAINS independent recurrences
  * a <- fma(a, m, b) for `iters` rounds, and writes one sum per block to the device
@@ -327,9 +327,10 @@ int mgcccs_fp64_probe(int blocks, int iters, double m, double b, double* out, vo
  *
  * V: device, k vectors of (nx-1)*(ny-1) values, vector i at V + i*ld (ld >= (nx-1)*(ny-1));
  * w: device, (nx-1)*(ny-1) values (gs_update overwrites it); out, coef: device, k values.
- * A vector V_i that is w itself (same address) gives out[i] = |w|^2.  The sums are FP64
- * in a fixed order (per-block partials, then one block), so repeated calls give identical
- * results.  mgcccs_gs_dots needs a handle set up with krylov_restart >= 1 and
+ * A vector V_i that is w itself (same address) gives out[i] = |w|^2.  Products are summed as
+ * integers of 57 bits on a common exponent, or with FP64 instructions out of their range, to the
+ * accuracy of FP64 sums, in a fixed order (per-block partials, then one block), so repeated calls
+ * give identical results.  mgcccs_gs_dots needs a handle set up with krylov_restart >= 1 and
  * k <= krylov_restart + 1 (it uses the handle's partial-sum buffer); mgcccs_gs_update
  * takes 1 <= k <= 61.  Async.  Errors: EINVAL (null pointer, k or ld out of range), ECUDA.
  */
