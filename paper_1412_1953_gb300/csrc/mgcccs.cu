@@ -1824,6 +1824,16 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
 
 int mgcccs_eig_fallbacks(mgcccs_t h) { return h ? h->eig_fallbacks : -1; }
 
+int mgcccs_integer_passes(mgcccs_t h, unsigned* levels, int* coarsest) {
+  if (!h) return MGCCCS_EINVAL;
+  if (levels) {
+    *levels = 0;
+    for (int l = 0; l < h->L; ++l) *levels |= h->lv[l].fx.on ? 1u << l : 0u;
+  }
+  if (coarsest) *coarsest = h->coarse_bp && h->bp_exp;
+  return MGCCCS_OK;
+}
+
 int mgcccs_set_solve_driver(mgcccs_t h, int driver) {
   if (!h || (driver != MGCCCS_DRIVER_GRAPH && driver != MGCCCS_DRIVER_HOST)) return MGCCCS_EINVAL;
   h->driver = driver;
