@@ -38,17 +38,27 @@ __global__ void __launch_bounds__(256) k_exponents(long long n, const cplx* __re
   }
 }
 
-// *most = the bits of the largest sum over a node of |re| + |im| of its five coefficients.
+// most[0] = the bits of the largest sum over a node of |re| + |im| of its five coefficients, most[1] of
+// that sum times |re| + |im| of the node's omega/D.
 __global__ void __launch_bounds__(256) k_row_bound(StencilView s, unsigned long long* __restrict__ most) {
   const long long n = (long long)s.mx * s.my;
-  double m = 0.0;
+  double m = 0.0, g = 0.0;
   for (long long p = blockIdx.x * 256LL + threadIdx.x; p < n; p += (long long)gridDim.x * 256) {
     const int i = (int)(p % s.mx), j = (int)(p / s.mx);
-    m = fmax(m, cabs1(s.D[p]) + cabs1(s.west_x[i]) + cabs1(s.east_x[i]) + cabs1(s.west_y[j]) + cabs1(s.east_y[j]));
+    const double row =
+        cabs1(s.D[p]) + cabs1(s.west_x[i]) + cabs1(s.east_x[i]) + cabs1(s.west_y[j]) + cabs1(s.east_y[j]);
+    m = fmax(m, row);
+    g = fmax(g, cabs1(s.Dinv[p]) * row);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(most, (unsigned long long)__double_as_longlong(m));
+  for (int o = 16; o > 0; o >>= 1) {
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(most, (unsigned long long)__double_as_longlong(m));
+    atomicMax(most + 1, (unsigned long long)__double_as_longlong(g));
+  }
 }
 
 __global__ void __launch_bounds__(256) k_split(long long n, const cplx* __restrict__ a, int E, int4* __restrict__ out) {
@@ -337,10 +347,10 @@ unsigned stride_blocks(long long n) {
 
 size_t level_fx_entries(int mx, int my) { return 2 * ((size_t)mx * my + mx + my); }
 
-// A level's exponents and bound into lim (six device ints, 8-byte aligned: largest and smallest
-// exponent of west, east, D; of omega/D; the bits of the bound).
+// A level's exponents and bounds into lim (FX_LIMITS device ints, 8-byte aligned: largest and smallest
+// exponent of west, east, D; of omega/D; the bits of the two bounds).
 cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t st) {
-  static const int init[6] = {0, 4096, 0, 4096, 0, 0};
+  static const int init[FX_LIMITS] = {0, 4096, 0, 4096, 0, 0, 0, 0};
   cudaError_t e = cudaMemcpyAsync(lim, init, sizeof(init), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
   const long long n = (long long)s.mx * s.my;
@@ -371,14 +381,15 @@ cudaError_t level_fx(const StencilView& s, const int* lim, int4* buf, StencilFx*
   x.ec = lim[0];
   x.ed = lim[2];
   const auto ok = [](int e) { return e >= FX_MIN && e <= FX_MAX; };
-  double bound;
-  std::memcpy(&bound, lim + 4, sizeof(bound));
+  double row, gain;
+  std::memcpy(&row, lim + 4, sizeof(row));
+  std::memcpy(&gain, lim + 6, sizeof(gain));
   x.kd = 2100 - x.ec - x.ed;
   // the exponents within their spread; every sum (H - E)u below 2^(ec - 1020) max |u|, which keeps
   // it in 64 bits; the update's scaling within fx_scaled's range, and f's unit no coarser than
-  // (omega/D) f needs (ec + ed >= 2042)
+  // (omega/D) f needs (ec + ed >= 2042); and the new value of k_pj_fx in 64 bits (FX_GAIN)
   x.on = lim[0] - lim[1] <= FX_SPREAD && lim[2] - lim[3] <= FX_SPREAD && ok(x.ec) && ok(x.ed) &&
-         std::isfinite(bound) && bound <= std::ldexp(1.0, x.ec - 1020) && x.kd >= 30 && x.kd <= 58;
+         std::isfinite(row) && row <= std::ldexp(1.0, x.ec - 1020) && x.kd >= 30 && x.kd <= 58 && gain <= FX_GAIN;
   if (x.on) {
     const long long n = (long long)s.mx * s.my;
     int4* D = buf;

@@ -288,7 +288,7 @@ void layout(mgcccs_handle* h, Carver& cv) {
   }
   h->norm_part = cv.take<double>(h->norm_nparts);
   h->norm_out = cv.take<double>(4);
-  h->fxlim = cv.take<int>(6 * MGC_MAX_LEVELS);
+  h->fxlim = cv.take<int>(FX_LIMITS * MGC_MAX_LEVELS);
   h->status = cv.take<int>(8);   // error bits, three flags, then the dense inverse's check (below)
   h->hu = cv.take<cplx>((size_t)mx * my);
   h->hf = cv.take<cplx>((size_t)mx * my);
@@ -428,19 +428,19 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
     }
   }
   // the levels' operators as limbs, where their exponents allow it
-  int lim[6 * MGC_MAX_LEVELS];
+  int lim[FX_LIMITS * MGC_MAX_LEVELS];
   for (int l = 0; l < h->L; ++l) {
     if (!h->lv[l].fxbuf) continue;
-    MGC_LAUNCH(launch_level_exponents(h->lv[l].sv, h->fxlim + 6 * l, st));
+    MGC_LAUNCH(launch_level_exponents(h->lv[l].sv, h->fxlim + FX_LIMITS * l, st));
     h->launches += 6;
   }
   if (!h->mixed) {
-    MGC_CUDA(cudaMemcpyAsync(lim, h->fxlim, sizeof(int) * 6 * h->L, cudaMemcpyDeviceToHost, st));
+    MGC_CUDA(cudaMemcpyAsync(lim, h->fxlim, sizeof(int) * FX_LIMITS * h->L, cudaMemcpyDeviceToHost, st));
     MGC_CUDA(cudaStreamSynchronize(st));
   }
   for (int l = 0; l < h->L; ++l) {
     LevelBufs& b = h->lv[l];
-    if (b.fxbuf) MGC_CUDA(level_fx(b.sv, lim + 6 * l, b.fxbuf, &b.fx, st));
+    if (b.fxbuf) MGC_CUDA(level_fx(b.sv, lim + FX_LIMITS * l, b.fxbuf, &b.fx, st));
     else b.fx = StencilFx{};
     b.fx.s = b.sv;
     if (b.fx.on) h->launches += 6;

@@ -21,6 +21,13 @@ struct StencilFx {
   const int4 *D, *Di;                      // [my*mx]
 };
 constexpr int FX_SPREAD = 6;
+// Most a node's |omega/D| times its row's sum of coefficients (|re| + |im| of each) may be.  In the
+// units of k_pj_fx v and (omega/D) f stay below 2^58, so (omega/D)(H - E) v stays below 2^58 times this
+// gain and the new value below (2 + gain) 2^58, 2^62.2; beyond 30 it would wrap.  An energy close to
+// the diagonal's 2/h^2 makes D small there: 2.7 at E = 0.5 on 256^2 cells of [0, 30]^2, 14 at E = 130, 47 at
+// E = 135.  A level beyond it keeps to FP64.
+constexpr double FX_GAIN = 16.0;
+constexpr int FX_LIMITS = 8;               // ints of launch_level_exponents
 // Levels of at least this many nodes run on the integer pipes: smaller ones are bound by a launch's
 // latency, and the exponent's reduction and barriers lengthen that.  The preconditioner by grid size
 // n, integer passes (three blocks an SM) on no level / on every level / from 60000 nodes (us): 128: 60.8 / 67.3 / 60.8,
@@ -167,7 +174,7 @@ __device__ __forceinline__ void block_exponent(int e, int* es) {
 
 // kernels_fx.cu
 size_t level_fx_entries(int mx, int my);                                  // int4 entries of a level's limbs
-cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t st);   // six device ints
+cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t st);   // FX_LIMITS device ints
 cudaError_t level_fx(const StencilView& s, const int* lim, int4* buf, StencilFx* out, cudaStream_t st);
 cudaError_t launch_zrr_fx(const StencilFx& x, const cplx* f, cplx* u, cplx* fc, bool zero, cudaStream_t st);
 cudaError_t launch_pj_fx(const StencilFx& x, const cplx* ec, const cplx* u, cplx* o, const cplx* f, cudaStream_t st);

@@ -28,6 +28,27 @@ def _solver(prob, levels, spike=0.0, **kw):
     return M.Solver(M.params_for(prob, levels=levels, **{"n_b": 0, **kw}), prob.v1, prob.v2, v12)
 
 
+def _composed(sv, levels, f, u, nu1, nu2):
+    """V(nu1, nu2) from u by the one-step calls, which use FP64 instructions."""
+    zeros = lambda l: torch.zeros(sv.level_size(l), dtype=torch.complex128, device="cuda")
+    fs, us = [f.reshape(-1)], []
+    for l in range(levels - 1):
+        v = u.reshape(-1).clone() if l == 0 else zeros(l)
+        sv.smooth(l, v, fs[l], nu1)
+        r, fc = zeros(l), zeros(l + 1)
+        sv.level_residual(l, v, fs[l], r)
+        sv.restrict(l, r, fc)
+        us.append(v)
+        fs.append(fc)
+    e = zeros(levels - 1)
+    sv.coarse_solve(fs[-1], e)
+    for l in reversed(range(levels - 1)):
+        sv.prolong_add(l, e, us[l])
+        sv.smooth(l, us[l], fs[l], nu2)
+        e = us[l]
+    return e.reshape(u.shape)
+
+
 # 60000 nodes and more: 255 x 255, 511 x 511 with 255 x 255, 591 x 431 with 295 x 215; a coarsest level multiplies
 # nothing itself; one large potential value spreads the fine diagonal
 @pytest.mark.parametrize("nx,ny,levels,spike,on", [(240, 240, 4, 0.0, []), (256, 256, 4, 0.0, [0]),
@@ -36,4 +57,24 @@ def _solver(prob, levels, spike=0.0, **kw):
 def test_levels_on_the_integer_pipes(nx, ny, levels, spike, on):
     sv = _solver(_problem(nx, ny), levels, spike)
     assert sv.integer_passes() == (on, False)
+    sv.close()
+
+
+# An energy near the diagonal's 2/h^2, or a large omega, makes |omega/D| times a row's coefficients
+# large: 14, 47, 72 and 32, where the integers of the prolongation and sweep hold an update of up to 30.
+# The two forms agree to 1e-13 at 2.7 (test_gpu_fixed_stencils.py); a sweep on either level amplifies a
+# difference by this factor, 72/2.7 squared: 1e-10.
+@pytest.mark.parametrize("E,omega,on", [(130.0, 2 / 3, True), (135.0, 2 / 3, False), (140.0, 2 / 3, False),
+                                        (0.5, 8.0, False)])
+def test_updates_beyond_64_bits(E, omega, on):
+    prob = _problem(256, 256, E=E)
+    sv = _solver(prob, 3, omega=omega, nu1=0, nu2=1)
+    f = torch.full(prob.f.shape, 1e-3, dtype=torch.complex128, device="cuda")
+    sign = torch.as_tensor(1.0 - 2.0 * (np.indices(prob.f.shape).sum(0) % 2)).to("cuda")
+    for u0 in (torch.full_like(f, 1.9), 1.9 * sign.to(f.dtype)):
+        u = u0.clone()
+        sv.vcycle(u, f)
+        ref = _composed(sv, 3, f, u0, 0, 1)
+        assert float((u - ref).abs().max() / ref.abs().max()) <= 1e-10
+    assert (0 in sv.integer_passes()[0]) == on
     sv.close()
