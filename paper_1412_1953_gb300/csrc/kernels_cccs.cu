@@ -131,13 +131,13 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
     __syncthreads();
     const int i1 = min(i0 + TX, s.mx), j1 = min(j0 + TY, s.my);
     if (oku) {
-      const double sc = -fx_pow2(eu + x.ec - 2101);
+      const double sc = -fx_pow2(eu + x.ec - 2104);
       fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
 #pragma unroll
         for (int q = 0; q < SY; ++q) {
           const int row = q * WY + wy, j = j0 + row;
           if (i >= s.mx || j >= s.my) continue;
-          const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value>(
+          const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(
               x, i, j, (size_t)j * s.mx + i, T + (row + 1) * PW + lane + 1, PW);
           r[q] = cmk(fma(sc, (double)h.x, r[q].x), fma(sc, (double)h.y, r[q].y));
         }

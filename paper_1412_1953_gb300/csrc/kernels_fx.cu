@@ -326,8 +326,8 @@ __global__ void __launch_bounds__(BX * PY) k_apply_fx(StencilFx x, const cplx* _
   const int i1 = min(i0 + BX, s.mx), j1 = min(j0 + PY, s.my);
   if (ok) {
     fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
-      const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value>(x, i, j, p, c, PW);
-      const double sc = fx_pow2(eu + x.ec - 2101);
+      const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(x, i, j, p, c, PW);
+      const double sc = fx_pow2(eu + x.ec - 2104);
       y[p] = cmk(sc * (double)h.x, sc * (double)h.y);
     });
   } else {

@@ -9,8 +9,10 @@
 #include "fixed.cuh"
 
 // A level's operator as limbs.  `on` when all of west, east and D lie within FX_SPREAD powers of
-// two of the largest, and all of omega/D likewise, so that one exponent costs none of them
-// precision a double would keep (level_fx in kernels_fx.cu); otherwise the level keeps to FP64.
+// two of the largest (each by the larger of its parts), and all of omega/D likewise: limbs keep 57
+// bits of the largest, so within four powers of two that larger part keeps the 53 bits of its double
+// (level_fx in kernels_fx.cu); otherwise the level keeps to FP64.  Square cells spread over three, cells
+// of twice the height over four; at five and six a coefficient was up to 2 and 4 units of 2^-53 off.
 struct StencilFx {
   StencilView s;
   int on;
@@ -20,7 +22,7 @@ struct StencilFx {
   const int4 *wx, *ex, *wy, *ey;           // per-node neighbour coefficients
   const int4 *D, *Di;                      // [my*mx]
 };
-constexpr int FX_SPREAD = 6;
+constexpr int FX_SPREAD = 4;
 // Most a node's |omega/D| times its row's sum of coefficients (|re| + |im| of each) may be.  In the
 // units of k_pj_fx v and (omega/D) f stay below 2^58, so (omega/D)(H - E) v stays below 2^58 times this
 // gain and the new value below (2 + gain) 2^58, 2^62.2; beyond 30 it would wrap.  An energy close to
@@ -96,8 +98,9 @@ __device__ __forceinline__ void fx_kinds(const StencilView& s, int i0, int i1, i
 
 // (H - E) u at node p = (i, j), whose value in units of 2^qu is t[0] of a tile with row pitch
 // `pitch` (values below 2^58, so that a sum of two still splits into 31-bit limbs), in units of
-// 2^(qu + ec - 1021), below 2^59.
-template <int KX, int KY, int RD>
+// 2^(qu + ec - 1021 - XB), below 2^(59 + XB).  XB = 3 where a double is made of it: a coefficient of
+// the spread's end times a value of 2^57 is then rounded to less than a double's last place.
+template <int KX, int KY, int RD, int XB = 0>
 __device__ __forceinline__ longlong2 fx_operator(const StencilFx& x, int i, int j, size_t p, const longlong2* t,
                                                  int pitch) {
   FxSum re{0, 0}, im{0, 0};
@@ -122,7 +125,8 @@ __device__ __forceinline__ longlong2 fx_operator(const StencilFx& x, int i, int 
     }
     fx_cmac(re, im, __ldg(x.D + p), t[0]);
   }
-  return make_longlong2(fx_total(re), fx_total(im));
+  if constexpr (XB > 0) return make_longlong2(fx_scaled(re, 58 - XB), fx_scaled(im, 58 - XB));
+  else return make_longlong2(fx_total(re), fx_total(im));
 }
 
 // A thread's share of a tile of ROWS x (32 + XC) complex values around the 32 columns i0..i0+31 and

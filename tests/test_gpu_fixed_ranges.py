@@ -78,3 +78,23 @@ def test_updates_beyond_64_bits(E, omega, on):
         assert float((u - ref).abs().max() / ref.abs().max()) <= 1e-10
     assert (0 in sv.integer_passes()[0]) == on
     sv.close()
+
+
+# Cells of aspect 1 to 4: the coefficients spread over 3 to 6 powers of two, and 57 bits of the largest
+# keep a double's 53 of all within four.  A unit vector's image is a column of coefficients: to half a
+# unit of 2^-53 of its modulus in either part (the larger one exact), exact in the real box.
+@pytest.mark.parametrize("nx,ny,on", [(256, 256, True), (512, 256, True), (768, 256, False), (1024, 256, False)])
+def test_coefficients_keep_their_bits(nx, ny, on):
+    prob = _problem(nx, ny)
+    sv = _solver(prob, 5)
+    x = torch.zeros(prob.f.shape, dtype=torch.complex128, device="cuda")
+    x[1::4, 1::4] = 1.0                              # columns that do not meet
+    y, r = torch.empty_like(x), torch.empty_like(x)
+    sv.matvec(x, y)
+    sv.level_residual(0, x.reshape(-1), torch.zeros(x.numel(), dtype=x.dtype, device="cuda"), r.reshape(-1))
+    d = torch.view_as_real(y + r).abs().amax(-1)
+    assert bool((d <= 2.0 ** -54 * r.abs()).all())
+    box = (slice(0, ny * 2 // 3 - 2), slice(0, nx * 2 // 3 - 2))
+    assert bool((y[box] == -r[box]).all())
+    assert (0 in sv.integer_passes()[0]) == on
+    sv.close()
