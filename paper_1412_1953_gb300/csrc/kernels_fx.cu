@@ -13,6 +13,8 @@ namespace {
 constexpr int BX = 32;
 
 __device__ __forceinline__ longlong2 ll2(long long a) { return make_longlong2(a, a); }
+// a quarter, to the nearest, ties to even
+__device__ __forceinline__ long long fx_quarter(long long a) { return (a + 1 + (a >> 2 & 1)) >> 2; }
 
 // f - (H - E) u with FP64 instructions from a tile of values
 template <class F>
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
       if (a >= 0 && b >= 0 && a < s.mx && b < s.my) {
         const longlong2* g = Ex + ((b >> 1) - (j0 / 2 - 1)) * PW + c + 1;
         const longlong2 y = fx_add(g[0], g[b & 1 ? 0 : -PW]);          // four times P e
-        w = fx_add(fx_int(z, qu), make_longlong2(y.x >> 2, y.y >> 2));
+        w = fx_add(fx_int(z, qu), make_longlong2(fx_quarter(y.x), fx_quarter(y.y)));
       }
       T[r * PW + c + 1] = w;
     });
