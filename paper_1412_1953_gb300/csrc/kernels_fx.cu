@@ -366,13 +366,12 @@ cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t 
   return cudaGetLastError();
 }
 
-// Limbs of one value on the host (as fx_limbs).
+// Limbs of one value on the host, those of fx_limbs (down = 0).
 static void host_limbs(double x, int E, int* h, int* l) {
-  const double m = std::floor(std::ldexp(std::fabs(x), 1079 - E) + 0.5);
-  const long long M = (long long)m;
+  const long long m = (long long)std::floor(std::ldexp(std::fabs(x), 1079 - E) + 0.5);
   const int sg = x < 0 ? -1 : 1;
-  *h = sg * (int)(M >> 29);
-  *l = sg * (int)(M & 0x1fffffff);
+  *h = sg * (int)((m + (1LL << 28)) >> 29);
+  *l = sg * ((int)(m & 0x1fffffff) - ((m >> 28 & 1) << 29));
 }
 
 // The level's operator as limbs in buf (level_fx_entries), if its exponents (lim, on the host)

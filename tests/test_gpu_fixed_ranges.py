@@ -117,3 +117,31 @@ def test_cycle_is_odd(nx, ny, levels, nu1, nu2):
     assert bool((u == -v).all()) and bool((z == -zm).all())
     assert 0 in sv.integer_passes()[0]
     sv.close()
+
+
+def test_inner_coefficients_are_split_about_zero():
+    """A sum drops the products of low limbs, of at most 2^28 each: a quarter of the unit of the sum.  The
+    box is such that the inner coefficient's low limb is near a multiple of 2^29, the constant field such that twice
+    its value has a low limb near 2^28: split from zero up, the four dropped products would make a whole unit; about zero
+    they vanish, and a quarter remains for the diagonal's, with the rounding of a double of E u."""
+    n = 256
+    u = ((700000001 << 28) + (1 << 27) - 32) * 2.0 ** -57
+    assert 1.0 <= u < 2.0
+    for L in np.linspace(29.0, 31.0, 20001):
+        c, ec = 0.5 / (L / n) ** 2, 1023 + math.frexp(2.0 / (L / n) ** 2)[1] - 1
+        if int(math.ldexp(c, 1079 - ec)) % (1 << 29) >= (1 << 29) - (1 << 20):
+            break
+    prob = inputs.free_problem(n, L, 2 * L / 3, math.pi / 6, 0.5, np.zeros((n - 1, n - 1), dtype=complex))
+    sv = _solver(prob, 4)
+    x = torch.full((n - 1, n - 1), u, dtype=torch.complex128, device="cuda")
+    y, r = torch.empty_like(x), torch.empty_like(x)
+    sv.matvec(x, y)
+    one = torch.zeros_like(x)
+    one[1::2, 1::2] = 1.0                            # the diagonal, and one axis' coefficients beside it
+    sv.level_residual(0, one.reshape(-1), torch.zeros_like(x).reshape(-1), r.reshape(-1))
+    i = np.arange(9, 129, 2)
+    D, w = (-r[j, 65].real.cpu().numpy().astype(np.longdouble) for j in (i, i + 1))
+    off = np.abs(y[i, 65].real.cpu().numpy() - u * (D + 2 * w))   # w: the south and north neighbours' sum
+    assert off.max() <= 0.5 * 2.0 ** (1023 + ec - 2101)
+    assert 0 in sv.integer_passes()[0]
+    sv.close()
