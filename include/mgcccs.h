@@ -240,7 +240,10 @@ int mgcccs_batch_solve(mgcccs_t* handles, int count, mgcccs_c128* const* u, cons
  * complex64 and z is its exact widening.  Async. */
 int mgcccs_precond_apply(mgcccs_t h, mgcccs_c128* z, const mgcccs_c128* r);
 
-/* y = (H-E)x on the fine level (Eq. (11)); x, y: device, distinct.  Async. */
+/* y = (H-E)x on the fine level (Eq. (11)); x, y: device, distinct.  Async.  An entry of y is
+ * within 2^-48 of the sum of the moduli of its five terms, however large the entries of x beside them
+ * (FP64 instructions give 2^-49); where the real and imaginary parts of x differ in size
+ * throughout, each part of y within that of its own terms. */
 int mgcccs_matvec(mgcccs_t h, const mgcccs_c128* x, mgcccs_c128* y);
 
 /* r = f - (H-E)u on the fine level (Eq. (11)); if norm2 is not NULL the

@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
   if constexpr (FXR) {
     // u as integers on the tile's exponent, each residual rounded to a double once
     __shared__ longlong2 T[(TY + 2) * PW];
-    __shared__ int eu_s;
-    if (t == 0) eu_s = 0;
+    __shared__ int2 eu_s;
+    if (t == 0) eu_s = make_int2(0, 0);
     __syncthreads();
     const auto ux = [](int q) { return q ? TX : -1; };
     TileShare<WY, TY + 2, 2> tu;
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
       r[q] = i < s.mx && j < s.my ? __ldg(f + (size_t)j * s.mx + i) : cmk(0.0, 0.0);
     }
     __syncthreads();
-    const int eu = eu_s;
+    const int eu = max(eu_s.x, eu_s.y);
     const bool oku = fx_ok(eu);
     tu.each(ux, [&](int row, int col, cplx z) {
       T[row * PW + col + 1] = oku ? fx_int(z, eu - 1080) : as_raw(z);

@@ -13,8 +13,6 @@ namespace {
 constexpr int BX = 32;
 
 __device__ __forceinline__ longlong2 ll2(long long a) { return make_longlong2(a, a); }
-// a quarter, to the nearest, ties to even
-__device__ __forceinline__ long long fx_quarter(long long a) { return (a + 1 + (a >> 2 & 1)) >> 2; }
 
 // f - (H - E) u with FP64 instructions from a tile of values
 template <class F>
@@ -63,16 +61,25 @@ __global__ void __launch_bounds__(256) k_row_bound(StencilView s, unsigned long 
   }
 }
 
+// the limbs of a value, or of a coefficient
+__device__ __forceinline__ int4 coef_limbs(cplx z, int E) {
+  const int4 v = fx_limbs(z, E);
+  int4 c;
+  fx_coef(((long long)v.x << 29) + v.y, &c.x, &c.y);
+  fx_coef(((long long)v.z << 29) + v.w, &c.z, &c.w);
+  return c;
+}
+template <bool COEF>
 __global__ void __launch_bounds__(256) k_split(long long n, const cplx* __restrict__ a, int E, int4* __restrict__ out) {
   for (long long p = blockIdx.x * 256LL + threadIdx.x; p < n; p += (long long)gridDim.x * 256)
-    out[p] = fx_limbs(a[p], E);
+    out[p] = COEF ? coef_limbs(a[p], E) : fx_limbs(a[p], E);
 }
 // An axis' west or east coefficients.  The inner region takes its closed form here as well, as the
 // FP64 passes do in a straddling block: the per-node values differ from it by the rounding of the
 // grid's coordinates (4e-14 of it at 592 nodes), and the two must be the same operator.
 __global__ void __launch_bounds__(256) k_split_axis(int n, AxisCoefT<cplx> ax, const cplx* __restrict__ a, int E,
                                                     int4* __restrict__ out) {
-  for (int p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) out[p] = fx_limbs(p < ax.u ? ax.cin : a[p], E);
+  for (int p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) out[p] = coef_limbs(p < ax.u ? ax.cin : a[p], E);
 }
 
 // ---- a level's (zero-start sweep,) residual and restriction.  A block takes 16 x DBY coarse nodes:
@@ -92,9 +99,9 @@ __global__ void __launch_bounds__(DT, 4) k_zrr_fx(StencilFx x, int mcx, int mcy,
   const StencilView& s = x.s;
   __shared__ longlong2 U[UR * DUW];
   __shared__ longlong2 Rt[RR * DRW];
-  __shared__ int eu_s, ef_s;
+  __shared__ int2 eu_s, ef_s;
   const int t = threadIdx.x, I0 = blockIdx.x * DBX, J0 = blockIdx.y * DBY, i0 = 2 * I0, j0 = 2 * J0;
-  if (t == 0) eu_s = ef_s = 0;
+  if (t == 0) eu_s = ef_s = make_int2(0, 0);
   __syncthreads();
   const auto ux = [](int c) { return c == 0 ? -1 : 31 + c; };          // columns -1, 32, 33
   const auto rx = [](int) { return 32; };
@@ -103,7 +110,7 @@ __global__ void __launch_bounds__(DT, 4) k_zrr_fx(StencilFx x, int mcx, int mcy,
   block_exponent(tu.load(ZERO ? f : u, s.mx, s.my, i0, j0 - 1, ux), &eu_s);
   block_exponent(tf.load(f, s.mx, s.my, i0, j0, rx), &ef_s);
   __syncthreads();
-  const int eu = eu_s, ef = ef_s;
+  const int eu = max(eu_s.x, eu_s.y), ef = max(ef_s.x, ef_s.y);
   const bool ok = fx_ok(eu) && fx_ok(ef);
   // units: of u (ZERO: the product of omega/D and f), below 2^58, and of the residuals, below 2^60,
   // so that four of them fit
@@ -210,25 +217,24 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
   static_assert(PE * PER <= BX * PY && PW * PER <= BX * PY, "one coarse value per thread");
   __shared__ longlong2 T[(PY + 2) * PW];
   __shared__ longlong2 Es[PER * PE], Ex[PER * PW];
-  __shared__ int eu_s, ef_s;
+  __shared__ int2 eu_s, ef_s;
   const int t = threadIdx.y * BX + threadIdx.x, i0 = blockIdx.x * BX, j0 = blockIdx.y * PY;
   const int i = i0 + threadIdx.x, j = j0 + threadIdx.y;
   const bool mine = i < s.mx && j < s.my;
-  if (t == 0) eu_s = ef_s = 0;
+  if (t == 0) eu_s = ef_s = make_int2(0, 0);
   __syncthreads();
   const auto ux = [](int c) { return c ? BX : -1; };
   TileShare<PY, PY + 2, 2> tu;
-  int eu = tu.load(u, s.mx, s.my, i0, j0 - 1, ux);
+  const int2 eu_t = tu.load(u, s.mx, s.my, i0, j0 - 1, ux);
   // coarse interior indices [i0/2 - 1, i0/2 + 16] x [j0/2 - 1, j0/2 + PY/2]
   const int er = t / PE, ei = t - er * PE, ci = i0 / 2 - 1 + ei, cj = j0 / 2 - 1 + er;
   const cplx e = t < PE * PER && ci >= 0 && cj >= 0 && ci < mcx && cj < mcy ? __ldg(ec + (size_t)cj * mcx + ci)
                                                                          : cmk(0.0, 0.0);
   const cplx fv = mine ? __ldg(f + (size_t)j * s.mx + i) : cmk(0.0, 0.0);
-  block_exponent(max(eu, fx_exp(e)), &eu_s);
-  block_exponent(fx_exp(fv), &ef_s);
+  block_exponent(fx_max_exp(eu_t, e), &eu_s);
+  block_exponent(fx_max_exp(make_int2(0, 0), fv), &ef_s);
   __syncthreads();
-  eu = eu_s;
-  const int ef = ef_s;
+  const int eu = max(eu_s.x, eu_s.y), ef = max(ef_s.x, ef_s.y);
   const bool ok = fx_ok(eu) && fx_ok(ef);
   // units: of v (u and P e below 2^57, (omega/D) f below 2^58) and of the residual (below 2^60)
   const int qu = max(eu, ef + x.ed - 1022) - 1079, qr = qu + x.ec - 1021;
@@ -310,17 +316,17 @@ __global__ void __launch_bounds__(BX * PY) k_apply_fx(StencilFx x, const cplx* _
   mgc_pdl_enter();
   const StencilView& s = x.s;
   __shared__ longlong2 T[(PY + 2) * PW];
-  __shared__ int eu_s;
+  __shared__ int2 eu_s;
   const int i0 = blockIdx.x * BX, j0 = blockIdx.y * PY, i = i0 + threadIdx.x, j = j0 + threadIdx.y;
-  if (threadIdx.x + threadIdx.y == 0) eu_s = 0;
+  if (threadIdx.x + threadIdx.y == 0) eu_s = make_int2(0, 0);
   __syncthreads();
   const auto ux = [](int c) { return c ? BX : -1; };
   TileShare<PY, PY + 2, 2> tu;
   block_exponent(tu.load(u, s.mx, s.my, i0, j0 - 1, ux), &eu_s);
   __syncthreads();
-  const int eu = eu_s;
-  const bool ok = fx_ok(eu);
-  tu.each(ux, [&](int r, int c, cplx z) { T[r * PW + c + 1] = ok ? fx_int(z, eu - 1080) : as_raw(z); });
+  const int eu = max(eu_s.x, eu_s.y);
+  bool ok = fx_tile_ok(eu_s);
+  if (ok) tu.each(ux, [&](int r, int c, cplx z) { T[r * PW + c + 1] = fx_int(z, eu - 1080); });
   __syncthreads();
   if (i >= s.mx || j >= s.my) return;
   const size_t p = (size_t)j * s.mx + i;
@@ -330,12 +336,16 @@ __global__ void __launch_bounds__(BX * PY) k_apply_fx(StencilFx x, const cplx* _
     fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
       const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(x, i, j, p, c, PW);
       const double sc = fx_pow2(eu + x.ec - 2104);
-      y[p] = cmk(sc * (double)h.x, sc * (double)h.y);
+      ok = fx_kept(fx_lead5(c, PW));
+      if (ok) y[p] = cmk(sc * (double)h.x, sc * (double)h.y);
     });
-  } else {
-    fp64_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
+  }
+  if (!ok) {
+    const cplx uw = ld_or_zero(u, p - 1, i > 0), ue = ld_or_zero(u, p + 1, i + 1 < s.mx);
+    const cplx us = ld_or_zero(u, p - s.mx, j > 0), un = ld_or_zero(u, p + s.mx, j + 1 < s.my);
+    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
       y[p] = apply_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
-          s, i, j, (int)p, as_cplx(c[0]), as_cplx(c[-1]), as_cplx(c[1]), as_cplx(c[-PW]), as_cplx(c[PW]));
+          s, i, j, (int)p, __ldg(u + p), uw, ue, us, un);
     });
   }
 }
@@ -366,12 +376,10 @@ cudaError_t launch_level_exponents(const StencilView& s, int* lim, cudaStream_t 
   return cudaGetLastError();
 }
 
-// Limbs of one value on the host, those of fx_limbs (down = 0).
-static void host_limbs(double x, int E, int* h, int* l) {
+// A coefficient's limbs on the host, those of coef_limbs.
+static void host_coef(double x, int E, int* h, int* l) {
   const long long m = (long long)std::floor(std::ldexp(std::fabs(x), 1079 - E) + 0.5);
-  const int sg = x < 0 ? -1 : 1;
-  *h = sg * (int)((m + (1LL << 28)) >> 29);
-  *l = sg * ((int)(m & 0x1fffffff) - ((m >> 28 & 1) << 29));
+  fx_coef(x < 0 ? -m : m, h, l);
 }
 
 // The level's operator as limbs in buf (level_fx_entries), if its exponents (lim, on the host)
@@ -398,16 +406,16 @@ cudaError_t level_fx(const StencilView& s, const int* lim, int4* buf, StencilFx*
     int4* a = buf + 2 * n;
     x.D = D; x.Di = Di;
     x.wx = a; x.ex = a + s.mx; x.wy = a + 2 * s.mx; x.ey = a + 2 * s.mx + s.my;
-    k_split<<<stride_blocks(n), 256, 0, st>>>(n, s.D, x.ec, D);
-    k_split<<<stride_blocks(n), 256, 0, st>>>(n, s.Dinv, x.ed, Di);
+    k_split<true><<<stride_blocks(n), 256, 0, st>>>(n, s.D, x.ec, D);
+    k_split<false><<<stride_blocks(n), 256, 0, st>>>(n, s.Dinv, x.ed, Di);
     k_split_axis<<<stride_blocks(s.mx), 256, 0, st>>>(s.mx, s.cx, s.west_x, x.ec, a);
     k_split_axis<<<stride_blocks(s.mx), 256, 0, st>>>(s.mx, s.cx, s.east_x, x.ec, a + s.mx);
     k_split_axis<<<stride_blocks(s.my), 256, 0, st>>>(s.my, s.cy, s.west_y, x.ec, a + 2 * s.mx);
     k_split_axis<<<stride_blocks(s.my), 256, 0, st>>>(s.my, s.cy, s.east_y, x.ec, a + 2 * s.mx + s.my);
-    host_limbs(s.cx.cin.x, x.ec, &x.cx.x, &x.cx.y);
-    host_limbs(s.cx.cin.y, x.ec, &x.cx.z, &x.cx.w);
-    host_limbs(s.cy.cin.x, x.ec, &x.cy.x, &x.cy.y);
-    host_limbs(s.cy.cin.y, x.ec, &x.cy.z, &x.cy.w);
+    host_coef(s.cx.cin.x, x.ec, &x.cx.x, &x.cx.y);
+    host_coef(s.cx.cin.y, x.ec, &x.cx.z, &x.cx.w);
+    host_coef(s.cy.cin.x, x.ec, &x.cy.x, &x.cy.y);
+    host_coef(s.cy.cin.y, x.ec, &x.cy.z, &x.cy.w);
   }
   *out = x;
   return cudaGetLastError();

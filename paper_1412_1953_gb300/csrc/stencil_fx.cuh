@@ -1,6 +1,8 @@
 // The 5-point operator on the integer pipes (fixed.cuh): a block turns its tile of grid values
 // into integers on one exponent, the operator's coefficients are kept as limbs on one exponent
-// per level, and a node's sums lose only the products of low limbs (2^-58 of the largest product).
+// per level, and a node's sums lose only the products of low limbs (2^-60 of the largest product).
+// One exponent for a tile leaves its small values fewer bits than a double has, so a tile or a
+// node takes FP64 instructions where that would show in a result (fx_tile_ok, fx_kept).
 // Where the operator cancels, the coarser levels amplify what a sum leaves on smooth data by its
 // condition, so every rounding here is to the nearest and without a mean.  V-cycles of 256^2 to 768 x 512
 // against extended precision with the device's coefficients: l2 error 0.5 to 1.06 times that of the
@@ -18,9 +20,9 @@ struct StencilFx {
   int on;
   int ec, ed;                              // exponents of west, east, D, and of omega/D
   int kd;                                  // 2100 - ec - ed, between 30 and 58
-  int4 cx, cy;                             // the inner regions' coefficients
-  const int4 *wx, *ex, *wy, *ey;           // per-node neighbour coefficients
-  const int4 *D, *Di;                      // [my*mx]
+  int4 cx, cy;                             // the inner regions' coefficients (fx_coef)
+  const int4 *wx, *ex, *wy, *ey;           // per-node neighbour coefficients (fx_coef)
+  const int4 *D, *Di;                      // [my*mx] (fx_coef; fx_limbs)
 };
 constexpr int FX_SPREAD = 4;
 // Most a node's |omega/D| times its row's sum of coefficients (|re| + |im| of each) may be.  In the
@@ -30,6 +32,14 @@ constexpr int FX_SPREAD = 4;
 // E = 135.  A level beyond it keeps to FP64.
 constexpr double FX_GAIN = 16.0;
 constexpr int FX_LIMITS = 8;               // ints of launch_level_exponents
+// A coefficient of 57 bits as h 2^27 + l / 4, |h| <= 2^30, |l| <= 2^28: finer in the low limb than a
+// value (split at 2^29), so that the products of low limbs that a sum drops are below 2^54, a quarter of
+// a unit for a value's last bit times the smallest neighbour coefficient of square cells.
+__host__ __device__ __forceinline__ void fx_coef(long long m, int* h, int* l) {
+  *h = (int)((m + (1 << 26)) >> 27);
+  *l = (int)(m - ((long long)*h << 27)) * 4;
+}
+
 // Levels of at least this many nodes run on the integer pipes: smaller ones are bound by a launch's
 // latency, and the exponent's reduction and barriers lengthen that.  The preconditioner by grid size
 // n, integer passes (three blocks an SM) on no level / on every level / from 60000 nodes (us): 128: 60.8 / 67.3 / 60.8,
@@ -58,6 +68,8 @@ __device__ __forceinline__ FxLimbs fx_split(long long v) {
   return FxLimbs{h, (int)((unsigned)v - ((unsigned)h << 29))};
 }
 __device__ __forceinline__ longlong2 fx_add(longlong2 a, longlong2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+// a quarter, to the nearest, ties to even
+__device__ __forceinline__ long long fx_quarter(long long a) { return (a + 1 + (a >> 2 & 1)) >> 2; }
 // (re, im) += a v, a complex (limbs) or real (its first two)
 __device__ __forceinline__ void fx_cmac(FxSum& re, FxSum& im, int4 a, longlong2 v) {
   const FxLimbs ax{a.x, a.y}, ay{a.z, a.w}, x = fx_split(v.x), y = fx_split(v.y);
@@ -71,9 +83,7 @@ __device__ __forceinline__ void fx_rmac(FxSum& re, FxSum& im, int ah, int al, lo
   fx_mac(re, a, fx_split(v.x));
   fx_mac(im, a, fx_split(v.y));
 }
-// The sum hh 2^58 + mid 2^29 divided by 2^58, or by 2^k, 30 <= k <= 58, rounded; the caller knows
-// that it fits.
-__device__ __forceinline__ long long fx_total(const FxSum& s) { return s.hh + ((s.mid + (1LL << 28)) >> 29); }
+// The sum hh 2^58 + mid 2^29 divided by 2^k, 30 <= k <= 58, rounded; the caller knows that it fits.
 __device__ __forceinline__ long long fx_scaled(const FxSum& s, int k) {
   return (s.hh << (58 - k)) + ((s.mid + (1LL << (k - 30))) >> (k - 29));
 }
@@ -125,8 +135,36 @@ __device__ __forceinline__ longlong2 fx_operator(const StencilFx& x, int i, int 
     }
     fx_cmac(re, im, __ldg(x.D + p), t[0]);
   }
-  if constexpr (XB > 0) return make_longlong2(fx_scaled(re, 58 - XB), fx_scaled(im, 58 - XB));
-  else return make_longlong2(fx_total(re), fx_total(im));
+  // the sums are hh 2^56 + mid 2^27 in products of units, hh and mid below 2^62; results in 2^58 or 2^55
+  const auto total = [](const FxSum& t) {
+    if constexpr (XB == 3) return (t.hh << 1) + ((t.mid + (1LL << 27)) >> 28);
+    else return fx_quarter(t.hh + ((t.mid + (1LL << 28)) >> 29));
+  };
+  static_assert(XB == 0 || XB == 3, "units of the result");
+  return make_longlong2(total(re), total(im));
+}
+
+__device__ __forceinline__ int2 fx_max_exp(int2 e, cplx z) {
+  return make_int2(max(e.x, fx_exp(z.x)), max(e.y, fx_exp(z.y)));
+}
+// Where one exponent will do for a tile of complex values with largest exponents e.x (real parts) and
+// e.y (imaginary parts): in range, and neither part more than 2^FX_NEAR below the other, unless it is zero.
+constexpr int FX_NEAR = 4;
+__device__ __forceinline__ bool fx_tile_ok(int2 e) {
+  const int hi = max(e.x, e.y), lo = min(e.x, e.y);
+  return fx_ok(hi) && (lo == 0 || hi - lo <= FX_NEAR);
+}
+// ... and for a node of it: of the values v that its sum takes (in units that put the tile's largest
+// between 2^57 and 2^58) at least one part is 2^53 or more, so that its rounding is no coarser than a
+// double's.  Collect the leading bits of all of them, then ask fx_kept.
+__device__ __forceinline__ int fx_lead(longlong2 v) {
+  const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
+  return (x ^ x >> 31) | (y ^ y >> 31);
+}
+__device__ __forceinline__ bool fx_kept(int lead) { return lead >= 1 << (53 - 32); }
+// of a node's five values
+__device__ __forceinline__ int fx_lead5(const longlong2* t, int pitch) {
+  return fx_lead(t[0]) | fx_lead(t[-1]) | fx_lead(t[1]) | fx_lead(t[-pitch]) | fx_lead(t[pitch]);
 }
 
 // A thread's share of a tile of ROWS x (32 + XC) complex values around the 32 columns i0..i0+31 and
@@ -137,20 +175,20 @@ struct TileShare {
   static constexpr int NR = (ROWS + NW - 1) / NW;
   static_assert(XC * ROWS <= 32 * NW, "one extra value per thread");
   cplx v[NR], x;
-  // loads from a (mx x my; zero outside) and returns the largest exponent
+  // loads from a (mx x my; zero outside) and returns the largest exponents of the parts
   template <class XF>
-  __device__ __forceinline__ int load(const cplx* __restrict__ a, int mx, int my, int i0, int jt, XF xc) {
+  __device__ __forceinline__ int2 load(const cplx* __restrict__ a, int mx, int my, int i0, int jt, XF xc) {
     const int lane = threadIdx.x & 31, t = threadIdx.x + threadIdx.y * blockDim.x, w = t >> 5, i = i0 + lane;
-    int e = 0;
+    int2 e = make_int2(0, 0);
 #pragma unroll
     for (int n = 0; n < NR; ++n) {
       const int r = w + NW * n, j = jt + r;
       v[n] = r < ROWS && i < mx && j >= 0 && j < my ? __ldg(a + (size_t)j * mx + i) : cmk(0.0, 0.0);
-      e = max(e, fx_exp(v[n]));
+      e = fx_max_exp(e, v[n]);
     }
     const int r = t / XC, i2 = i0 + xc(t - r * XC), j2 = jt + r;
     x = t < XC * ROWS && i2 >= 0 && i2 < mx && j2 >= 0 && j2 < my ? __ldg(a + (size_t)j2 * mx + i2) : cmk(0.0, 0.0);
-    return max(e, fx_exp(x));
+    return fx_max_exp(e, x);
   }
   template <class XF, class F>
   __device__ __forceinline__ void each(XF xc, F&& put) const {
@@ -170,10 +208,17 @@ __device__ __forceinline__ cplx as_cplx(longlong2 v) {
 __device__ __forceinline__ longlong2 as_raw(cplx v) {
   return make_longlong2(__double_as_longlong(v.x), __double_as_longlong(v.y));
 }
-// The largest exponent over the block, in *es (cleared before).
-__device__ __forceinline__ void block_exponent(int e, int* es) {
-  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if ((threadIdx.x & 31) == 0) atomicMax(es, e);
+// The largest exponents over the block, in *es (cleared before).
+__device__ __forceinline__ void block_exponent(int2 e, int2* es) {
+  e.x = (int)__reduce_max_sync(0xffffffffu, (unsigned)e.x);
+  e.y = (int)__reduce_max_sync(0xffffffffu, (unsigned)e.y);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&es->x, e.x);
+    atomicMax(&es->y, e.y);
+  }
+}
+__device__ __forceinline__ cplx ld_or_zero(const cplx* __restrict__ a, size_t p, bool ok) {
+  return ok ? __ldg(a + p) : cmk(0.0, 0.0);
 }
 
 // kernels_fx.cu

@@ -7,6 +7,7 @@ import pytest
 
 from paper_1412_1953_gb300 import build, inputs
 from paper_1412_1953_gb300 import mgcccs as M
+from test_gpu_fixed_bias import _apply, _coefficients
 
 torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu,
@@ -144,4 +145,50 @@ def test_inner_coefficients_are_split_about_zero():
     off = np.abs(y[i, 65].real.cpu().numpy() - u * (D + 2 * w))   # w: the south and north neighbours' sum
     assert off.max() <= 0.5 * 2.0 ** (1023 + ec - 2101)
     assert 0 in sv.integer_passes()[0]
+    sv.close()
+
+
+def _field(kind, shape, g):
+    """Values of very different size: entries of 2^60 among ones; 2^-2 a node along x, 2^-1 along y; parts of
+    different size; zeros but for a few patches; standing waves with nodal lines."""
+    u = g.standard_normal(shape) + 1j * g.standard_normal(shape)
+    j, i = np.indices(shape)
+    if kind == "spikes":
+        u[::37, ::23] = 2.0 ** 60
+    elif kind == "decaying":
+        u *= np.exp2(-2.0 * (i % 250) - 1.0 * j)
+    elif kind == "parts":
+        u = u.real * 2.0 ** 50 + 1j * u.imag
+    elif kind == "patches":
+        u[(i // 10 + j // 10) % 7 > 0] = 0.0
+    elif kind == "waves":
+        u = np.sin(0.11 * i) * np.sin(0.07 * j) * (1.0 + 1j)
+    return u
+
+
+FIELDS = ["gauss", "spikes", "decaying", "parts", "patches", "waves"]
+
+
+def _moduli(A, v, f=0.0):
+    """|f| + the sum of the moduli of a node's five terms."""
+    return np.abs(f) + _apply([np.abs(a) for a in A], np.abs(v))
+
+
+# A sum takes the integer pipes where some value of it keeps 53 bits: five values to half a unit and ten
+# dropped products to a quarter of the smallest coefficient's are 22 units of 2^-53 of the sum of moduli, 32 with
+# cells that are not square; FP64 instructions are within 14.
+@pytest.mark.parametrize("kind", FIELDS)
+def test_operator_entry_by_entry(kind):
+    prob = _problem(320, 256)
+    sv = _solver(prob, 4)
+    A = _coefficients(sv, 0, prob.f.shape)
+    x = _field(kind, prob.f.shape, np.random.default_rng(3))
+    y = torch.empty(prob.f.shape, dtype=torch.complex128, device="cuda")
+    sv.matvec(torch.as_tensor(x).to("cuda"), y)
+    y, v = y.cpu().numpy(), x.astype(np.clongdouble)
+    assert (np.abs(y - _apply(A, v)) <= 32 * 2.0 ** -53 * _moduli(A, v)).all()
+    if kind == "parts":                              # real coefficients keep the parts apart
+        box = (slice(0, 168), slice(0, 210))
+        im = v.imag.astype(np.clongdouble)
+        assert (np.abs(y.imag - _apply(A, im).real) <= 32 * 2.0 ** -53 * _moduli(A, im))[box].all()
     sv.close()
