@@ -14,12 +14,6 @@ constexpr int BX = 32;
 
 __device__ __forceinline__ longlong2 ll2(long long a) { return make_longlong2(a, a); }
 
-// f - (H - E) u with FP64 instructions from a tile of values
-template <class F>
-__device__ __forceinline__ void fp64_kinds(const StencilView& s, int i0, int i1, int j0, int j1, F&& f) {
-  dispatch_kinds(s, i0, i1, j0, j1, f);
-}
-
 // ---- level operator as limbs
 
 // lim[0], lim[1] = largest and smallest exponent of the n values (of the larger component).
@@ -86,8 +80,10 @@ __global__ void __launch_bounds__(256) k_split_axis(int n, AxisCoefT<cplx> ax, c
 // u on the fine nodes [2 I0 - 1, 2 I0 + 33] x [2 J0 - 1, 2 J0 + 2 DBY + 1] as integers in shared
 // memory, the residuals on the tile less its rim as integers in f's and (H - E)u's common unit,
 // then the weighted sums, shifts and additions only, and one conversion per coarse value.  With
-// ZERO, u = (omega/D) f is formed first (and stored for the nodes the block owns).  Bound by the
-// integer pipe and the latency of its three barriers.  With cold L2 at 1023^2, zero start: 39.5 us
+// ZERO, u = (omega/D) f is formed first, with FP64 instructions (two or four, which keep each value's
+// bits), and stored for the nodes the block owns.  A block of which some residual's terms all lie
+// below 2^53 units takes FP64 instructions throughout: its coarse values are made of such residuals.
+// Bound by the integer pipe and the latency of its barriers.  With cold L2 at 1023^2, zero start: 39.5 us
 // (sweep 11.5 + residual and restriction 47.3 us with FP64 instructions).  Four blocks an SM: the
 // preconditioner takes 226 us with three, 220 us with four.
 constexpr int DBX = 16, DBY = 8, DT = 256, UR = 2 * DBY + 3, RR = 2 * DBY + 1, DUW = 2 * DBX + 3, DRW = 2 * DBX + 1;
@@ -105,92 +101,96 @@ __global__ void __launch_bounds__(DT, 4) k_zrr_fx(StencilFx x, int mcx, int mcy,
   __syncthreads();
   const auto ux = [](int c) { return c == 0 ? -1 : 31 + c; };          // columns -1, 32, 33
   const auto rx = [](int) { return 32; };
+  const bool box = s.rbox && i0 + DUW - 1 <= s.cx.u && j0 + UR - 1 <= s.cy.u;   // omega/D real throughout
+  const auto sweep = [&](size_t p, cplx fp) {                           // (omega/D) f
+    return box ? cscal(ldre(s.Dinv, (int)p), fp) : cmul(__ldg(s.Dinv + p), fp);
+  };
   TileShare<DT / 32, UR, 3> tu;
   TileShare<DT / 32, RR, 1> tf;                                         // f at the residual nodes
-  block_exponent(tu.load(ZERO ? f : u, s.mx, s.my, i0, j0 - 1, ux), &eu_s);
+  int2 eu_t = tu.load(ZERO ? f : u, s.mx, s.my, i0, j0 - 1, ux);
   block_exponent(tf.load(f, s.mx, s.my, i0, j0, rx), &ef_s);
+  if constexpr (ZERO) {
+    eu_t = make_int2(0, 0);
+    tu.each(ux, [&](int r, int c, cplx& z) {
+      const int i = i0 + c, j = j0 - 1 + r;
+      if (i < 0 || j < 0 || i >= s.mx || j >= s.my) return;
+      const size_t p = (size_t)j * s.mx + i;
+      z = sweep(p, z);
+      const int oi = min(i >> 1, mcx - 1), oj = min(j >> 1, mcy - 1);
+      if (oi >= I0 && oi < I0 + DBX && oj >= J0 && oj < J0 + DBY) u[p] = z;
+      eu_t = fx_max_exp(eu_t, z);
+    });
+  }
+  block_exponent(eu_t, &eu_s);
   __syncthreads();
   const int eu = max(eu_s.x, eu_s.y), ef = max(ef_s.x, ef_s.y);
-  const bool ok = fx_ok(eu) && fx_ok(ef);
-  // units: of u (ZERO: the product of omega/D and f), below 2^58, and of the residuals, below 2^60,
-  // so that four of them fit
-  const int qu = ZERO ? eu + x.ed - 2101 : eu - 1080, qt = qu + x.ec - 1021, qr = max(qt, ef - 1081);
-  tu.each(ux, [&](int r, int c, cplx z) {
-    const int i = i0 + c, j = j0 - 1 + r;
-    longlong2 w = ll2(0);
-    if (i >= 0 && j >= 0 && i < s.mx && j < s.my) {
-      const size_t p = (size_t)j * s.mx + i;
-      const int oi = min(i >> 1, mcx - 1), oj = min(j >> 1, mcy - 1);
-      const bool own = ZERO && oi >= I0 && oi < I0 + DBX && oj >= J0 && oj < J0 + DBY;
-      if (!ok) {
-        if constexpr (ZERO) {
-          z = cmul(__ldg(s.Dinv + p), z);
-          if (own) u[p] = z;
-        }
-        w = as_raw(z);
-      } else if constexpr (ZERO) {
-        FxSum re{0, 0}, im{0, 0};
-        fx_cmac(re, im, __ldg(x.Di + p), fx_int(z, eu - 1079));
-        w = make_longlong2(fx_scaled(re, 57), fx_scaled(im, 57));
-        if (own) {
-          const double sc = fx_pow2(qu);
-          u[p] = cmk(sc * (double)w.x, sc * (double)w.y);
-        }
-      } else {
-        w = fx_int(z, qu);
-      }
-    }
-    U[r * DUW + c + 1] = w;
-  });
-  __syncthreads();
+  bool ok = fx_tile_ok(eu_s) && fx_tile_ok(ef_s);
+  // units: of u, below 2^58, and of the residuals, below 2^60, so that four of them fit
+  const int qu = eu - 1080, qt = qu + x.ec - 1021, qr = max(qt, ef - 1081);
   const int i1 = min(i0 + DRW, s.mx), j1 = min(j0 + RR, s.my);
   if (ok) {
+    tu.each(ux, [&](int r, int c, cplx z) { U[r * DUW + c + 1] = fx_int(z, qu); });
+    __syncthreads();
     const int d = qr - qt;                               // positive only where f exceeds (H - E)u's range
+    bool low = false;
     fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
       tf.each(rx, [&](int r, int c, cplx z) {
         const int i = i0 + c, j = j0 + r;
         if (i >= s.mx || j >= s.my) return;
+        const longlong2* q = U + (r + 1) * DUW + c + 1;
         longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value>(
-            x, i, j, (size_t)j * s.mx + i, U + (r + 1) * DUW + c + 1, DUW);
-        if (!ZERO && d > 0) {
+            x, i, j, (size_t)j * s.mx + i, q, DUW);
+        int lead = fx_lead5(q, DUW);
+        if (d > 0) {
           const int k = min(d, 62);
           const long long b = (1LL << (k - 1)) - 1;                     // to the nearest, ties to even
           h = make_longlong2((h.x + b + (h.x >> k & 1)) >> k, (h.y + b + (h.y >> k & 1)) >> k);
+          lead >>= min(d, 31);
         }
         const longlong2 fi = fx_int(z, qr);
+        low = low || !fx_kept(lead | fx_lead(fi));
         Rt[r * DRW + c] = make_longlong2(fi.x - h.x, fi.y - h.y);
       });
     });
-  } else {
-    fp64_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
+    ok = !__syncthreads_or(low);
+  }
+  if (!ok) {
+    const auto val = [&](size_t p, bool in) {
+      if (!in) return cmk(0.0, 0.0);
+      const cplx z = __ldg((ZERO ? f : u) + p);
+      return ZERO ? sweep(p, z) : z;
+    };
+    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
       tf.each(rx, [&](int r, int c, cplx z) {
         const int i = i0 + c, j = j0 + r;
         if (i >= s.mx || j >= s.my) return;
-        const longlong2* q = U + (r + 1) * DUW + c + 1;
-        Rt[r * DRW + c] = as_raw(residual_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value,
-                                               decltype(dg)::value>(s, i, j, j * s.mx + i, as_cplx(q[0]),
-                                                                    as_cplx(q[-1]), as_cplx(q[1]), as_cplx(q[-DUW]),
-                                                                    as_cplx(q[DUW]), z));
+        const size_t p = (size_t)j * s.mx + i;
+        Rt[r * DRW + c] = as_raw(
+            residual_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
+                s, i, j, (int)p, val(p, true), val(p - 1, i > 0), val(p + 1, i + 1 < s.mx), val(p - s.mx, j > 0),
+                val(p + s.mx, j + 1 < s.my), z));
       });
     });
+    __syncthreads();
   }
-  __syncthreads();
   const int I = I0 + t % DBX, J = J0 + t / DBX;
   if (t >= DBX * DBY || I >= mcx || J >= mcy) return;
   const longlong2* c = Rt + (2 * (t / DBX) + 1) * DRW + 2 * (t % DBX) + 1;   // on fine node (2I+1, 2J+1)
   if (ok) {
+    // a sixteenth of 4 centre + 2 edge + corner as a double: exact before its rounding below 2^58, else
+    // first to the nearest integer, ties to even (a floor's constant bias is a smooth residual, which
+    // the coarse levels amplify: measured 60 times the error)
+    const double sc = fx_pow2(qr);
     auto weigh = [&](auto get) {
       const long long edge = get(-1) + get(1) + get(-DRW) + get(DRW);
       const long long corner = get(-DRW - 1) + get(-DRW + 1) + get(DRW - 1) + get(DRW + 1);
-      // a sixteenth of 4 centre + 2 edge + corner, to the nearest, ties to even: a floor's constant
-      // bias is a smooth residual, which the coarse levels amplify (measured 60 times the error)
       const long long whole = (get(0) >> 2) + (edge >> 3) + (corner >> 4);
       const int rest = 4 * (int)(get(0) & 3) + 2 * (int)(edge & 7) + (int)(corner & 15);
-      return whole + ((rest + 7 + ((int)(whole + (rest >> 4)) & 1)) >> 4);
+      const bool fits = (whole ^ whole >> 63) >> 58 == 0;
+      const long long sum = fits ? (whole << 4) + rest : whole + ((rest + 7 + ((int)(whole + (rest >> 4)) & 1)) >> 4);
+      return (fits ? 0.0625 * sc : sc) * (double)sum;
     };
-    const double sc = fx_pow2(qr);
-    fc[(size_t)J * mcx + I] = cmk(sc * (double)weigh([&](int o) { return c[o].x; }),
-                                  sc * (double)weigh([&](int o) { return c[o].y; }));
+    fc[(size_t)J * mcx + I] = cmk(weigh([&](int o) { return c[o].x; }), weigh([&](int o) { return c[o].y; }));
   } else {
     auto get = [&](int o) { return as_cplx(c[o]); };
     const cplx corner = cadd(cadd(get(-DRW - 1), get(-DRW + 1)), cadd(get(DRW - 1), get(DRW + 1)));
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
       o[p] = cmk(sc * (double)(c[0].x + fx_scaled(re, x.kd)), sc * (double)(c[0].y + fx_scaled(im, x.kd)));
     });
   } else {
-    fp64_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
+    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
       o[p] = jacobi_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
           s, i, j, (int)p, as_cplx(c[0]), as_cplx(c[-1]), as_cplx(c[1]), as_cplx(c[-PW]), as_cplx(c[PW]), fv);
     });

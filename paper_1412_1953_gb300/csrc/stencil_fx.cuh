@@ -191,7 +191,7 @@ struct TileShare {
     return fx_max_exp(e, x);
   }
   template <class XF, class F>
-  __device__ __forceinline__ void each(XF xc, F&& put) const {
+  __device__ __forceinline__ void each(XF xc, F&& put) {
     const int lane = threadIdx.x & 31, t = threadIdx.x + threadIdx.y * blockDim.x, w = t >> 5;
 #pragma unroll
     for (int n = 0; n < NR; ++n) {

@@ -192,3 +192,58 @@ def test_operator_entry_by_entry(kind):
         im = v.imag.astype(np.clongdouble)
         assert (np.abs(y.imag - _apply(A, im).real) <= 32 * 2.0 ** -53 * _moduli(A, im))[box].all()
     sv.close()
+
+
+# At E = -200 the operator's inverse decays from node to node on every level, so more than 30 nodes from a
+# spike of 2^70 an entry is far below the 2^13 that the last bit of its tile's largest is worth. There
+# the cycle agrees with the one-step calls to 1e-12 of the largest entry within 4 nodes (1e-13 of the
+# largest of all on ordinary data): both take the spike's remainder through the same coarse levels.
+@pytest.mark.parametrize("nu1,nu2", [(1, 0)])
+def test_cycle_beside_spikes(nu1, nu2):
+    prob = _problem(256, 256, E=-200.0)
+    sv = _solver(prob, 4, nu1=nu1, nu2=nu2)
+    g = np.random.default_rng(17)
+    shape = prob.f.shape
+    far = np.ones(shape, bool)
+    j, i = np.indices(shape)
+    spikes = np.zeros(shape, complex)
+    for b in range(0, shape[0], 64):
+        for a in range(0, shape[1], 96):             # the corner of a 32 x 16 and of a 32 x 8 tile
+            spikes[b, a] = 2.0 ** 70
+            far &= abs(i - a) + abs(j - b) > 30
+    f, u0 = (g.standard_normal(shape) + 1j * g.standard_normal(shape) for _ in range(2))
+    far = torch.as_tensor(far).to("cuda")
+    near = lambda x: torch.nn.functional.max_pool2d(x.abs()[None], 9, 1, 4)[0]   # the largest within 4 nodes
+    for df, du in ((300.0, 0.0), (0.0, 1.0)):
+        fd, u = (torch.as_tensor(x).to("cuda") for x in (300.0 * f + df * spikes, u0 + du * spikes))
+        ref = _composed(sv, 4, fd, u, nu1, nu2)
+        sv.vcycle(u, fd)
+        assert bool(((u - ref).abs() <= 1e-12 * near(ref))[far].all())
+        z = torch.zeros_like(fd)
+        sv.precond_apply(z, fd)
+        ref = _composed(sv, 4, fd, torch.zeros_like(fd), nu1, nu2)
+        assert bool(((z - ref).abs() <= 1e-12 * near(ref))[far].all())
+    assert 0 in sv.integer_passes()[0]
+    sv.close()
+
+
+# Without complex scaling and rotation everything is real, and the two parts are two separate cycles: one
+# 2^-70 of the other is as precise as alone.
+@pytest.mark.parametrize("nu1,nu2", [(1, 0)])
+def test_parts_of_different_size(nu1, nu2):
+    prob = inputs.temkin_poet(256, L=30.0, R0=30.0, theta=0.0, E=-400.0, seed=3, ny=256)
+    sv = _solver(prob, 4, nu1=nu1, nu2=nu2, coarse_gamma=0.0)
+    g = np.random.default_rng(19)
+    f, u0 = (torch.as_tensor(g.standard_normal((2,) + prob.f.shape)).to("cuda") for _ in range(2))
+    join = lambda a, s: torch.complex(a[0] * s, a[1])
+    u, v = join(u0, 2.0 ** 70), join(u0, 1.0)
+    sv.vcycle(u, join(f, 2.0 ** 79))
+    sv.vcycle(v, join(f, 2.0 ** 9))
+    assert float((u.real / 2.0 ** 70 - v.real).abs().max() / v.real.abs().max()) <= 1e-13
+    f[1] *= 2.0 ** 9
+    u, v = join(u0, 2.0 ** 70), join(u0, 1.0)
+    sv.vcycle(u, join(f, 2.0 ** 79))
+    sv.vcycle(v, join(f, 2.0 ** 9))
+    assert float((u.imag - v.imag).abs().max() / v.imag.abs().max()) <= 1e-13
+    assert 0 in sv.integer_passes()[0]
+    sv.close()
