@@ -12,7 +12,6 @@ namespace {
 
 constexpr int BX = 32;
 
-__device__ __forceinline__ longlong2 ll2(long long a) { return make_longlong2(a, a); }
 
 // ---- level operator as limbs
 
@@ -204,10 +203,43 @@ __global__ void __launch_bounds__(DT, 4) k_zrr_fx(StencilFx x, int mcx, int mcy,
 // ---- a level's prolongation and first post-smoothing sweep, o = v + (omega/D)(f - (H - E) v) with
 // v = u + P e.  A block forms twice the coarse values of its region interpolated along x, then v on
 // its 32 x 8 nodes and a rim of one as integers in a unit that also holds (omega/D) f, the residual
-// as integers, and the update as one integer per component.  Bound by the integer pipe:
+// as integers, and the update as one integer per component.  A node whose terms all lie below 2^53
+// units takes FP64 instructions, from the arrays (pj_node).  Bound by the integer pipe:
 // 33.6 us at 1023^2 with cold L2 (prolongation 13.2 + sweep 34.9 us with FP64 instructions).  Four
 // blocks an SM: 220 us for the preconditioner, against 231 us with three and 229 us with five.
 constexpr int PW = BX + 2, PY = 8, PE = BX / 2 + 2, PER = PY / 2 + 2;
+
+// One node with FP64 instructions.  Out of line: few nodes need it, and inlined its registers are
+// the pass's.
+__device__ __noinline__ cplx pj_node(const StencilView& s, int mcx, int mcy, const cplx* __restrict__ ec,
+                                     const cplx* __restrict__ u, const cplx* __restrict__ f, int i, int j) {
+  const auto v = [&](int a, int b) {
+    if (a < 0 || b < 0 || a >= s.mx || b >= s.my) return cmk(0.0, 0.0);
+    const auto e = [&](int q, int r) {
+      return ld_or_zero(ec, (size_t)r * mcx + q, q >= 0 && r >= 0 && q < mcx && r < mcy);
+    };
+    // on coarse index a >> 1 where a is odd, else between that and the one before
+    const int q = a >> 1, r = b >> 1;
+    cplx y = e(q, r);
+    double h = 1.0;
+    if (!(a & 1) && !(b & 1)) {
+      y = cadd(cadd(e(q - 1, r - 1), e(q, r - 1)), cadd(e(q - 1, r), y));
+      h = 0.25;
+    } else if (!(a & 1)) {
+      y = cadd(e(q - 1, r), y);
+      h = 0.5;
+    } else if (!(b & 1)) {
+      y = cadd(e(q, r - 1), y);
+      h = 0.5;
+    }
+    const cplx z = __ldg(u + (size_t)b * s.mx + a);
+    return cmk(fma(h, y.x, z.x), fma(h, y.y, z.y));
+  };
+  const int p = j * s.mx + i;
+  const cplx c = v(i, j), w = v(i - 1, j), e = v(i + 1, j), so = v(i, j - 1), n = v(i, j + 1), fp = __ldg(f + p);
+  if (s.cx.in_real && s.cy.in_real) return jacobi_vals<AX_GEN, AX_GEN, 1, DG_GEN>(s, i, j, p, c, w, e, so, n, fp);
+  return jacobi_vals<AX_GEN, AX_GEN, 0, DG_GEN>(s, i, j, p, c, w, e, so, n, fp);
+}
 
 __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int mcy, const cplx* __restrict__ ec,
                                                    const cplx* __restrict__ u, cplx* __restrict__ o,
@@ -235,12 +267,12 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
   block_exponent(fx_max_exp(make_int2(0, 0), fv), &ef_s);
   __syncthreads();
   const int eu = max(eu_s.x, eu_s.y), ef = max(ef_s.x, ef_s.y);
-  const bool ok = fx_ok(eu) && fx_ok(ef);
+  bool ok = fx_tile_ok(eu_s) && fx_tile_ok(ef_s);
   // units: of v (u and P e below 2^57, (omega/D) f below 2^58) and of the residual (below 2^60)
   const int qu = max(eu, ef + x.ed - 1022) - 1079, qr = qu + x.ec - 1021;
-  if (t < PE * PER) Es[t] = ok ? fx_int(e, qu) : as_raw(e);
-  __syncthreads();
   if (ok) {
+    if (t < PE * PER) Es[t] = fx_int(e, qu);
+    __syncthreads();
     // column a = i0 - 1 + q odd: on coarse index a >> 1, even: between that and the one before
     if (t < PW * PER) {
       const int r = t / PW, q = t - r * PW;
@@ -250,7 +282,7 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
     __syncthreads();
     tu.each(ux, [&](int r, int c, cplx z) {
       const int a = i0 + c, b = j0 - 1 + r;
-      longlong2 w = ll2(0);
+      longlong2 w = make_longlong2(0, 0);
       if (a >= 0 && b >= 0 && a < s.mx && b < s.my) {
         const longlong2* g = Ex + ((b >> 1) - (j0 / 2 - 1)) * PW + c + 1;
         const longlong2 y = fx_add(g[0], g[b & 1 ? 0 : -PW]);          // four times P e
@@ -258,39 +290,19 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
       }
       T[r * PW + c + 1] = w;
     });
-  } else {
-    tu.each(ux, [&](int r, int c, cplx z) {
-      const int a = i0 + c, b = j0 - 1 + r;
-      cplx y = cmk(0.0, 0.0);
-      if (a >= 0 && b >= 0 && a < s.mx && b < s.my) {
-        const longlong2* g = Es + ((b >> 1) - (j0 / 2 - 1)) * PE + (a >> 1) - (i0 / 2 - 1);
-        double h = 1.0;
-        y = as_cplx(g[0]);
-        if (!(a & 1) && !(b & 1)) {
-          y = cadd(cadd(as_cplx(g[-PE - 1]), as_cplx(g[-PE])), cadd(as_cplx(g[-1]), y));
-          h = 0.25;
-        } else if (!(a & 1)) {
-          y = cadd(as_cplx(g[-1]), y);
-          h = 0.5;
-        } else if (!(b & 1)) {
-          y = cadd(as_cplx(g[-PE]), y);
-          h = 0.5;
-        }
-        y = cmk(fma(h, y.x, z.x), fma(h, y.y, z.y));
-      }
-      T[r * PW + c + 1] = as_raw(y);
-    });
+    __syncthreads();
   }
-  __syncthreads();
   if (!mine) return;
   const size_t p = (size_t)j * s.mx + i;
-  const longlong2* c = T + (threadIdx.y + 1) * PW + threadIdx.x + 1;
-  const int i1 = min(i0 + BX, s.mx), j1 = min(j0 + PY, s.my);
   if (ok) {
+    const longlong2* c = T + (threadIdx.y + 1) * PW + threadIdx.x + 1;
+    const int i1 = min(i0 + BX, s.mx), j1 = min(j0 + PY, s.my);
     fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
       const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value>(x, i, j, p, c, PW);
       const longlong2 fi = fx_int(fv, qr);
       const longlong2 r = make_longlong2(fi.x - h.x, fi.y - h.y);
+      // (omega/D) f is at least 2^(52 - kd) f in units of v
+      ok = fx_kept(fx_lead5(c, PW) | fx_lead(fi) >> max(x.kd - 52, 0));
       FxSum re{0, 0}, im{0, 0};
       if constexpr (decltype(rd)::value) {
         const int2 d = __ldg(reinterpret_cast<const int2*>(x.Di + p));
@@ -299,14 +311,10 @@ __global__ void __launch_bounds__(BX * PY, 4) k_pj_fx(StencilFx x, int mcx, int 
         fx_cmac(re, im, __ldg(x.Di + p), r);
       }
       const double sc = fx_pow2(qu);
-      o[p] = cmk(sc * (double)(c[0].x + fx_scaled(re, x.kd)), sc * (double)(c[0].y + fx_scaled(im, x.kd)));
-    });
-  } else {
-    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
-      o[p] = jacobi_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
-          s, i, j, (int)p, as_cplx(c[0]), as_cplx(c[-1]), as_cplx(c[1]), as_cplx(c[-PW]), as_cplx(c[PW]), fv);
+      if (ok) o[p] = cmk(sc * (double)(c[0].x + fx_scaled(re, x.kd)), sc * (double)(c[0].y + fx_scaled(im, x.kd)));
     });
   }
+  if (!ok) o[p] = pj_node(s, mcx, mcy, ec, u, f, i, j);
 }
 
 // ---- y = (H - E) x.  Four FP64 instructions a node (two conversions, two products) and as much

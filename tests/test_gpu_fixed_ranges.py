@@ -198,7 +198,7 @@ def test_operator_entry_by_entry(kind):
 # spike of 2^70 an entry is far below the 2^13 that the last bit of its tile's largest is worth. There
 # the cycle agrees with the one-step calls to 1e-12 of the largest entry within 4 nodes (1e-13 of the
 # largest of all on ordinary data): both take the spike's remainder through the same coarse levels.
-@pytest.mark.parametrize("nu1,nu2", [(1, 0)])
+@pytest.mark.parametrize("nu1,nu2", [(1, 0), (0, 1), (1, 1)])
 def test_cycle_beside_spikes(nu1, nu2):
     prob = _problem(256, 256, E=-200.0)
     sv = _solver(prob, 4, nu1=nu1, nu2=nu2)
@@ -229,7 +229,7 @@ def test_cycle_beside_spikes(nu1, nu2):
 
 # Without complex scaling and rotation everything is real, and the two parts are two separate cycles: one
 # 2^-70 of the other is as precise as alone.
-@pytest.mark.parametrize("nu1,nu2", [(1, 0)])
+@pytest.mark.parametrize("nu1,nu2", [(1, 0), (0, 1), (1, 1)])
 def test_parts_of_different_size(nu1, nu2):
     prob = inputs.temkin_poet(256, L=30.0, R0=30.0, theta=0.0, E=-400.0, seed=3, ny=256)
     sv = _solver(prob, 4, nu1=nu1, nu2=nu2, coarse_gamma=0.0)
