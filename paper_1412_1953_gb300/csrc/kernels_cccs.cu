@@ -91,23 +91,44 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
 // (rows).  A residual's 2 n_b complex products then cost 24 n_b integer multiply-adds, 96 n_b
 // cycles of a quarter of an SM, against 8 n_b FP64 instructions, 512 n_b cycles.  FXR: the
 // residuals are formed from u on the tile's exponent as well (stencil_fx.cuh); of the tile heights
-// only 4 rows a warp, whose grids are large enough for it.  1023^2, n_b = 3, cold L2: 76.6 us with
+// only 4 rows a warp, whose grids are large enough for it.  A residual whose terms all lie below
+// 2^53 units takes FP64 instructions, and so does a tile with a row's (column's) projection whose
+// products all lie below 2^-FX_NEAR of the tile's largest: 3 to 7 % of the tiles of 32 rows in a
+// solve at 512^2, up to 19 % at 256^2.  1023^2, n_b = 3, cold L2: 76.6 us with
 // FP64 instructions, 41.2 us with integer projections, 36.2 us with both; 127^2: 19.2 us in tiles of 32 rows (16 blocks), 7.4
 // us in tiles of 8 (cold L2).
 template <int NB, int SY, bool FXR>
 __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CCView c, const cplx* __restrict__ u,
-                                                                 const cplx* __restrict__ f) {
-  mgc_pdl_enter();
+                                                                const cplx* __restrict__ f) {
   const StencilView& s = x.s;
   constexpr int TY = SY * WY, PW = TX + 2;
   __shared__ int4 R[TY][TX + 1];                         // limbs, or the values themselves
   __shared__ int4 wl[NB][TX], wr[NB][TY];
+  __shared__ int xl[NB][TX], xr[NB][TY];                 // exponents of the weighted values
   __shared__ int ewl[NB], ewr[NB], eR, bad;
+  __shared__ int pmax[NB][TX];                           // largest exponent of a column's products
   const int lane = threadIdx.x, wy = threadIdx.y, t = wy * TX + lane;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, i = i0 + lane;
   if (t == 0) eR = bad = 0;
+  if (t < NB * TX) pmax[t / TX][t % TX] = 0;
   __syncthreads();
+  for (int p = wy; p < 2 * NB; p += WY) {                // a warp converts one state's values of the tile
+    const int m = p >> 1, n = p & 1 ? TY : TX, k = (p & 1 ? j0 : i0) + lane, len = p & 1 ? s.my : s.mx;
+    const cplx w = lane < n && k < len ? __ldg((p & 1 ? c.wvphi : c.wphi) + (size_t)m * len + k) : cmk(0.0, 0.0);
+    const int e = fx_exp(w), ew = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+    if (lane < n) {
+      (p & 1 ? wr[m] : wl[m])[lane] = fx_limbs(w, ew, lane & 1);
+      (p & 1 ? xr[m] : xl[m])[lane] = e;
+    }
+    if (lane == 0) {
+      (p & 1 ? ewr : ewl)[m] = ew;
+      if (!fx_ok(ew)) bad = 1;
+    }
+  }
+  mgc_pdl_enter();                                       // the states were written at setup
+  const int i1 = min(i0 + TX, s.mx), j1 = min(j0 + TY, s.my);
   cplx r[SY];
+  unsigned plain = ~0u;                                  // bit q: r[q] is to be formed with FP64 instructions
   if constexpr (FXR) {
     // u as integers on the tile's exponent, each residual rounded to a double once
     __shared__ longlong2 T[(TY + 2) * PW];
@@ -124,42 +145,32 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
     }
     __syncthreads();
     const int eu = max(eu_s.x, eu_s.y);
-    const bool oku = fx_ok(eu);
-    tu.each(ux, [&](int row, int col, cplx z) {
-      T[row * PW + col + 1] = oku ? fx_int(z, eu - 1080) : as_raw(z);
-    });
-    __syncthreads();
-    const int i1 = min(i0 + TX, s.mx), j1 = min(j0 + TY, s.my);
-    if (oku) {
+    if (fx_tile_ok(eu_s)) {
+      tu.each(ux, [&](int row, int col, cplx z) { T[row * PW + col + 1] = fx_int(z, eu - 1080); });
+      __syncthreads();
+      plain = 0;
       const double sc = -fx_pow2(eu + x.ec - 2104);
       fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
 #pragma unroll
         for (int q = 0; q < SY; ++q) {
           const int row = q * WY + wy, j = j0 + row;
           if (i >= s.mx || j >= s.my) continue;
+          const longlong2* v = T + (row + 1) * PW + lane + 1;
           const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(
-              x, i, j, (size_t)j * s.mx + i, T + (row + 1) * PW + lane + 1, PW);
+              x, i, j, (size_t)j * s.mx + i, v, PW);
+          // f of 2^53 times the unit of a sum hides its rounding as well
+          if (!fx_kept(fx_lead5(v, PW)) && fx_exp(r[q]) < eu + x.ec - 1025) plain |= 1u << q;
           r[q] = cmk(fma(sc, (double)h.x, r[q].x), fma(sc, (double)h.y, r[q].y));
         }
       });
-    } else {
-      dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
-#pragma unroll
-        for (int q = 0; q < SY; ++q) {
-          const int row = q * WY + wy, j = j0 + row;
-          const longlong2* v = T + (row + 1) * PW + lane + 1;
-          if (i >= s.mx || j >= s.my) continue;
-          r[q] = residual_vals<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
-              s, i, j, j * s.mx + i, as_cplx(v[0]), as_cplx(v[-1]), as_cplx(v[1]), as_cplx(v[-PW]), as_cplx(v[PW]),
-              r[q]);
-        }
-      });
     }
-  } else {
-    dispatch_kinds(s, i0, min(i0 + TX, s.mx), j0, min(j0 + TY, s.my), [&](auto kx, auto ky, auto ir, auto dg) {
+  }
+  if (plain) {
+    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
 #pragma unroll
       for (int q = 0; q < SY; ++q) {
         const int j = j0 + q * WY + wy;
+        if (!(plain >> q & 1)) continue;
         r[q] = (i < s.mx && j < s.my)
                    ? residual_at<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
                          s, u, f, i, j)
@@ -167,24 +178,42 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
       }
     });
   }
-  int e = 0;
+  // the exponent of the residuals, and how far the largest products of any row (any column, by way of
+  // pmax) stay below the largest of its state and the tile
+  int e = 0, far = 0;
+  __syncwarp();
+  if constexpr (!FXR) __syncthreads();                   // xl, xr, pmax
 #pragma unroll
-  for (int q = 0; q < SY; ++q) e = max(e, fx_exp(r[q]));
-  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if (lane == 0) atomicMax(&eR, e);
-  for (int p = wy; p < 2 * NB; p += WY) {                // a warp converts one state's values of the tile
-    const int m = p >> 1, n = p & 1 ? TY : TX, k = (p & 1 ? j0 : i0) + lane, len = p & 1 ? s.my : s.mx;
-    const cplx w = lane < n && k < len ? __ldg((p & 1 ? c.wvphi : c.wphi) + (size_t)m * len + k) : cmk(0.0, 0.0);
-    const int ew = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(w));
-    if (lane < n) (p & 1 ? wr[m] : wl[m])[lane] = fx_limbs(w, ew, lane & 1);
-    if (lane == 0) {
-      (p & 1 ? ewr : ewl)[m] = ew;
-      if (!fx_ok(ew)) bad = 1;
+  for (int q = 0; q < SY; ++q) {
+    const int eq = fx_exp(r[q]);
+    e = max(e, eq);
+    if (__any_sync(0xffffffffu, eq != 0)) {
+#pragma unroll
+      for (int m = 0; m < NB; ++m) {
+        const int k = (int)__reduce_max_sync(0xffffffffu, (unsigned)(eq ? eq + xl[m][lane] : 0));
+        far = max(far, ewl[m] + 4096 - k);
+      }
     }
   }
+#pragma unroll
+  for (int m = 0; m < NB; ++m) {
+    int k = 0;
+#pragma unroll
+    for (int q = 0; q < SY; ++q) {
+      const int eq = fx_exp(r[q]);
+      if (eq) k = max(k, eq + xr[m][q * WY + wy]);
+    }
+    atomicMax(&pmax[m][lane], k);
+  }
+  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (lane == 0) atomicMax(&eR, e);
   __syncthreads();
   const int E = eR;
-  const bool ok = fx_ok(E) && !bad;
+  if (t < NB * TX) {
+    const int k = pmax[t / TX][t % TX];
+    if (k) far = max(far, ewr[t / TX] + 4096 - k);
+  }
+  const bool ok = !__syncthreads_or(!fx_ok(E) || bad || far > 4096 - E + FX_NEAR);
 #pragma unroll
   for (int q = 0; q < SY; ++q) {
     int4 v;
@@ -535,6 +564,8 @@ __global__ void __launch_bounds__(256) k_cccs_correct(int mx, int my, const C* _
 // exponent over the block, and aligns the 2 n_b products to the largest of their exponents by
 // shifting e^A and vphi on conversion; a node then takes 24 n_b integer multiply-adds and four
 // FP64 instructions (two conversions, two additions) against 8 n_b FP64 instructions.
+// A node whose products and value of u all lie below 2^-FX_NEAR of the tile's largest product takes
+// the FP64 multiply-adds, and so does a tile out of the integer range.
 // 1023^2, n_b = 3: 45.0 us with FP64 multiply-adds, 17.4 us so; 127^2: 9.6 and, with RT = 1, 4.5 us
 // (cold L2).
 template <int NB, int RT>
@@ -544,6 +575,7 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
   mgc_pdl_enter();
   constexpr int TYC = 8 * RT;
   __shared__ int4 col[2 * NB][32], row[2 * NB][TYC];     // [phi | e^B], [e^A | vphi]
+  __shared__ int xc[2 * NB][32], xr[2 * NB][TYC];        // their exponents
   __shared__ int ec[2 * NB], er[2 * NB];
   const int lane = threadIdx.x, wy = threadIdx.y;
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * TYC, i = i0 + lane, jt = j0 + wy * RT;
@@ -557,7 +589,9 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
     return k < len && (!side || lane < TYC) ? __ldg(a + (size_t)m * len + k) : cmk(0.0, 0.0);
   };
   for (int p = wy; p < 4 * NB; p += 8) {
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(value(p >> 1, p & 1)));
+    const int ex = fx_exp(value(p >> 1, p & 1)), e = (int)__reduce_max_sync(0xffffffffu, (unsigned)ex);
+    if (!(p & 1)) xc[p >> 1][lane] = ex;
+    else if (lane < TYC) xr[p >> 1][lane] = ex;
     if (lane == 0) (p & 1 ? er : ec)[p >> 1] = e;
   }
   __syncthreads();
@@ -568,17 +602,18 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
     E2 = max(E2, ec[p] + er[p]);
     ok = ok && fx_ok(ec[p]) && fx_ok(er[p]);
   }
+  const auto plain = [&](int r) {
+    const int j = jt + r;
+    cplx w = v[r];
+    for (int m = 0; m < NB; ++m) w = cfma(__ldg(phi + m * mx + i), __ldg(eA + m * my + j), w);
+    for (int l = 0; l < NB; ++l) w = cfma(__ldg(eB + l * mx + i), __ldg(vphi + l * my + j), w);
+    u[(size_t)j * mx + i] = w;
+  };
   if (!ok) {
     if (i >= mx) return;
 #pragma unroll
-    for (int r = 0; r < RT; ++r) {
-      const int j = jt + r;
-      if (j >= my) break;
-      cplx w = v[r];
-      for (int m = 0; m < NB; ++m) w = cfma(__ldg(phi + m * mx + i), __ldg(eA + m * my + j), w);
-      for (int l = 0; l < NB; ++l) w = cfma(__ldg(eB + l * mx + i), __ldg(vphi + l * my + j), w);
-      u[(size_t)j * mx + i] = w;
-    }
+    for (int r = 0; r < RT; ++r)
+      if (jt + r < my) plain(r);
     return;
   }
   for (int p = wy; p < 4 * NB; p += 8) {
@@ -597,6 +632,15 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
     if (jt + r >= my) break;
+    int k = fx_exp(v[r]) + 1023;
+    if (k < E2 - FX_NEAR) {
+#pragma unroll
+      for (int p = 0; p < 2 * NB; ++p) k = max(k, xc[p][lane] + xr[p][wy * RT + r]);
+      if (k < E2 - FX_NEAR) {
+        plain(r);
+        continue;
+      }
+    }
     FxSum re{0, 0}, im{0, 0};
 #pragma unroll
     for (int p = 0; p < 2 * NB; ++p) {

@@ -247,3 +247,36 @@ def test_parts_of_different_size(nu1, nu2):
     assert float((u.imag - v.imag).abs().max() / v.imag.abs().max()) <= 1e-13
     assert 0 in sv.integer_passes()[0]
     sv.close()
+
+
+# A spike of 2^60 where the states are 2^-22, in the corner of a tile of 32 columns and 32, 16 or 8 rows: 22
+# nodes on, its share of the projections has decayed (by 2^-2.4 a node and more at these energies), and the rest of
+# the row's (column's) projection comes from where the states are large.  The correction there
+# agrees with the oracle's to 1e-9, the bound of the parity tests, of the largest within 4 nodes.
+@pytest.mark.parametrize("n,E,rows", [(640, -800.0, 32), (512, -500.0, 16), (256, -200.0, 8)])
+@pytest.mark.parametrize("where", ["f", "u"])
+def test_correction_beside_a_spike(n, E, rows, where):
+    from oracle import mgcccs_oracle as O
+    prob = _problem(n, n, E=E)
+    levels = 5
+    so = O.Solver(O.params_from_problem(prob, levels=levels, n_b=1), prob.v1, prob.v2, prob.v12)
+    sv = _solver(prob, levels, n_b=1)
+    g = np.random.default_rng(n)
+    f, u = (g.standard_normal(prob.f.shape) + 1j * g.standard_normal(prob.f.shape) for _ in range(2))
+    f *= -E
+    a = int(18.0 * n / 30.0) // 32 * 32
+    if where == "f":
+        f[a, a] = 2.0 ** 60
+    else:
+        u[a, a] = 2.0 ** 60
+    ref = so.cccs(u, f) - u
+    ud = torch.as_tensor(u).to("cuda")
+    sv.cccs(ud, torch.as_tensor(f).to("cuda"))
+    d = torch.as_tensor(ud.cpu().numpy() - u - ref)
+    near = torch.nn.functional.max_pool2d(torch.as_tensor(ref).abs()[None], 9, 1, 4)[0]
+    near += torch.as_tensor(np.abs(u)) * 1e-6            # the rounding of u itself
+    own = slice(a + 22, a + 32)
+    assert bool((d.abs() <= 1e-9 * near)[:a // 2, own].all())
+    if rows == 32:
+        assert bool((d.abs() <= 1e-9 * near)[own, :a // 2].all())
+    sv.close()
