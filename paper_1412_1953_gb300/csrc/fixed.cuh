@@ -12,7 +12,8 @@
 // that shares E with one up to 16 times as large is still exact to its last bit.  It is held as two
 // limbs h 2^29 + l (|h| <= 2^28, |l| <= 2^28).  In a product (h h' 2^58 + (h l' + l h')
 // 2^29 + l l') the last term, below 2^-56 of the largest product, is dropped; the sums of the others
-// are exact in 64 bits for FX_TERMS complex terms, and are then rounded to a double once.  What is
+// are exact in 64 bits for FX_TERMS complex terms, and are then rounded to a double once.  (Gram-Schmidt
+// sums take 59 bits and FX_TERMS_59 terms: a quarter of the error at the same cost.)  What is
 // dropped must have no mean, or a long sum that cancels keeps it, so low limbs lie about zero and
 // conversions round without a preference.  (With low limbs of the operands' signs and cut conversions, a dot product of
 // 1023^2 skewed, nearly cancelling terms was 1e-17 to 1e-16 |v| |w| off its 64-bit value, and 2e-19
@@ -26,6 +27,11 @@
 
 constexpr int FX_MIN = 600, FX_MAX = 1446;       // biased exponents; a product's scale stays normal
 constexpr int FX_TERMS = 8;                      // complex terms between two roundings
+constexpr int FX_TERMS_59 = 6;                   // the same for limbs of 59 bits
+
+// How many powers of two below the largest operands' an integer sum's own largest term may lie: further
+// down its conversions could leave more than the roundings of FP64 instructions, which then take it.
+constexpr int FX_NEAR = 4;
 
 __device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ bool fx_ok(int E) { return (unsigned)(E - FX_MIN) <= (unsigned)(FX_MAX - FX_MIN); }
@@ -37,14 +43,18 @@ struct FxLimbs {
 // from position 7 + E - e on rounded, split at 2^29 with l in [-2^28, 2^28), and the sign multiplied in (on
 // the other integer pipe).  Ties, one in 2^d of the values that lose d bits, go away from zero, or
 // towards it with down = 1: long sums alternate it by lane, so that ties leave no mean either.
+// X = 2: 59 bits, split at 2^30.
+template <int X = 0>
 __device__ __forceinline__ FxLimbs fx_limbs(double x, int e, int E, int down = 0) {
+  static_assert(X == 0 || X == 2, "57 or 59 bits");
+  constexpr int S = 29 + X / 2;
   const int hi = __double2hiint(x), s = (hi >> 31) | 1;
   const unsigned lo = (unsigned)__double2loint(x);
   const unsigned a1 = __funnelshift_l(lo, ((unsigned)hi & 0xfffffu) | 0x100000u, 11), a0 = lo << 11;
   unsigned long long r;                                  // with a bit more, for rounding; 0 for E - e > 57
-  asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(((unsigned long long)a1 << 32 | a0) - down), "r"(E + 6 - e));
-  r += (1u << 29) + 1;
-  const int h = (int)(r >> 30), l = (int)(((unsigned)r & 0x3fffffffu) >> 1) - (1 << 28);
+  asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(((unsigned long long)a1 << 32 | a0) - down), "r"(E + 6 - X - e));
+  r += (1u << S) + 1;
+  const int h = (int)(r >> (S + 1)), l = (int)(((unsigned)r & ((2u << S) - 1)) >> 1) - (1 << (S - 1));
   return FxLimbs{h * s, l * s};
 }
 __device__ __forceinline__ FxLimbs fx_neg(FxLimbs a) { return FxLimbs{-a.h, -a.l}; }
@@ -78,8 +88,10 @@ __device__ __forceinline__ int4 fx_limbs(cplx z, int E, int down = 0) {
   return make_int4(x.h, x.l, y.h, y.l);
 }
 // acc + the sum of products with exponents that add up to E2, rounded; the sum is cleared.
+template <int X = 0>
 __device__ __forceinline__ double fx_flush(FxSum& s, int E2, double acc) {
-  const long long t = s.hh + ((s.mid + (1LL << 28)) >> 29);
+  constexpr int S = 29 + X / 2;
+  const long long t = s.hh + ((s.mid + (1LL << (S - 1))) >> S);
   s.hh = s.mid = 0;
-  return fma((double)t, __hiloint2double((E2 - 2100 + 1023) << 20, 0), acc);
+  return fma((double)t, __hiloint2double((E2 - 2100 - X + 1023) << 20, 0), acc);
 }

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
           const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(
               x, i, j, (size_t)j * s.mx + i, v, PW);
           // f of 2^53 times the unit of a sum hides its rounding as well
-          if (!fx_kept(fx_lead5(v, PW)) && fx_exp(r[q]) < eu + x.ec - 1025) plain |= 1u << q;
+          if (!fx_kept(fx_lead5(v, PW)) && fx_exp(r[q]) < eu + x.ec - 1021 - FX_NEAR) plain |= 1u << q;
           r[q] = cmk(fma(sc, (double)h.x, r[q].x), fma(sc, (double)h.y, r[q].y));
         }
       });

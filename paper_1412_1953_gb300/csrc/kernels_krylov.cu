@@ -86,14 +86,16 @@ __device__ __forceinline__ void copy_wait() {
 
 // The multi-dot: a block takes DG vectors, so that w is converted once for all of them, and a
 // warp DU x 32 consecutive points at a time, the last 32 of them with FP64 instructions, which
-// otherwise idle.  The exponents of w and of each vector are the largest met so far (a warp's
-// own); a larger one first rounds the sums held so far.  The sequence of chunks (w, then each
+// otherwise idle.  The exponents of w and of each vector are a warp's own and follow its chunks
+// (within D_SLACK; a new one first rounds the sums held so far).  A chunk in which no product comes
+// within 2^-FX_NEAR of the largest of both, so that its sum could be as small as what the conversions
+// leave, is summed with FP64 instructions.  The sequence of chunks (w, then each
 // vector, of one tile after another) is fetched DS - 1 chunks ahead.  About 90 instructions a
 // product and the 16 warps that 128 registers allow bound it.  1023^2, 12 vectors (12 and 1
 // of 16.7 MB read): 88.0 us with FP64 multiply-adds, 63 with 64-bit shifts of masked keys in the
 // conversion, 58 before the FP64 share, 53.7 with it, 56.9 us with conversions that leave no mean
 // (fixed.cuh; ties alternate by lane: 4 us of a pair), 3.5 TB/s.
-constexpr int DG = 4, DU = 4, DS = 4;
+constexpr int DG = 4, DU = 4, DS = 4, D_SLACK = 2;
 
 __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const cplx* __restrict__ V, long long ld,
                                                        const cplx* __restrict__ w, cplx* __restrict__ partial,
@@ -160,8 +162,8 @@ __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const
   }
   auto flush = [&](int i) {
     if (!fx_ok(Ew) || !fx_ok(E[i])) return;            // nothing was summed at these exponents
-    sum[i].x = fx_flush(re[i], Ew + E[i], sum[i].x);
-    sum[i].y = fx_flush(im[i], Ew + E[i], sum[i].y);
+    sum[i].x = fx_flush<2>(re[i], Ew + E[i], sum[i].x);
+    sum[i].y = fx_flush<2>(im[i], Ew + E[i], sum[i].y);
   };
 #pragma unroll
   for (int c = 0; c < DS - 1; ++c) fetch();
@@ -169,33 +171,38 @@ __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const
   for (; p0 < n; p0 += step) {
     cplx v[DU];
     const int et = take(v);
-    if (et > Ew || held + DU - 1 > FX_TERMS) {
+    if (et > Ew || et < Ew - D_SLACK || held + DU - 1 > FX_TERMS_59) {
 #pragma unroll
       for (int i = 0; i < DG; ++i) flush(i);
       held = 0;
-      Ew = max(Ew, et);
+      if (et > Ew || et < Ew - D_SLACK) Ew = et;
     }
     held += DU - 1;
     FxLimbs wx[DU - 1], wy[DU - 1];
+    int ew[DU - 1];
     const cplx wl = v[DU - 1];
 #pragma unroll
     for (int u = 0; u < DU - 1; ++u) {
-      wx[u] = fx_limbs(v[u].x, ex[u], Ew, lane & 1);
-      wy[u] = fx_limbs(v[u].y, ey[u], Ew, lane & 1);
+      wx[u] = fx_limbs<2>(v[u].x, ex[u], Ew, lane & 1);
+      wy[u] = fx_limbs<2>(v[u].y, ey[u], Ew, lane & 1);
+      ew[u] = max(ex[u], ey[u]);
     }
 #pragma unroll
     for (int i = 0; i < DG; ++i) {
       if (i >= nv) break;
       const int ei = take(v);
-      if (ei > E[i]) {
+      if (ei > E[i] || ei < E[i] - D_SLACK) {
         flush(i);
         E[i] = ei;
       }
-      if (fx_ok(Ew) && fx_ok(E[i])) {
+      int k = 0;
+#pragma unroll
+      for (int u = 0; u < DU - 1; ++u) k = max(k, max(ex[u], ey[u]) + ew[u]);
+      if (__any_sync(0xffffffffu, k >= Ew + E[i] - FX_NEAR) && fx_ok(Ew) && fx_ok(E[i])) {
 #pragma unroll
         for (int u = 0; u < DU - 1; ++u) {
-          const FxLimbs ax = fx_limbs(v[u].x, ex[u], E[i], lane & 1);
-          const FxLimbs ay = fx_limbs(v[u].y, ey[u], E[i], lane & 1);
+          const FxLimbs ax = fx_limbs<2>(v[u].x, ex[u], E[i], lane & 1);
+          const FxLimbs ay = fx_limbs<2>(v[u].y, ey[u], E[i], lane & 1);
           fx_mac(re[i], ax, wx[u]);
           fx_mac(re[i], ay, wy[u]);
           fx_mac(im[i], ax, wy[u]);

@@ -149,7 +149,6 @@ __device__ __forceinline__ int2 fx_max_exp(int2 e, cplx z) {
 }
 // Where one exponent will do for a tile of complex values with largest exponents e.x (real parts) and
 // e.y (imaginary parts): in range, and neither part more than 2^FX_NEAR below the other, unless it is zero.
-constexpr int FX_NEAR = 4;
 __device__ __forceinline__ bool fx_tile_ok(int2 e) {
   const int hi = max(e.x, e.y), lo = min(e.x, e.y);
   return fx_ok(hi) && (lo == 0 || hi - lo <= FX_NEAR);
@@ -161,7 +160,7 @@ __device__ __forceinline__ int fx_lead(longlong2 v) {
   const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
   return (x ^ x >> 31) | (y ^ y >> 31);
 }
-__device__ __forceinline__ bool fx_kept(int lead) { return lead >= 1 << (53 - 32); }
+__device__ __forceinline__ bool fx_kept(int lead) { return lead >= 1 << (57 - FX_NEAR - 32); }
 // of a node's five values
 __device__ __forceinline__ int fx_lead5(const longlong2* t, int pitch) {
   return fx_lead(t[0]) | fx_lead(t[-1]) | fx_lead(t[1]) | fx_lead(t[-pitch]) | fx_lead(t[pitch]);

@@ -280,3 +280,42 @@ def test_correction_beside_a_spike(n, E, rows, where):
     if rows == 32:
         assert bool((d.abs() <= 1e-9 * near)[own, :a // 2].all())
     sv.close()
+
+
+def _basis(kind, k, n, g):
+    """Vectors and w of ordinary size; entries of 2^45 and 2^-45 that meet the other's 2^-45 and 2^45; 2^-90 over
+    the vector in one and growing in the other; spikes of 2^60 in the vectors only; a step of 2^80 on the way."""
+    V, w = (g.standard_normal(s) + 1j * g.standard_normal(s) for s in ((k, n), (n,)))
+    q = np.arange(n)
+    if kind == "opposed":
+        s = np.where(q % 3 == 0, 2.0 ** 45, 2.0 ** -45)
+        V, w = V * s, w / s
+    elif kind == "slopes":
+        s = np.exp2(-90.0 * q / n)
+        V, w = V * s, w / s
+    elif kind == "spikes":
+        V[:, ::997] *= 2.0 ** 60
+        w[::997] = 0.0
+    elif kind == "step":
+        V[:, :n // 2] *= 2.0 ** 80
+        w[:n // 2] *= 2.0 ** -80
+    return V, w
+
+
+BASES = ["gauss", "opposed", "slopes", "spikes", "step"]
+
+
+# A dot product is good to a few units of 2^-53 of the sum of its terms' moduli, as FP64 multiply-adds give
+# it: some 30 partial sums a thread and block, and what a chunk's conversions leave, 2^-59 of its largest
+# operands' product a term, 12 units of its largest term's 2^-53 at the guard for 96 terms that all err one way.
+@pytest.mark.parametrize("nx,ny,k", [(32, 32, 5), (320, 256, 9), (1024, 512, 4)])
+@pytest.mark.parametrize("kind", BASES)
+def test_dots_term_by_term(nx, ny, k, kind):
+    prob = _problem(nx, ny)
+    sv = _solver(prob, 1 if nx == 32 else 5, krylov_restart=20)
+    V, w = _basis(kind, k, sv.n, np.random.default_rng(k))
+    h = torch.empty(k, dtype=torch.complex128, device="cuda")
+    sv.gs_dots(torch.as_tensor(V).to("cuda"), k, torch.as_tensor(w).to("cuda"), h)
+    terms = V.conj().astype(np.clongdouble) * w
+    assert (np.abs(h.cpu().numpy() - terms.sum(1)) <= 32 * 2.0 ** -53 * np.abs(terms).sum(1)).all()
+    sv.close()
