@@ -252,9 +252,12 @@ static_assert(MULTIDOT_SMEM >= 2 * DG * NT * (int)sizeof(double), "the block sum
 // The update w += sgn sum_i coef[i] V_i.  The coefficients are converted once per block, each
 // with its own exponent; a warp's sums over the vectors share the exponent of the largest product
 // met so far (at first that of the largest coefficient and the first vector).  A warp takes
-// UU x 32 points at a time and fetches the chunks (w, then each vector) ahead, as above.
+// UU x 32 points at a time and fetches the chunks (w, then each vector) ahead, as above.  Points whose
+// own products and w all lie below 2^-U_NEAR of that largest product are done again with FP64
+// instructions, from the arrays: 59 bits leave them fewer than a double has.
 // 1023^2, 11 vectors: 90.1 us with FP64 multiply-adds, 50.0 us now (UU = 4; 58 with UU = 2, which
 // is the faster at 255^2: 7.6 against 11.4 us, few tiles a warp), 4.4 TB/s.
+constexpr int U_NEAR = 6;
 constexpr int UF = 16;                                 // chunks in flight x points a lane
 
 template <int UU>
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
   for (int i = tid; i < k; i += NT) {
     const cplx q = cscal(sgn, coef[i]);
     const int ex = fx_exp(q.x), ey = fx_exp(q.y), e = max(ex, ey);
-    const FxLimbs x = fx_limbs(q.x, ex, e), y = fx_limbs(q.y, ey, e);
+    const FxLimbs x = fx_limbs<2>(q.x, ex, e), y = fx_limbs<2>(q.y, ey, e);
     sc[i] = q;
     sl[i] = make_int4(x.h, x.l, y.h, y.l);
     se[i] = e;
@@ -325,15 +328,19 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
     cplx acc[UU];
     FxSum re[UU], im[UU];
     take(acc);
+    int top[UU];                                       // exponent of a point's largest term
 #pragma unroll
-    for (int u = 0; u < UU; ++u) re[u] = im[u] = FxSum{0, 0};
+    for (int u = 0; u < UU; ++u) {
+      re[u] = im[u] = FxSum{0, 0};
+      top[u] = fx_exp(acc[u]) + 1023;
+    }
     int E2 = 0, held = 0;
     auto flush = [&]() {
       if (held == 0) return;
 #pragma unroll
       for (int u = 0; u < UU; ++u) {
-        acc[u].x = fx_flush(re[u], E2, acc[u].x);
-        acc[u].y = fx_flush(im[u], E2, acc[u].y);
+        acc[u].x = fx_flush<2>(re[u], E2, acc[u].x);
+        acc[u].y = fx_flush<2>(im[u], E2, acc[u].y);
       }
       held = 0;
     };
@@ -349,7 +356,7 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
       }
       const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)e), ec = se[i];
       if (fx_ok(ev) && fx_ok(ec)) {
-        if (ev + ec > E2 || held == FX_TERMS) {
+        if (ev + ec > E2 || held == FX_TERMS_59) {
           flush();
           // the first time: room for the largest coefficient
           E2 = max(E2, i == 0 && fx_ok(smax) ? ev + smax : ev + ec);
@@ -360,7 +367,8 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
         const int E = E2 - ec;
 #pragma unroll
         for (int u = 0; u < UU; ++u) {
-          const FxLimbs x = fx_limbs(v[u].x, ex[u], E), y = fx_limbs(v[u].y, ey[u], E);
+          const FxLimbs x = fx_limbs<2>(v[u].x, ex[u], E), y = fx_limbs<2>(v[u].y, ey[u], E);
+          top[u] = max(top[u], max(ex[u], ey[u]) + ec);
           fx_mac(re[u], x, cx);
           fx_mac(re[u], y, my);
           fx_mac(im[u], y, cx);
@@ -372,6 +380,21 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
       }
     }
     flush();
+    unsigned low = 0;
+#pragma unroll
+    for (int u = 0; u < UU; ++u)
+      if (p0 + lane + 32 * u < n && top[u] < E2 - U_NEAR) low |= 1u << u;
+    if (low) {
+#pragma unroll
+      for (int u = 0; u < UU; ++u) {
+        if (!(low >> u & 1)) continue;
+        const long long p = p0 + lane + 32 * u;
+        cplx a = w[p];
+#pragma unroll 1
+        for (int i = 0; i < k; ++i) a = cfma(sc[i], __ldg(V + i * ld + p), a);
+        acc[u] = a;
+      }
+    }
 #pragma unroll
     for (int u = 0; u < UU; ++u)
       if (p0 + lane + 32 * u < n) {

@@ -319,3 +319,25 @@ def test_dots_term_by_term(nx, ny, k, kind):
     terms = V.conj().astype(np.clongdouble) * w
     assert (np.abs(h.cpu().numpy() - terms.sum(1)) <= 32 * 2.0 ** -53 * np.abs(terms).sum(1)).all()
     sv.close()
+
+
+# An entry of the update is good to the roundings of its own 2 k multiply-adds a part, as FP64 instructions
+# give it, and as much again for k conversions at the guard.
+@pytest.mark.parametrize("nx,ny,k", [(32, 32, 5), (320, 256, 9), (1024, 512, 4)])
+@pytest.mark.parametrize("kind", BASES + ["coefficients"])
+def test_update_entry_by_entry(nx, ny, k, kind):
+    prob = _problem(nx, ny)
+    sv = _solver(prob, 1 if nx == 32 else 5, krylov_restart=20)
+    g = np.random.default_rng(k)
+    V, w = _basis(kind, k, sv.n, g)
+    c = g.standard_normal(k) + 1j * g.standard_normal(k)
+    if kind == "coefficients":                       # the largest coefficient on a vector that is zero in places
+        c *= np.exp2(-30.0 * np.arange(k))
+        V[0, :sv.n // 2] = 0.0
+        w[:sv.n // 2] *= 2.0 ** -60
+    wd = torch.as_tensor(w).to("cuda")
+    sv.gs_update(torch.as_tensor(V).to("cuda"), k, torch.as_tensor(c).to("cuda"), wd)
+    terms = c[:, None].astype(np.clongdouble) * V
+    size = np.abs(w) + np.abs(terms).sum(0)
+    assert (np.abs(wd.cpu().numpy() - (w - terms.sum(0))) <= (8 * k + 16) * 2.0 ** -53 * size).all()
+    sv.close()
