@@ -184,11 +184,10 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
  * setup of h (0 normally), or -1 for a NULL handle. */
 int mgcccs_eig_fallbacks(mgcccs_t h);
 
-/* Which of h's complex128 passes multiply on the integer pipes, as setup chose from the
+/* Which levels' complex128 passes multiply on the integer pipes, as setup chose from the
  * operator's coefficients: bit l of *levels for the passes of level l (and for l = 0 the
- * operator and the CCCS residual), *coarsest for the block-reduction coarsest solve.  Either
- * may be NULL.  No device work.  EINVAL for a NULL handle. */
-int mgcccs_integer_passes(mgcccs_t h, unsigned* levels, int* coarsest);
+ * operator and the CCCS residual).  No device work.  EINVAL for a NULL pointer. */
+int mgcccs_integer_passes(mgcccs_t h, unsigned* levels);
 
 /* Solve drivers for mgcccs_set_solve_driver. */
 enum { MGCCCS_DRIVER_GRAPH = 0, MGCCCS_DRIVER_HOST = 1 };

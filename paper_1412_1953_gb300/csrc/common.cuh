@@ -619,13 +619,9 @@ cudaError_t launch_bpcr_setup(const StencilView& s, cplx* fac, cplx* scratch, in
 size_t block_inverse_scratch(int mx, int my);
 cudaError_t launch_block_inverse(const StencilView& s, cplx* scratch, cplx* Ainv, int* status,
                                  unsigned long long* worst, cudaStream_t st);
-size_t bpcr_exponents(int my);                               // ints for launch_bpcr_split
-cudaError_t launch_bpcr_split(int mx, int my, cplx* fac, int* e, int* bad, cudaStream_t st);
-// u = A_c^{-1} f through the factors (exps: those of the split factors, or null); buf holds 2 mx my
-// complex entries
+// u = A_c^{-1} f through the factors; buf holds 2 mx my complex entries
 template <class C>
-cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const int* exps, const C* f, C* u, cplx* buf,
-                              cudaStream_t st);
+cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const C* f, C* u, cplx* buf, cudaStream_t st);
 // eig: all m eigenvalues (eig_aberth, or launch_qr_spectrum when that did not converge)
 cudaError_t launch_bound_states(int m, const cplx* west, const cplx* east, const cplx* v, const cplx* w, int nb,
                                 cplx* lam, cplx* phi, cplx* scratch, int* status, cudaStream_t st, const cplx* eig);

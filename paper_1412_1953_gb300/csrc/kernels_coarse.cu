@@ -24,7 +24,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "fixed.cuh"
+#include "common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -323,147 +323,11 @@ __global__ void __launch_bounds__(32 * BP_KQ) k_bp_level(int nr, int m, int s, c
   }
 }
 
-// The same with the factors as limbs (fixed.cuh), each block on its own exponent (eA, eG, eD: per
-// block row; 0 for a block of zeros).  The three products share the exponent of the largest by
-// shifting b's rows on conversion.  Per thread 24 complex products, 96 FP64 instructions of 64
-// cycles before, are 288 integer multiply-adds of 4; FP64 remains for the conversion of a thread's
-// sum and for adding the warps' sums.  63 x 63, per level with cold L2: 9.4 us with FP64
-// instructions, 6.1 us so.  Rows of b out of the integer range are multiplied in FP64 with the
-// factors' values restored from their limbs.
-__device__ __forceinline__ cplx limbs_value(int4 f, int e) {
-  const double sc = __hiloint2double((e - 1079 + 1023) << 20, 0);
-  return cmk(sc * (double)((long long)f.x * (1LL << 29) + f.y), sc * (double)((long long)f.z * (1LL << 29) + f.w));
-}
-
 template <class CI, class CO>
-__global__ void __launch_bounds__(32 * BP_KQ) k_bp_level_fx(int nr, int m, int s, const int4* __restrict__ AT,
-                                                            const int4* __restrict__ GT, const int4* __restrict__ DT,
-                                                            const int* __restrict__ eA, const int* __restrict__ eG,
-                                                            const int* __restrict__ eD, const CI* __restrict__ b,
-                                                            CO* __restrict__ out) {
-  __shared__ cplx part[BP_KQ][32];
-  __shared__ cplx bs[3][BP_KQ * BP_KC];
-  __shared__ int4 bl[3][BP_KQ * BP_KC];
-  __shared__ int eb[3];
-  const int j = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int i = blockIdx.y * 32 + lane;
-  const bool has[3] = {j - s >= 0, DT != nullptr, j + s < nr};
-  const size_t mm = (size_t)m * m;
-  const int ii = i < m ? i : 0, k0 = w * BP_KC;
-  int4 f[3][BP_KC];                                      // written at setup: read ahead of the wait
-  const int4* const F[3] = {AT, DT, GT};
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int q = 0; q < BP_KC; ++q) {
-      const int k = k0 + q;
-      f[r][q] = k < m && has[r] ? __ldg(F[r] + j * mm + (size_t)k * m + ii) : make_int4(0, 0, 0, 0);
-    }
-  const int ef[3] = {has[0] ? eA[j] : 0, has[1] ? eD[j] : 0, has[2] ? eG[j] : 0};
-  if (t < 3) eb[t] = 0;
-  for (int q = t; q < 3 * BP_KQ * BP_KC; q += 32 * BP_KQ) (&bs[0][0])[q] = cmk(0.0, 0.0);
-  __syncthreads();
-  mgc_pdl_enter();
-  const int r = t / m, k = t - r * m, jr = j + (r - 1) * s;
-  const bool mine = t < 3 * m && jr >= 0 && jr < nr;
-  cplx v = cmk(0.0, 0.0);
-  if (mine) {
-    v = to_c128(b[(size_t)jr * m + k]);
-    bs[r][k] = v;
-    atomicMax(&eb[r], fx_exp(v));
-  }
-  __syncthreads();
-  int E2 = 0;
-  bool ok = true;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    if (!has[q] || ef[q] == 0) continue;
-    ok = ok && fx_ok(eb[q]);
-    E2 = max(E2, ef[q] + eb[q]);
-  }
-  if (ok && t < 3 * BP_KQ * BP_KC) {
-    // alpha and gamma are subtracted
-    const int r2 = t / (BP_KQ * BP_KC), k2 = t - r2 * BP_KQ * BP_KC;
-    const cplx x = bs[r2][k2];
-    bl[r2][k2] = fx_limbs(r2 == 1 ? x : cneg(x), E2 - ef[r2], k2 & 1);
-  }
-  __syncthreads();
-  cplx acc = cmk(0.0, 0.0);
-  if (ok) {
-    FxSum re{0, 0}, im{0, 0};
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      if (!has[q] || ef[q] == 0) continue;
-#pragma unroll
-      for (int c = 0; c < BP_KC; ++c) fx_cmac(re, im, f[q][c], bl[q][k0 + c]);
-      fx_carry(re);
-      fx_carry(im);
-    }
-    if (E2 > 0) acc = cmk(fx_flush(re, E2, 0.0), fx_flush(im, E2, 0.0));
-  } else {
-    for (int q = 0; q < 3; ++q) {
-      if (!has[q] || ef[q] == 0) continue;
-#pragma unroll
-      for (int c = 0; c < BP_KC; ++c) {
-        const cplx y = limbs_value(f[q][c], ef[q]), x = bs[q][k0 + c];
-        acc = q == 1 ? cfma(y, x, acc) : cfms(y, x, acc);
-      }
-    }
-  }
-  part[w][lane] = acc;
-  __syncthreads();
-  if (t < 64) {                                          // component t >> 5 of lane
-    const double* p = reinterpret_cast<const double*>(&part[0][lane]) + (t >> 5);
-    double tot = p[0];
-#pragma unroll
-    for (int q = 1; q < BP_KQ; ++q) tot += p[q * 64];
-    if (i < m) {
-      if (!DT) tot += t < 32 ? bs[1][i].x : bs[1][i].y;
-      reinterpret_cast<typename CT<CO>::R*>(out + (size_t)j * m + i)[t >> 5] = (typename CT<CO>::R)tot;
-    }
-  }
-}
-
-// Exponents of the factor blocks (one block each), and whether all are in the integer range.
-__global__ void __launch_bounds__(256) k_bp_exponents(int mm, const cplx* __restrict__ fac, int* __restrict__ e,
-                                                      int* __restrict__ bad) {
-  __shared__ int es;
-  if (threadIdx.x == 0) es = 0;
-  __syncthreads();
-  int m = 0;
-  for (int q = threadIdx.x; q < mm; q += 256) m = max(m, fx_exp(fac[(size_t)blockIdx.x * mm + q]));
-  atomicMax(&es, m);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    e[blockIdx.x] = es;
-    if (es != 0 && !fx_ok(es)) *bad = 1;
-  }
-}
-// The factors as limbs, in place, unless one is out of range.
-__global__ void __launch_bounds__(256) k_bp_split(int mm, cplx* fac, const int* __restrict__ e,
-                                                  const int* __restrict__ bad) {
-  if (*bad) return;
-  const int E = e[blockIdx.x];
-  for (int q = threadIdx.x; q < mm; q += 256) {
-    cplx* p = fac + (size_t)blockIdx.x * mm + q;
-    *reinterpret_cast<int4*>(p) = E == 0 ? make_int4(0, 0, 0, 0) : fx_limbs(*p, E);
-  }
-}
-
-// The level of factor matrices a, g (and d) of the solve: indices into the factors and exponents.
-template <class CI, class CO>
-cudaError_t launch_level(int nr, int m, int s, const cplx* fac, const int* exps, int a, int g, int d, const CI* b,
-                         CO* out, cudaStream_t st) {
-  const size_t B = (size_t)nr * m * m;
-  const dim3 grid(nr, (m + 31) / 32), block(32 * BP_KQ);
-  if (exps) {
-    auto mat = [&](int q) { return q < 0 ? nullptr : reinterpret_cast<const int4*>(fac + q * B); };
-    auto ex = [&](int q) { return q < 0 ? nullptr : exps + (size_t)q * nr; };
-    return mgc_launch(k_bp_level_fx<CI, CO>, grid, block, 0, st, nr, m, s, mat(a), mat(g), mat(d), ex(a), ex(g), ex(d),
-                      b, out);
-  }
-  auto mat = [&](int q) { return q < 0 ? nullptr : fac + q * B; };
-  return mgc_launch(k_bp_level<CI, CO>, grid, block, 0, st, nr, m, s, mat(a), mat(g), mat(d), b, out);
+cudaError_t launch_level(int nr, int m, int s, const cplx* AT, const cplx* GT, const cplx* DT, const CI* b, CO* out,
+                         cudaStream_t st) {
+  return mgc_launch(k_bp_level<CI, CO>, dim3(nr, (m + 31) / 32), dim3(32 * BP_KQ), 0, st, nr, m, s, AT, GT, DT, b,
+                    out);
 }
 
 }  // namespace
@@ -670,38 +534,28 @@ cudaError_t launch_block_inverse(const StencilView& s, cplx* scratch, cplx* Ainv
   return cudaGetLastError();
 }
 
-size_t bpcr_exponents(int my) { return (size_t)(2 * bp_levels(my) + 1) * my; }
-
-// The factors of launch_bpcr_setup as limbs in place, with their blocks' exponents in e; *bad (cleared
-// by the caller) is set, and the factors left, if one is out of the integer range.
-cudaError_t launch_bpcr_split(int mx, int my, cplx* fac, int* e, int* bad, cudaStream_t st) {
-  const int blocks = (int)bpcr_exponents(my), mm = mx * mx;
-  k_bp_exponents<<<blocks, 256, 0, st>>>(mm, fac, e, bad);
-  k_bp_split<<<blocks, 256, 0, st>>>(mm, fac, e, bad);
-  return cudaGetLastError();
-}
-
 template <class C>
-cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const int* exps, const C* f, C* u, cplx* buf,
-                              cudaStream_t st) {
+cudaError_t launch_bpcr_solve(int mx, int my, const cplx* fac, const C* f, C* u, cplx* buf, cudaStream_t st) {
   const int m = mx, nr = my;
   if (!bpcr_fits(m, nr)) return cudaErrorInvalidValue;
-  const int Lp = bp_levels(nr), D = 2 * Lp;
-  if (Lp == 0) return launch_level<C, C>(nr, m, 1, fac, exps, -1, -1, D, f, u, st);
+  const size_t B = (size_t)nr * m * m;
+  const int Lp = bp_levels(nr);
+  const cplx* DfT = fac + (size_t)2 * Lp * B;
+  if (Lp == 0) return launch_level<C, C>(nr, m, 1, nullptr, nullptr, DfT, f, u, st);
   cplx* pb[2] = {buf, buf + (size_t)nr * m};
   cudaError_t e = cudaSuccess;
   for (int l = 0, s = 1; l < Lp && e == cudaSuccess; ++l, s *= 2) {
-    const int a = 2 * l, g = 2 * l + 1;
+    const cplx* AT = fac + (size_t)(2 * l) * B;
+    const cplx* GT = fac + (size_t)(2 * l + 1) * B;
     const bool first = l == 0, last = l == Lp - 1;
-    if (first && last) e = launch_level<C, C>(nr, m, s, fac, exps, a, g, D, f, u, st);
-    else if (first) e = launch_level<C, cplx>(nr, m, s, fac, exps, a, g, -1, f, pb[0], st);
-    else if (last) e = launch_level<cplx, C>(nr, m, s, fac, exps, a, g, D, pb[(l - 1) & 1], u, st);
-    else e = launch_level<cplx, cplx>(nr, m, s, fac, exps, a, g, -1, pb[(l - 1) & 1], pb[l & 1], st);
+    if (first && last) e = launch_level<C, C>(nr, m, s, AT, GT, DfT, f, u, st);
+    else if (first) e = launch_level<C, cplx>(nr, m, s, AT, GT, nullptr, f, pb[0], st);
+    else if (last) e = launch_level<cplx, C>(nr, m, s, AT, GT, DfT, pb[(l - 1) & 1], u, st);
+    else e = launch_level<cplx, cplx>(nr, m, s, AT, GT, nullptr, pb[(l - 1) & 1], pb[l & 1], st);
   }
   return e;
 }
 
-template cudaError_t launch_bpcr_solve<double2>(int, int, const cplx*, const int*, const double2*, double2*, cplx*,
+template cudaError_t launch_bpcr_solve<double2>(int, int, const cplx*, const double2*, double2*, cplx*,
                                                 cudaStream_t);
-template cudaError_t launch_bpcr_solve<float2>(int, int, const cplx*, const int*, const float2*, float2*, cplx*,
-                                               cudaStream_t);
+template cudaError_t launch_bpcr_solve<float2>(int, int, const cplx*, const float2*, float2*, cplx*, cudaStream_t);

@@ -42,8 +42,6 @@ struct mgcccs_handle {
   cplx* aug;
   int coarse_bp;           // 1: larger coarsest grid, solved by block cyclic reduction
   cplx *bp_fac, *bp_scr, *bp_buf;
-  int* bp_exp;             // the factors are limbs on these exponents (null: they are values)
-  int* bp_exp_buf;
   int nb;
   cplx *lam, *mu, *phi, *vphi, *wphi, *wvphi, *VA, *VB;
   CRSystem crA, crB;       // channel A (along y, x bound states), channel B (along x)
@@ -182,7 +180,6 @@ void layout(mgcccs_handle* h, Carver& cv) {
     h->bp_fac = cv.take<cplx>(bpcr_factor_entries(c.mx, c.my));
     h->bp_scr = cv.take<cplx>(bpcr_scratch_entries(c.mx, c.my));
     h->bp_buf = cv.take<cplx>((size_t)2 * h->nc);
-    h->bp_exp_buf = cv.take<int>(bpcr_exponents(c.my));
   } else {
     h->Ainv = cv.take<cplx>((size_t)h->nc * h->nc);
     h->aug = cv.take<cplx>(std::max(coarse_inverse_scratch(h->nc), block_inverse_scratch(c.mx, c.my)));
@@ -353,16 +350,13 @@ int read_status(mgcccs_handle* h) {
 // all rows takes its place.
 constexpr double MGC_INVERSE_RESIDUAL = 1e-11;
 int coarse_inverse_check(mgcccs_handle* h) {
+  if (h->coarse_bp) return MGCCCS_OK;
   struct {
     int pivot, pad;
     double worst;
   } c;
   MGC_CUDA(cudaMemcpyAsync(&c, h->status + 4, sizeof(c), cudaMemcpyDeviceToHost, h->st));
   MGC_CUDA(cudaStreamSynchronize(h->st));
-  if (h->coarse_bp) {
-    h->bp_exp = c.pivot ? nullptr : h->bp_exp_buf;       // here: a factor out of the integer range
-    return MGCCCS_OK;
-  }
   if (c.pivot == 0 && c.worst <= MGC_INVERSE_RESIDUAL) return MGCCCS_OK;
   MGC_LAUNCH(launch_coarse_inverse(h->lv[h->L - 1].sv, h->aug, h->Ainv, h->status, h->st));
   return MGCCCS_OK;
@@ -446,10 +440,7 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
     if (b.fx.on) h->launches += 6;
   }
   if (h->coarse_bp) {
-    const LevelBufs& c = h->lv[h->L - 1];
-    MGC_LAUNCH(launch_bpcr_setup(c.sv, h->bp_fac, h->bp_scr, h->status, st));
-    MGC_LAUNCH(launch_bpcr_split(c.mx, c.my, h->bp_fac, h->bp_exp_buf, h->status + 4, st));
-    h->launches += 1;
+    MGC_LAUNCH(launch_bpcr_setup(h->lv[h->L - 1].sv, h->bp_fac, h->bp_scr, h->status, st));
   } else {
     // its zero pivots go to status[4], its largest residual to status[6..7] (read at the end)
     MGC_LAUNCH(launch_block_inverse(h->lv[h->L - 1].sv, h->aug, h->Ainv, h->status + 4,
@@ -559,7 +550,7 @@ const CCViewT<float2>& cc_view<float2>(mgcccs_handle* h) { return h->cc32; }
 template <class C>
 cudaError_t coarse_solve(mgcccs_handle* h, const C* f, C* u, cudaStream_t st) {
   const LevelBufs& c = h->lv[h->L - 1];
-  if (h->coarse_bp) return launch_bpcr_solve<C>(c.mx, c.my, h->bp_fac, h->bp_exp, f, u, h->bp_buf, st);
+  if (h->coarse_bp) return launch_bpcr_solve<C>(c.mx, c.my, h->bp_fac, f, u, h->bp_buf, st);
   return launch_coarse_solve(h->nc, h->Ainv, f, u, st);
 }
 
@@ -1824,13 +1815,10 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
 
 int mgcccs_eig_fallbacks(mgcccs_t h) { return h ? h->eig_fallbacks : -1; }
 
-int mgcccs_integer_passes(mgcccs_t h, unsigned* levels, int* coarsest) {
-  if (!h) return MGCCCS_EINVAL;
-  if (levels) {
-    *levels = 0;
-    for (int l = 0; l < h->L; ++l) *levels |= h->lv[l].fx.on ? 1u << l : 0u;
-  }
-  if (coarsest) *coarsest = h->coarse_bp && h->bp_exp;
+int mgcccs_integer_passes(mgcccs_t h, unsigned* levels) {
+  if (!h || !levels) return MGCCCS_EINVAL;
+  *levels = 0;
+  for (int l = 0; l < h->L; ++l) *levels |= h->lv[l].fx.on ? 1u << l : 0u;
   return MGCCCS_OK;
 }
 
