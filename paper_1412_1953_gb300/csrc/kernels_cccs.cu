@@ -413,7 +413,7 @@ k_channel_solve(CRSystem SA, CRSystem SB) {
     // the factors were written at setup: fetch them ahead of the wait for the projections
     if (in_smem) {
       for (size_t e = tid; e < len; e += CR_THREADS) copy_async16(X + R * NB + e, F + e);
-    } else if (tid == 0) {
+    } else if (tid == 0 && len > 0) {                // no factors where a CTA owns one row
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(F), "r"((unsigned)(len * sizeof(cplx)))
                    : "memory");
     }
