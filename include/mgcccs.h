@@ -184,11 +184,6 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
  * setup of h (0 normally), or -1 for a NULL handle. */
 int mgcccs_eig_fallbacks(mgcccs_t h);
 
-/* Which levels' complex128 passes multiply on the integer pipes, as setup chose from the
- * operator's coefficients: bit l of *levels for the passes of level l (and for l = 0 the
- * operator and the CCCS residual).  No device work.  EINVAL for a NULL pointer. */
-int mgcccs_integer_passes(mgcccs_t h, unsigned* levels);
-
 /* Solve drivers for mgcccs_set_solve_driver. */
 enum { MGCCCS_DRIVER_GRAPH = 0, MGCCCS_DRIVER_HOST = 1 };
 int mgcccs_set_solve_driver(mgcccs_t h, int driver);
@@ -239,10 +234,7 @@ int mgcccs_batch_solve(mgcccs_t* handles, int count, mgcccs_c128* const* u, cons
  * complex64 and z is its exact widening.  Async. */
 int mgcccs_precond_apply(mgcccs_t h, mgcccs_c128* z, const mgcccs_c128* r);
 
-/* y = (H-E)x on the fine level (Eq. (11)); x, y: device, distinct.  Async.  An entry of y is
- * within 2^-48 of the sum of the moduli of its five terms, however large the entries of x beside them
- * (FP64 instructions give 2^-49); where the real and imaginary parts of x differ in size
- * throughout, each part of y within that of its own terms. */
+/* y = (H-E)x on the fine level (Eq. (11)); x, y: device, distinct.  Async. */
 int mgcccs_matvec(mgcccs_t h, const mgcccs_c128* x, mgcccs_c128* y);
 
 /* r = f - (H-E)u on the fine level (Eq. (11)); if norm2 is not NULL the

@@ -585,8 +585,9 @@ __host__ __device__ constexpr bool cr_pack_in_smem(int m, int nb, bool shared_gp
 int cc_tiles_x(int mx);
 int cc_tile_rows(int mx, int my);   // rows per warp of a CCCS tile (8 warps): 1, 2 or 4
 int cc_tiles_y(int mx, int my);
-cudaError_t launch_residual_project(const StencilView32& s, const CCView32& c, const float2* u, const float2* f,
-                                    cudaStream_t st);   // complex128: stencil_fx.cuh
+template <class C>
+cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f,
+                                    cudaStream_t st);
 template <class C>
 cudaError_t launch_reduce_projections(const CCViewT<C>& c, cudaStream_t st);
 cudaError_t channel_solve_prepare(int nb, int mA, int mB);

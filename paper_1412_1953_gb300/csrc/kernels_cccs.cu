@@ -16,7 +16,7 @@
 
 #include <mutex>
 
-#include "stencil_fx.cuh"
+#include "fixed.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -89,19 +89,15 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
 // The same in complex128 with the projections on the integer pipes (fixed.cuh): the tile's
 // residuals share one exponent, and so do each state's weighted values over the tile's columns
 // (rows).  A residual's 2 n_b complex products then cost 24 n_b integer multiply-adds, 96 n_b
-// cycles of a quarter of an SM, against 8 n_b FP64 instructions, 512 n_b cycles.  FXR: the
-// residuals are formed from u on the tile's exponent as well (stencil_fx.cuh); of the tile heights
-// only 4 rows a warp, whose grids are large enough for it.  A residual whose terms all lie below
-// 2^53 units takes FP64 instructions, and so does a tile with a row's (column's) projection whose
-// products all lie below 2^-FX_NEAR of the tile's largest: 3 to 7 % of the tiles of 32 rows in a
-// solve at 512^2, up to 19 % at 256^2.  1023^2, n_b = 3, cold L2: 76.6 us with
-// FP64 instructions, 41.2 us with integer projections, 36.2 us with both; 127^2: 19.2 us in tiles of 32 rows (16 blocks), 7.4
-// us in tiles of 8 (cold L2).
-template <int NB, int SY, bool FXR>
-__global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CCView c, const cplx* __restrict__ u,
+// cycles of a quarter of an SM, against 8 n_b FP64 instructions, 512 n_b cycles.  A tile with a row's
+// (column's) projection whose products all lie below 2^-FX_NEAR of the tile's largest takes the FP64
+// instructions: 3 to 7 % of the tiles of 32 rows in a solve at 512^2, up to 19 % at 256^2.  1023^2,
+// n_b = 3, cold L2: 76.6 us with FP64 instructions, 41.8 us with integer projections; 127^2: 19.2 us in tiles of 32
+// rows (16 blocks), 7.4 us in tiles of 8.
+template <int NB, int SY>
+__global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilView s, CCView c, const cplx* __restrict__ u,
                                                                 const cplx* __restrict__ f) {
-  const StencilView& s = x.s;
-  constexpr int TY = SY * WY, PW = TX + 2;
+  constexpr int TY = SY * WY;
   __shared__ int4 R[TY][TX + 1];                         // limbs, or the values themselves
   __shared__ int4 wl[NB][TX], wr[NB][TY];
   __shared__ int xl[NB][TX], xr[NB][TY];                 // exponents of the weighted values
@@ -126,63 +122,21 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilFx x, CC
     }
   }
   mgc_pdl_enter();                                       // the states were written at setup
-  const int i1 = min(i0 + TX, s.mx), j1 = min(j0 + TY, s.my);
   cplx r[SY];
-  unsigned plain = ~0u;                                  // bit q: r[q] is to be formed with FP64 instructions
-  if constexpr (FXR) {
-    // u as integers on the tile's exponent, each residual rounded to a double once
-    __shared__ longlong2 T[(TY + 2) * PW];
-    __shared__ int2 eu_s;
-    if (t == 0) eu_s = make_int2(0, 0);
-    __syncthreads();
-    const auto ux = [](int q) { return q ? TX : -1; };
-    TileShare<WY, TY + 2, 2> tu;
-    block_exponent(tu.load(u, s.mx, s.my, i0, j0 - 1, ux), &eu_s);
+  dispatch_kinds(s, i0, min(i0 + TX, s.mx), j0, min(j0 + TY, s.my), [&](auto kx, auto ky, auto ir, auto dg) {
 #pragma unroll
     for (int q = 0; q < SY; ++q) {
       const int j = j0 + q * WY + wy;
-      r[q] = i < s.mx && j < s.my ? __ldg(f + (size_t)j * s.mx + i) : cmk(0.0, 0.0);
+      r[q] = (i < s.mx && j < s.my)
+                 ? residual_at<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
+                       s, u, f, i, j)
+                 : cmk(0.0, 0.0);
     }
-    __syncthreads();
-    const int eu = max(eu_s.x, eu_s.y);
-    if (fx_tile_ok(eu_s)) {
-      tu.each(ux, [&](int row, int col, cplx z) { T[row * PW + col + 1] = fx_int(z, eu - 1080); });
-      __syncthreads();
-      plain = 0;
-      const double sc = -fx_pow2(eu + x.ec - 2104);
-      fx_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto rd) {
-#pragma unroll
-        for (int q = 0; q < SY; ++q) {
-          const int row = q * WY + wy, j = j0 + row;
-          if (i >= s.mx || j >= s.my) continue;
-          const longlong2* v = T + (row + 1) * PW + lane + 1;
-          const longlong2 h = fx_operator<decltype(kx)::value, decltype(ky)::value, decltype(rd)::value, 3>(
-              x, i, j, (size_t)j * s.mx + i, v, PW);
-          // f of 2^53 times the unit of a sum hides its rounding as well
-          if (!fx_kept(fx_lead5(v, PW)) && fx_exp(r[q]) < eu + x.ec - 1021 - FX_NEAR) plain |= 1u << q;
-          r[q] = cmk(fma(sc, (double)h.x, r[q].x), fma(sc, (double)h.y, r[q].y));
-        }
-      });
-    }
-  }
-  if (plain) {
-    dispatch_kinds(s, i0, i1, j0, j1, [&](auto kx, auto ky, auto ir, auto dg) {
-#pragma unroll
-      for (int q = 0; q < SY; ++q) {
-        const int j = j0 + q * WY + wy;
-        if (!(plain >> q & 1)) continue;
-        r[q] = (i < s.mx && j < s.my)
-                   ? residual_at<decltype(kx)::value, decltype(ky)::value, decltype(ir)::value, decltype(dg)::value>(
-                         s, u, f, i, j)
-                   : cmk(0.0, 0.0);
-      }
-    });
-  }
+  });
   // the exponent of the residuals, and how far the largest products of any row (any column, by way of
   // pmax) stay below the largest of its state and the tile
   int e = 0, far = 0;
-  __syncwarp();
-  if constexpr (!FXR) __syncthreads();                   // xl, xr, pmax
+  __syncthreads();                                       // xl, xr, pmax
 #pragma unroll
   for (int q = 0; q < SY; ++q) {
     const int eq = fx_exp(r[q]);
@@ -654,27 +608,18 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
   }
 }
 
-template <int NB>
-cudaError_t rp_launch(const StencilFx& s, const CCView& c, const cplx* u, const cplx* f, cudaStream_t st) {
-  auto go = [&](auto kern) {
-    return mgc_launch(kern, dim3(cc_tiles_x(s.s.mx), cc_tiles_y(s.s.mx, s.s.my)), dim3(TX, WY), 0, st, s, c, u, f);
-  };
-  switch (cc_tile_rows(s.s.mx, s.s.my)) {
-    case 1: return go(k_residual_project_fx<NB, 1, false>);
-    case 2: return go(k_residual_project_fx<NB, 2, false>);
-    default: return s.on ? go(k_residual_project_fx<NB, 4, true>) : go(k_residual_project_fx<NB, 4, false>);
-  }
-}
-template <int NB>
-cudaError_t rp_launch(const StencilView32& s, const CCView32& c, const float2* u, const float2* f, cudaStream_t st) {
+template <int NB, class C>
+cudaError_t rp_launch(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f, cudaStream_t st) {
   auto go = [&](auto kern) {
     return mgc_launch(kern, dim3(cc_tiles_x(s.mx), cc_tiles_y(s.mx, s.my)), dim3(TX, WY), 0, st, s, c, u, f);
   };
-  switch (cc_tile_rows(s.mx, s.my)) {
-    case 1: return go(k_residual_project<NB, 1, float2>);
-    case 2: return go(k_residual_project<NB, 2, float2>);
-    default: return go(k_residual_project<NB, 4, float2>);
-  }
+  const int rows = cc_tile_rows(s.mx, s.my);
+  if constexpr (sizeof(C) == sizeof(cplx))
+    return rows == 1 ? go(k_residual_project_fx<NB, 1>)
+                     : rows == 2 ? go(k_residual_project_fx<NB, 2>) : go(k_residual_project_fx<NB, 4>);
+  else
+    return rows == 1 ? go(k_residual_project<NB, 1, C>)
+                     : rows == 2 ? go(k_residual_project<NB, 2, C>) : go(k_residual_project<NB, 4, C>);
 }
 
 template <int NB, class C>
@@ -710,26 +655,20 @@ int cc_tiles_y(int mx, int my) {
   return (my + ty - 1) / ty;
 }
 
-template <class S, class V, class C>
-static cudaError_t residual_project(const S& s, const V& c, const C* u, const C* f, cudaStream_t st) {
+template <class C>
+cudaError_t launch_residual_project(const StencilViewT<C>& s, const CCViewT<C>& c, const C* u, const C* f,
+                                    cudaStream_t st) {
   switch (c.nb) {
-    case 1: return rp_launch<1>(s, c, u, f, st);
-    case 2: return rp_launch<2>(s, c, u, f, st);
-    case 3: return rp_launch<3>(s, c, u, f, st);
-    case 4: return rp_launch<4>(s, c, u, f, st);
-    case 5: return rp_launch<5>(s, c, u, f, st);
-    case 6: return rp_launch<6>(s, c, u, f, st);
-    case 7: return rp_launch<7>(s, c, u, f, st);
-    case 8: return rp_launch<8>(s, c, u, f, st);
+    case 1: return rp_launch<1, C>(s, c, u, f, st);
+    case 2: return rp_launch<2, C>(s, c, u, f, st);
+    case 3: return rp_launch<3, C>(s, c, u, f, st);
+    case 4: return rp_launch<4, C>(s, c, u, f, st);
+    case 5: return rp_launch<5, C>(s, c, u, f, st);
+    case 6: return rp_launch<6, C>(s, c, u, f, st);
+    case 7: return rp_launch<7, C>(s, c, u, f, st);
+    case 8: return rp_launch<8, C>(s, c, u, f, st);
   }
   return cudaErrorInvalidValue;
-}
-cudaError_t launch_residual_project(const StencilFx& s, const CCView& c, const cplx* u, const cplx* f, cudaStream_t st) {
-  return residual_project(s, c, u, f, st);
-}
-cudaError_t launch_residual_project(const StencilView32& s, const CCView32& c, const float2* u, const float2* f,
-                                    cudaStream_t st) {
-  return residual_project(s, c, u, f, st);
 }
 
 template <class C>
@@ -803,6 +742,8 @@ cudaError_t launch_cccs_correct(const CCViewT<C>& c, C* u, cudaStream_t st) {
 }
 
 #define MGC_INSTANTIATE(C)                                                                                  \
+  template cudaError_t launch_residual_project<C>(const StencilViewT<C>&, const CCViewT<C>&, const C*,    \
+                                                 const C*, cudaStream_t);                               \
   template cudaError_t launch_reduce_projections<C>(const CCViewT<C>&, cudaStream_t);                     \
   template cudaError_t launch_cccs_correct<C>(const CCViewT<C>&, C*, cudaStream_t);
 MGC_INSTANTIATE(double2)

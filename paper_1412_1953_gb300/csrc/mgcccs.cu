@@ -9,7 +9,7 @@
 #include <new>
 #include <vector>
 
-#include "stencil_fx.cuh"
+#include "common.cuh"
 
 namespace {
 
@@ -22,8 +22,6 @@ struct LevelBufs {
   cplx *D, *Dinv;
   cplx *u, *f, *t, *r;     // level 0: only t, r (u and f belong to the caller)
   StencilView sv;
-  StencilFx fx;            // the complex128 operator as limbs (fx.on: the integer passes apply)
-  int4* fxbuf;
   // complex64 copies for the mixed-precision preconditioner (precision == 1)
   float2 *west_x32, *east_x32, *west_y32, *east_y32, *D32, *Dinv32;
   float2 *u32, *f32, *t32, *r32;
@@ -55,7 +53,6 @@ struct mgcccs_handle {
   int norm_nparts;
   double* norm_out;
   int* status;
-  int* fxlim;               // exponent ranges of the levels (setup)
   cplx *hu, *hf;
   cplx* wdot_part;         // partials of the weighted dot products
   // mixed precision: complex64 states, projections and GMRES basis; FP64 outer residual
@@ -150,9 +147,6 @@ void layout(mgcccs_handle* h, Carver& cv) {
     b.Dinv = cv.take<cplx>(n2);
     b.t = cv.take<cplx>(n2);
     b.r = cv.take<cplx>(n2);
-    // limbs for the levels that smooth (a mixed-precision handle smooths in complex64), if large
-    const bool fx = p.precision == 0 && (l == 0 || l + 1 < L) && (long long)b.mx * b.my >= FX_NODES;
-    b.fxbuf = fx ? cv.take<int4>(level_fx_entries(b.mx, b.my)) : nullptr;
     if (l > 0) {
       b.u = cv.take<cplx>(n2);
       b.f = cv.take<cplx>(n2);
@@ -285,7 +279,6 @@ void layout(mgcccs_handle* h, Carver& cv) {
   }
   h->norm_part = cv.take<double>(h->norm_nparts);
   h->norm_out = cv.take<double>(4);
-  h->fxlim = cv.take<int>(FX_LIMITS * MGC_MAX_LEVELS);
   h->status = cv.take<int>(8);   // error bits, three flags, then the dense inverse's check (below)
   h->hu = cv.take<cplx>((size_t)mx * my);
   h->hf = cv.take<cplx>((size_t)mx * my);
@@ -422,24 +415,6 @@ int do_setup(mgcccs_handle* h, const cplx* v1, const cplx* v2, const cplx* v12, 
       s.rbox = complex_seen ? 0 : 1;
     }
   }
-  // the levels' operators as limbs, where their exponents allow it
-  int lim[FX_LIMITS * MGC_MAX_LEVELS];
-  for (int l = 0; l < h->L; ++l) {
-    if (!h->lv[l].fxbuf) continue;
-    MGC_LAUNCH(launch_level_exponents(h->lv[l].sv, h->fxlim + FX_LIMITS * l, st));
-    h->launches += 6;
-  }
-  if (!h->mixed) {
-    MGC_CUDA(cudaMemcpyAsync(lim, h->fxlim, sizeof(int) * FX_LIMITS * h->L, cudaMemcpyDeviceToHost, st));
-    MGC_CUDA(cudaStreamSynchronize(st));
-  }
-  for (int l = 0; l < h->L; ++l) {
-    LevelBufs& b = h->lv[l];
-    if (b.fxbuf) MGC_CUDA(level_fx(b.sv, lim + FX_LIMITS * l, b.fxbuf, &b.fx, st));
-    else b.fx = StencilFx{};
-    b.fx.s = b.sv;
-    if (b.fx.on) h->launches += 6;
-  }
   if (h->coarse_bp) {
     MGC_LAUNCH(launch_bpcr_setup(h->lv[h->L - 1].sv, h->bp_fac, h->bp_scr, h->status, st));
   } else {
@@ -546,6 +521,11 @@ const CCViewT<cplx>& cc_view<cplx>(mgcccs_handle* h) { return h->cc; }
 template <>
 const CCViewT<float2>& cc_view<float2>(mgcccs_handle* h) { return h->cc32; }
 
+// One V-cycle on level l.  `u` holds the initial guess unless zero_init; the result is
+// returned in *out (either u or the level's t buffer).
+// Whether level passes are fused (zero-start sweep + residual + restriction; prolongation +
+// first post-smoothing sweep): always for complex64, whose FP32 work is cheap; for
+// complex128 below 512^2 nodes, where launch latency outweighs the halo recomputation.
 // The coarsest-level solve u = A_c^{-1} f: the dense inverse, or block cyclic reduction
 // for coarsest grids beyond MGC_MAX_COARSE unknowns.
 template <class C>
@@ -555,42 +535,11 @@ cudaError_t coarse_solve(mgcccs_handle* h, const C* f, C* u, cudaStream_t st) {
   return launch_coarse_solve(h->nc, h->Ainv, f, u, st);
 }
 
-// Whether level passes are fused (zero-start sweep + residual + restriction; prolongation +
-// first post-smoothing sweep): always for complex64, whose FP32 work is cheap; for
-// complex128 below 512^2 nodes, where launch latency outweighs the halo recomputation.
 template <class C>
 bool fuse_level(const LevelIO<C>& b) {
   return sizeof(C) == sizeof(float2) || (long long)b.mx * b.my < 512LL * 512;
 }
 
-// Whether level l's complex128 passes run on the integer pipes; there they are always fused.
-template <class C>
-bool level_on_fx(mgcccs_handle* h, int l) {
-  return sizeof(C) == sizeof(cplx) && h->lv[l].fx.on;
-}
-// The level passes: zero-start sweep (zero), residual and restriction; prolongation and sweep;
-// operator.
-template <class C>
-cudaError_t level_down(mgcccs_handle* h, int l, const C* f, C* u, C* fc, bool zero) {
-  if constexpr (sizeof(C) == sizeof(cplx))
-    if (h->lv[l].fx.on) return launch_zrr_fx(h->lv[l].fx, f, u, fc, zero, h->st);
-  return launch_zero_residual_restrict(*level_io<C>(h, l).sv, f, u, fc, zero, h->st);
-}
-template <class C>
-cudaError_t level_up(mgcccs_handle* h, int l, const C* ec, const C* u, C* o, const C* f) {
-  if constexpr (sizeof(C) == sizeof(cplx))
-    if (h->lv[l].fx.on) return launch_pj_fx(h->lv[l].fx, ec, u, o, f, h->st);
-  return launch_prolong_jacobi(*level_io<C>(h, l).sv, ec, u, o, f, h->st);
-}
-template <class C>
-cudaError_t fine_apply(mgcccs_handle* h, const C* x, C* y) {
-  if constexpr (sizeof(C) == sizeof(cplx))
-    if (h->lv[0].fx.on) return launch_apply_fx(h->lv[0].fx, x, y, h->st);
-  return launch_apply(*level_io<C>(h, 0).sv, x, y, h->st, (double*)nullptr);
-}
-
-// One V-cycle on level l.  `u` holds the initial guess unless zero_init; the result is
-// returned in *out (either u or the level's t buffer).
 template <class C>
 int vcycle_rec(mgcccs_handle* h, int l, C* u, const C* f, bool zero_init, C** out) {
   MgcRange nvtx_range(mgc_level_range_name(l));
@@ -605,17 +554,10 @@ int vcycle_rec(mgcccs_handle* h, int l, C* u, const C* f, bool zero_init, C** ou
   C* oth = b.t;
   bool zero = zero_init;
   LevelIO<C> c = level_io<C>(h, l + 1);
-  const bool on_fx = level_on_fx<C>(h, l), fuse = on_fx || fuse_level(b);
-  if (on_fx && zero && h->p.nu1 == 1 && l == 0 && h->pend_norm2) {
-    // the Krylov vector f = w is normalised first (see issue_arnoldi_step): the fused pass below
-    // from a normalised f beats the two that normalise on the way (17 + 47 us at 1023^2)
-    MGC_LAUNCH(launch_scale_by_norm((long long)b.mx * b.my, f, const_cast<C*>(f), h->pend_norm2, (cplx*)nullptr,
-                                    krylov_blocks((long long)b.mx * b.my, 8), st));
-    h->pend_norm2 = nullptr;
-  }
+  const bool fuse = fuse_level(b);
   if (fuse && zero && h->p.nu1 == 1 && !(l == 0 && h->pend_norm2)) {
     // the zero-start sweep, residual and restriction in one pass
-    MGC_LAUNCH(level_down<C>(h, l, f, oth, c.f, true));
+    MGC_LAUNCH(launch_zero_residual_restrict(*b.sv, f, oth, c.f, true, st));
     cur = oth;
     oth = u;
   } else {
@@ -637,7 +579,7 @@ int vcycle_rec(mgcccs_handle* h, int l, C* u, const C* f, bool zero_init, C** ou
       MGC_CUDA(cudaMemsetAsync(cur, 0, sizeof(C) * (size_t)b.mx * b.my, st));
     }
     // the residual and the restriction in one pass
-    MGC_LAUNCH(level_down<C>(h, l, f, cur, c.f, false));
+    MGC_LAUNCH(launch_zero_residual_restrict(*b.sv, f, cur, c.f, false, st));
   }
   C* ec = nullptr;
   int rc = vcycle_rec<C>(h, l + 1, c.u, c.f, true, &ec);
@@ -650,7 +592,7 @@ int vcycle_rec(mgcccs_handle* h, int l, C* u, const C* f, bool zero_init, C** ou
     }
   } else {
     // the prolongation and the first post-smoothing sweep in one pass
-    MGC_LAUNCH(level_up<C>(h, l, (const C*)ec, (const C*)cur, oth, f));
+    MGC_LAUNCH(launch_prolong_jacobi(*b.sv, (const C*)ec, (const C*)cur, oth, f, st));
     C* tmp = cur; cur = oth; oth = tmp;
   }
   for (int s = 1; s < h->p.nu2; ++s) {
@@ -677,10 +619,7 @@ template <class C>
 int cccs_fine(mgcccs_handle* h, C* u, const C* f) {
   cudaStream_t st = h->st;
   const CCViewT<C>& cc = cc_view<C>(h);
-  if constexpr (sizeof(C) == sizeof(cplx))
-    MGC_LAUNCH(launch_residual_project(h->lv[0].fx, cc, (const C*)u, f, st));
-  else
-    MGC_LAUNCH(launch_residual_project(h->lv[0].sv32, cc, (const C*)u, f, st));
+  MGC_LAUNCH(launch_residual_project(*level_io<C>(h, 0).sv, cc, (const C*)u, f, st));
   MGC_LAUNCH(launch_reduce_projections(cc, st));
   MGC_LAUNCH(launch_channel_solve(h->crA, h->crB, st));
   MGC_LAUNCH(launch_cccs_correct(cc, u, st));
@@ -820,7 +759,7 @@ int issue_arnoldi_step(mgcccs_handle* h, int j) {
   h->pend_norm2 = nullptr;
   if (rc) return rc;
   // w = A z_j
-  MGC_LAUNCH(fine_apply<C>(h, (const C*)zj, w));
+  MGC_LAUNCH(launch_apply(s0, (const C*)zj, w, st, (double*)nullptr));
   // Gram-Schmidt, first pass: H(0:j, j) = V^H w ; w -= V H(0:j, j).  w is column j+1 of V,
   // so the multi-dot over columns 0..j+1 also yields |w|^2 (for the reorthogonalisation
   // test), left in H(j+1, j) until the Givens rotation writes that entry.
@@ -1597,7 +1536,7 @@ int mgcccs_precond_apply(mgcccs_t h, mgcccs_c128* z, const mgcccs_c128* r) {
 int mgcccs_matvec(mgcccs_t h, const mgcccs_c128* x, mgcccs_c128* y) {
   mgc_not_a_kernel();   // the caller's stream: start a new chain of programmatic launches
   if (!h || !x || !y || (const void*)x == (const void*)y) return MGCCCS_EINVAL;
-  MGC_LAUNCH(fine_apply<cplx>(h, reinterpret_cast<const cplx*>(x), reinterpret_cast<cplx*>(y)));
+  MGC_LAUNCH(launch_apply(h->lv[0].sv, reinterpret_cast<const cplx*>(x), reinterpret_cast<cplx*>(y), h->st));
   return MGCCCS_OK;
 }
 
@@ -1816,13 +1755,6 @@ int mgcccs_axis_spectrum(mgcccs_t h, int axis, int method, mgcccs_c128* lam_host
 
 int mgcccs_eig_fallbacks(mgcccs_t h) { return h ? h->eig_fallbacks : -1; }
 
-int mgcccs_integer_passes(mgcccs_t h, unsigned* levels) {
-  if (!h || !levels) return MGCCCS_EINVAL;
-  *levels = 0;
-  for (int l = 0; l < h->L; ++l) *levels |= h->lv[l].fx.on ? 1u << l : 0u;
-  return MGCCCS_OK;
-}
-
 int mgcccs_set_solve_driver(mgcccs_t h, int driver) {
   if (!h || (driver != MGCCCS_DRIVER_GRAPH && driver != MGCCCS_DRIVER_HOST)) return MGCCCS_EINVAL;
   h->driver = driver;
@@ -1835,7 +1767,6 @@ int mgcccs_set_tile_rows(mgcccs_t h, int rows) {
   for (int l = 0; l < h->L; ++l) {
     h->lv[l].sv.tile_rows = rows;
     h->lv[l].sv32.tile_rows = rows;
-    h->lv[l].fx.s.tile_rows = rows;
   }
   // the cached graphs hold the old launch shapes
   for (int j = 0; j < MGC_MAX_RESTART; ++j) {

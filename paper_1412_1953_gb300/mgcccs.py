@@ -65,7 +65,6 @@ _SIGS = {
     "mgcccs_set_tile_rows": (_i, [_vp, _i]),
     "mgcccs_axis_spectrum": (_i, [_vp, _i, _i, _vp]),
     "mgcccs_eig_fallbacks": (_i, [_vp]),
-    "mgcccs_integer_passes": (_i, [_vp, ctypes.POINTER(ctypes.c_uint)]),
     "mgcccs_batch_create": (_i, [ctypes.POINTER(_vp), ctypes.POINTER(_vp), _i, ctypes.POINTER(_vp),
                                  ctypes.POINTER(_vp), _vp]),
     "mgcccs_batch_run": (_i, [_vp, _d, _i, ctypes.POINTER(_i), ctypes.POINTER(_d), ctypes.POINTER(_i)]),
@@ -408,12 +407,6 @@ class Solver:
 
     def eig_fallbacks(self) -> int:
         return int(lib().mgcccs_eig_fallbacks(self.h))
-
-    def integer_passes(self):
-        """Levels whose complex128 passes multiply on the integer pipes (see include/mgcccs.h)."""
-        bits = ctypes.c_uint(0)
-        _check(lib().mgcccs_integer_passes(self.h, ctypes.byref(bits)), "mgcccs_integer_passes")
-        return [l for l in range(self.p.levels) if bits.value >> l & 1]
 
     def set_tile_rows(self, rows: int):
         """Block height of the passes on the levels too small to fill the GPU (2, 4, 8; 0 =

@@ -1,5 +1,6 @@
-"""Where the complex128 passes on the integer pipes apply: which levels setup puts there, operators
-whose updates do not fit 64 bits, and operands of very different size inside a tile."""
+"""Complex128 results entry by entry, on operands of very different size side by side and on operators
+with a small or widely spread diagonal: passes that sum on a common exponent must not lose what is
+small beside what is large."""
 import math
 
 import numpy as np
@@ -50,24 +51,12 @@ def _composed(sv, levels, f, u, nu1, nu2):
     return e.reshape(u.shape)
 
 
-# 60000 nodes and more: 255 x 255, 511 x 511 with 255 x 255, 591 x 431 with 295 x 215; a coarsest level multiplies
-# nothing itself; one large potential value spreads the fine diagonal
-@pytest.mark.parametrize("nx,ny,levels,spike,on", [(240, 240, 4, 0.0, []), (256, 256, 4, 0.0, [0]),
-                                                   (512, 512, 5, 0.0, [0, 1]), (592, 432, 5, 0.0, [0, 1]),
-                                                   (592, 432, 5, 1e6, [1])])
-def test_levels_on_the_integer_pipes(nx, ny, levels, spike, on):
-    sv = _solver(_problem(nx, ny), levels, spike)
-    assert sv.integer_passes() == on
-    sv.close()
-
-
 # An energy near the diagonal's 2/h^2, or a large omega, makes |omega/D| times a row's coefficients
-# large: 14, 47, 72 and 32, where the integers of the prolongation and sweep hold an update of up to 30.
+# large: 14, 47, 72 and 32 against 2.7 (an update in 64-bit integers on v's unit wraps beyond 30).
 # The two forms agree to 1e-13 at 2.7 (test_gpu_fixed_stencils.py); a sweep on either level amplifies a
 # difference by this factor, 72/2.7 squared: 1e-10.
-@pytest.mark.parametrize("E,omega,on", [(130.0, 2 / 3, True), (135.0, 2 / 3, False), (140.0, 2 / 3, False),
-                                        (0.5, 8.0, False)])
-def test_updates_beyond_64_bits(E, omega, on):
+@pytest.mark.parametrize("E,omega", [(130.0, 2 / 3), (135.0, 2 / 3), (140.0, 2 / 3), (0.5, 8.0)])
+def test_updates_beyond_64_bits(E, omega):
     prob = _problem(256, 256, E=E)
     sv = _solver(prob, 3, omega=omega, nu1=0, nu2=1)
     f = torch.full(prob.f.shape, 1e-3, dtype=torch.complex128, device="cuda")
@@ -77,15 +66,13 @@ def test_updates_beyond_64_bits(E, omega, on):
         sv.vcycle(u, f)
         ref = _composed(sv, 3, f, u0, 0, 1)
         assert float((u - ref).abs().max() / ref.abs().max()) <= 1e-10
-    assert (0 in sv.integer_passes()) == on
     sv.close()
 
 
-# Cells of aspect 1 to 4: the coefficients spread over 3 to 6 powers of two, and 57 bits of the largest
-# keep a double's 53 of all within four.  A unit vector's image is a column of coefficients: to half a
+# Cells of aspect 1 to 4: the coefficients spread over 3 to 6 powers of two.  A unit vector's image is a column of coefficients: to half a
 # unit of 2^-53 of its modulus in either part (the larger one exact), exact in the real box.
-@pytest.mark.parametrize("nx,ny,on", [(256, 256, True), (512, 256, True), (768, 256, False), (1024, 256, False)])
-def test_coefficients_keep_their_bits(nx, ny, on):
+@pytest.mark.parametrize("nx,ny", [(256, 256), (512, 256), (768, 256), (1024, 256)])
+def test_coefficients_keep_their_bits(nx, ny):
     prob = _problem(nx, ny)
     sv = _solver(prob, 5)
     x = torch.zeros(prob.f.shape, dtype=torch.complex128, device="cuda")
@@ -97,7 +84,6 @@ def test_coefficients_keep_their_bits(nx, ny, on):
     assert bool((d <= 2.0 ** -54 * r.abs()).all())
     box = (slice(0, ny * 2 // 3 - 2), slice(0, nx * 2 // 3 - 2))
     assert bool((y[box] == -r[box]).all())
-    assert (0 in sv.integer_passes()) == on
     sv.close()
 
 
@@ -116,35 +102,6 @@ def test_cycle_is_odd(nx, ny, levels, nu1, nu2):
     sv.precond_apply(z, f)
     sv.precond_apply(zm, -f)
     assert bool((u == -v).all()) and bool((z == -zm).all())
-    assert 0 in sv.integer_passes()
-    sv.close()
-
-
-def test_inner_coefficients_are_split_about_zero():
-    """A sum drops the products of low limbs, of at most 2^28 each: a quarter of the unit of the sum.  The
-    box is such that the inner coefficient's low limb is near a multiple of 2^29, the constant field such that twice
-    its value has a low limb near 2^28: split from zero up, the four dropped products would make a whole unit; about zero
-    they vanish, and a quarter remains for the diagonal's, with the rounding of a double of E u."""
-    n = 256
-    u = ((700000001 << 28) + (1 << 27) - 32) * 2.0 ** -57
-    assert 1.0 <= u < 2.0
-    for L in np.linspace(29.0, 31.0, 20001):
-        c, ec = 0.5 / (L / n) ** 2, 1023 + math.frexp(2.0 / (L / n) ** 2)[1] - 1
-        if int(math.ldexp(c, 1079 - ec)) % (1 << 29) >= (1 << 29) - (1 << 20):
-            break
-    prob = inputs.free_problem(n, L, 2 * L / 3, math.pi / 6, 0.5, np.zeros((n - 1, n - 1), dtype=complex))
-    sv = _solver(prob, 4)
-    x = torch.full((n - 1, n - 1), u, dtype=torch.complex128, device="cuda")
-    y, r = torch.empty_like(x), torch.empty_like(x)
-    sv.matvec(x, y)
-    one = torch.zeros_like(x)
-    one[1::2, 1::2] = 1.0                            # the diagonal, and one axis' coefficients beside it
-    sv.level_residual(0, one.reshape(-1), torch.zeros_like(x).reshape(-1), r.reshape(-1))
-    i = np.arange(9, 129, 2)
-    D, w = (-r[j, 65].real.cpu().numpy().astype(np.longdouble) for j in (i, i + 1))
-    off = np.abs(y[i, 65].real.cpu().numpy() - u * (D + 2 * w))   # w: the south and north neighbours' sum
-    assert off.max() <= 0.5 * 2.0 ** (1023 + ec - 2101)
-    assert 0 in sv.integer_passes()
     sv.close()
 
 
@@ -174,9 +131,7 @@ def _moduli(A, v, f=0.0):
     return np.abs(f) + _apply([np.abs(a) for a in A], np.abs(v))
 
 
-# A sum takes the integer pipes where some value of it keeps 53 bits: five values to half a unit and ten
-# dropped products to a quarter of the smallest coefficient's are 22 units of 2^-53 of the sum of moduli, 32 with
-# cells that are not square; FP64 instructions are within 14.
+# Ten multiply-adds a part are within 14 units of 2^-53 of the sum of moduli; up to 32 for sums in integers.
 @pytest.mark.parametrize("kind", FIELDS)
 def test_operator_entry_by_entry(kind):
     prob = _problem(320, 256)
@@ -223,7 +178,6 @@ def test_cycle_beside_spikes(nu1, nu2):
         sv.precond_apply(z, fd)
         ref = _composed(sv, 4, fd, torch.zeros_like(fd), nu1, nu2)
         assert bool(((z - ref).abs() <= 1e-12 * near(ref))[far].all())
-    assert 0 in sv.integer_passes()
     sv.close()
 
 
@@ -245,7 +199,6 @@ def test_parts_of_different_size(nu1, nu2):
     sv.vcycle(u, join(f, 2.0 ** 79))
     sv.vcycle(v, join(f, 2.0 ** 9))
     assert float((u.imag - v.imag).abs().max() / v.imag.abs().max()) <= 1e-13
-    assert 0 in sv.integer_passes()
     sv.close()
 
 
