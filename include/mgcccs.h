@@ -136,6 +136,8 @@ int mgcccs_vcycle(mgcccs_t h, mgcccs_c128* u, const mgcccs_c128* f);
  * residual r = f - (H-E)u, projections onto the bound states with the
  * conventions of Eqs. (25)-(27), the coupled-channel solves of Eqs. (28)-(29)
  * for the error, and u += sum_m e^A_m(y) phi_m(x) + sum_l e^B_l(x) vphi_l(y).
+ * Complex128 projections and the correction are summed as integers where that keeps each sum's own
+ * terms to a double's bits (relative to their moduli), else with FP64 instructions.
  * Requires n_b > 0.  Async. */
 int mgcccs_cccs(mgcccs_t h, mgcccs_c128* u, const mgcccs_c128* f);
 
@@ -328,9 +330,10 @@ int mgcccs_fp64_probe(int blocks, int iters, double m, double b, double* out, vo
  * V: device, k vectors of (nx-1)*(ny-1) values, vector i at V + i*ld (ld >= (nx-1)*(ny-1));
  * w: device, (nx-1)*(ny-1) values (gs_update overwrites it); out, coef: device, k values.
  * A vector V_i that is w itself (same address) gives out[i] = |w|^2.  Products are summed as
- * integers of 57 bits on a common exponent, or with FP64 instructions out of their range, to the
- * accuracy of FP64 sums, in a fixed order (per-block partials, then one block), so repeated calls
- * give identical results.  mgcccs_gs_dots needs a handle set up with krylov_restart >= 1 and
+ * integers of 59 bits on a common exponent, or with FP64 instructions where one exponent does not do
+ * for a sum's terms: a dot product is within a few units of 2^-53 of the sum of its terms' moduli, an
+ * entry of the update within (8 k + 16) of its own, as with FP64 multiply-adds.  The order is fixed
+ * (per-block partials, then one block), so repeated calls give identical results.  mgcccs_gs_dots needs a handle set up with krylov_restart >= 1 and
  * k <= krylov_restart + 1 (it uses the handle's partial-sum buffer); mgcccs_gs_update
  * takes 1 <= k <= 61.  Async.  Errors: EINVAL (null pointer, k or ld out of range), ECUDA.
  */

@@ -17,8 +17,14 @@
 // dropped must have no mean, or a long sum that cancels keeps it, so low limbs lie about zero and
 // conversions round without a preference.  (With low limbs of the operands' signs and cut conversions, a dot product of
 // 1023^2 skewed, nearly cancelling terms was 1e-17 to 1e-16 |v| |w| off its 64-bit value, and 2e-19
-// with FP64 multiply-adds.)  Against these, which round each partial sum to 2^-53 of itself, the
-// error then stays within that of the same sum (measured at each kernel).
+// with FP64 multiply-adds.)
+//
+// An operand far below the one whose exponent it shares has fewer bits than its double, so a sum on a
+// common exponent is good to the largest operands' scale, not to its own terms', where these are
+// small.  Each kernel therefore looks for a term near the largest, and takes FP64 instructions for the chunk,
+// tile or entry that has none: within 2^-FX_NEAR with 57 bits, 2^-6 with 59 (U_NEAR, C_NEAR), so that the
+// roundings of FP64 multiply-adds of the same terms are no smaller.  That costs a few instructions a
+// product; the stencils, with few products a value, lost to it what the integers gave and are FP64.
 //
 // Largest exponents outside FX_MIN..FX_MAX (nothing but zeros and subnormals, huge, infinite or
 // NaN operands) take the FP64 instructions; fx_ok tells.
@@ -29,8 +35,7 @@ constexpr int FX_MIN = 600, FX_MAX = 1446;       // biased exponents; a product'
 constexpr int FX_TERMS = 8;                      // complex terms between two roundings
 constexpr int FX_TERMS_59 = 6;                   // the same for limbs of 59 bits
 
-// How many powers of two below the largest operands' an integer sum's own largest term may lie: further
-// down its conversions could leave more than the roundings of FP64 instructions, which then take it.
+// How many powers of two below the largest operands' product a sum's own largest term may lie.
 constexpr int FX_NEAR = 4;
 
 __device__ __forceinline__ int fx_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -69,9 +74,11 @@ __device__ __forceinline__ void fx_mac(FxSum& s, FxLimbs a, FxLimbs b) {
   s.mid += (long long)a.l * b.h;
 }
 // Carry the middle sum into the upper one, so that FX_TERMS more terms fit (the upper sum itself
-// holds 4 FX_TERMS terms).
+// holds 4 FX_TERMS terms, of 59 bits 2 FX_TERMS_59).
+template <int X = 0>
 __device__ __forceinline__ void fx_carry(FxSum& s) {
-  s.hh += (s.mid + (1LL << 28)) >> 29;
+  constexpr int S = 29 + X / 2;
+  s.hh += (s.mid + (1LL << (S - 1))) >> S;
   s.mid = 0;
 }
 // (re, im) += a b for complex a = (ax, ay), b = (bx, by).
@@ -83,8 +90,9 @@ __device__ __forceinline__ void fx_cmac(FxSum& re, FxSum& im, int4 a, int4 b) {
   fx_mac(im, ay, bx);
 }
 __device__ __forceinline__ int fx_exp(cplx z) { return max(fx_exp(z.x), fx_exp(z.y)); }
+template <int X = 0>
 __device__ __forceinline__ int4 fx_limbs(cplx z, int E, int down = 0) {
-  const FxLimbs x = fx_limbs(z.x, fx_exp(z.x), E, down), y = fx_limbs(z.y, fx_exp(z.y), E, down);
+  const FxLimbs x = fx_limbs<X>(z.x, fx_exp(z.x), E, down), y = fx_limbs<X>(z.y, fx_exp(z.y), E, down);
   return make_int4(x.h, x.l, y.h, y.l);
 }
 // acc + the sum of products with exponents that add up to E2, rounded; the sum is cleared.

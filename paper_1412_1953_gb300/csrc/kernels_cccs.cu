@@ -518,10 +518,12 @@ __global__ void __launch_bounds__(256) k_cccs_correct(int mx, int my, const C* _
 // exponent over the block, and aligns the 2 n_b products to the largest of their exponents by
 // shifting e^A and vphi on conversion; a node then takes 24 n_b integer multiply-adds and four
 // FP64 instructions (two conversions, two additions) against 8 n_b FP64 instructions.
-// A node whose products and value of u all lie below 2^-FX_NEAR of the tile's largest product takes
-// the FP64 multiply-adds, and so does a tile out of the integer range.
-// 1023^2, n_b = 3: 45.0 us with FP64 multiply-adds, 17.4 us so; 127^2: 9.6 and, with RT = 1, 4.5 us
+// Limbs of 59 bits; a node whose products and value of u all lie below 2^-C_NEAR of the tile's largest
+// product takes the FP64 multiply-adds, and so does a tile out of the integer range.
+// 1023^2, n_b = 3: 45.0 us with FP64 multiply-adds, 22 us so; 127^2: 9.6 and, with RT = 1, 4.5 us
 // (cold L2).
+constexpr int C_NEAR = 6;
+
 template <int NB, int RT>
 __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const cplx* __restrict__ phi,
                                                          const cplx* __restrict__ vphi, const cplx* __restrict__ eA,
@@ -556,26 +558,28 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
     E2 = max(E2, ec[p] + er[p]);
     ok = ok && fx_ok(ec[p]) && fx_ok(er[p]);
   }
-  const auto plain = [&](int r) {
-    const int j = jt + r;
-    cplx w = v[r];
-    for (int m = 0; m < NB; ++m) w = cfma(__ldg(phi + m * mx + i), __ldg(eA + m * my + j), w);
-    for (int l = 0; l < NB; ++l) w = cfma(__ldg(eB + l * mx + i), __ldg(vphi + l * my + j), w);
-    u[(size_t)j * mx + i] = w;
+  // the rows of `which` with FP64 instructions, from the arrays
+  const auto plain = [&](unsigned which) {
+#pragma unroll 1
+    for (; which; which &= which - 1) {
+      const int j = jt + __ffs(which) - 1;
+      if (j >= my) break;
+      cplx w = u[(size_t)j * mx + i];
+      for (int m = 0; m < NB; ++m) w = cfma(__ldg(phi + m * mx + i), __ldg(eA + m * my + j), w);
+      for (int l = 0; l < NB; ++l) w = cfma(__ldg(eB + l * mx + i), __ldg(vphi + l * my + j), w);
+      u[(size_t)j * mx + i] = w;
+    }
   };
   if (!ok) {
-    if (i >= mx) return;
-#pragma unroll
-    for (int r = 0; r < RT; ++r)
-      if (jt + r < my) plain(r);
+    if (i < mx) plain((1u << RT) - 1);
     return;
   }
   for (int p = wy; p < 4 * NB; p += 8) {
     const int q = p >> 1;
     if (p & 1) {
-      if (lane < TYC) row[q][lane] = fx_limbs(value(q, 1), E2 - ec[q]);
+      if (lane < TYC) row[q][lane] = fx_limbs<2>(value(q, 1), E2 - ec[q]);
     } else {
-      col[q][lane] = fx_limbs(value(q, 0), ec[q]);
+      col[q][lane] = fx_limbs<2>(value(q, 0), ec[q]);
     }
   }
   __syncthreads();
@@ -583,29 +587,29 @@ __global__ void __launch_bounds__(256) k_cccs_correct_fx(int mx, int my, const c
   int4 a[2 * NB];
 #pragma unroll
   for (int p = 0; p < 2 * NB; ++p) a[p] = col[p][lane];
+  unsigned low = 0;                                      // rows left to FP64 instructions
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
     if (jt + r >= my) break;
     int k = fx_exp(v[r]) + 1023;
-    if (k < E2 - FX_NEAR) {
-#pragma unroll
+    if (k < E2 - C_NEAR)
       for (int p = 0; p < 2 * NB; ++p) k = max(k, xc[p][lane] + xr[p][wy * RT + r]);
-      if (k < E2 - FX_NEAR) {
-        plain(r);
-        continue;
-      }
-    }
     FxSum re{0, 0}, im{0, 0};
 #pragma unroll
     for (int p = 0; p < 2 * NB; ++p) {
       fx_cmac(re, im, a[p], row[p][wy * RT + r]);
-      if (p + 1 == FX_TERMS) {
-        fx_carry(re);
-        fx_carry(im);
+      if (p + 1 == 2 * FX_TERMS_59 && p + 1 < 2 * NB) {  // the upper sum holds no more of 59 bits
+        v[r].x = fx_flush<2>(re, E2, v[r].x);
+        v[r].y = fx_flush<2>(im, E2, v[r].y);
+      } else if ((p + 1) % FX_TERMS_59 == 0) {
+        fx_carry<2>(re);
+        fx_carry<2>(im);
       }
     }
-    u[(size_t)(jt + r) * mx + i] = cmk(fx_flush(re, E2, v[r].x), fx_flush(im, E2, v[r].y));
+    if (k < E2 - C_NEAR) low |= 1u << r;
+    else u[(size_t)(jt + r) * mx + i] = cmk(fx_flush<2>(re, E2, v[r].x), fx_flush<2>(im, E2, v[r].y));
   }
+  if (low) plain(low);
 }
 
 template <int NB, class C>
