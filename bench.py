@@ -394,7 +394,7 @@ def mixed_gs_roofline(args, rounds=10, sets=3):
 def kernel_rooflines(args, solver, stream, f_d, flush, workload_name, device_index):
     """Roofline of the Gram-Schmidt update k_multiaxpy_fx, which with the multi-dot leads a complex128
     Arnoldi step by time.  Its products are summed on the integer pipes, so the FP64 pipe is no
-    ceiling for it: it is reported against the HBM copy bandwidth.  It is timed live with CUDA events on the handle's stream over 50 launches of the same kernel
+    ceiling for it: it is bound by latency and reported against the HBM copy bandwidth.  It is timed live with CUDA events on the handle's stream over 50 launches of the same kernel
     and launch shape the solve uses, with GS_VECTORS = 11 basis vectors of the fine level
     (11 x 16.7 MB, larger than L2, so every launch streams from HBM).  Beside it: the
     Gram-Schmidt dot pass (12 vectors, w included: the first pass of step j = 10) and the

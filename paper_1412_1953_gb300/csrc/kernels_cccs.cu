@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(TX * WY) k_residual_project(StencilViewT<C> s,
 // cycles of a quarter of an SM, against 8 n_b FP64 instructions, 512 n_b cycles.  A tile with a row's
 // (column's) projection whose products all lie below 2^-FX_NEAR of the tile's largest takes the FP64
 // instructions: 3 to 7 % of the tiles of 32 rows in a solve at 512^2, up to 19 % at 256^2.  1023^2,
-// n_b = 3, cold L2: 76.6 us with FP64 instructions, 41.8 us with integer projections; 127^2: 19.2 us in tiles of 32
-// rows (16 blocks), 7.4 us in tiles of 8.
+// n_b = 3, cold L2: 76.6 us with FP64 instructions, 41.8 us with integer projections (48 in a solve); 127^2: 19.2
+// us in tiles of 32 rows (16 blocks), 7.4 us in tiles of 8.
 template <int NB, int SY>
 __global__ void __launch_bounds__(TX * WY) k_residual_project_fx(StencilView s, CCView c, const cplx* __restrict__ u,
                                                                 const cplx* __restrict__ f) {

@@ -93,8 +93,9 @@ __device__ __forceinline__ void copy_wait() {
 // vector, of one tile after another) is fetched DS - 1 chunks ahead.  About 90 instructions a
 // product and the 16 warps that 128 registers allow bound it.  1023^2, 12 vectors (12 and 1
 // of 16.7 MB read): 88.0 us with FP64 multiply-adds, 63 with 64-bit shifts of masked keys in the
-// conversion, 58 before the FP64 share, 53.7 with it, 56.9 us with conversions that leave no mean
-// (fixed.cuh; ties alternate by lane: 4 us of a pair), 3.5 TB/s.
+// conversion, 58 before the FP64 share, 53.7 with it, 56.9 with conversions that leave no mean
+// (fixed.cuh; ties alternate by lane: 4 us of a pair), 61 us with exponents that follow the chunks and
+// the look for a near product, 3.3 TB/s.
 constexpr int DG = 4, DU = 4, DS = 4, D_SLACK = 2;
 
 __global__ void __launch_bounds__(NT, 2) k_multidot_fx(long long n, int k, const cplx* __restrict__ V, long long ld,
@@ -255,8 +256,10 @@ static_assert(MULTIDOT_SMEM >= 2 * DG * NT * (int)sizeof(double), "the block sum
 // UU x 32 points at a time and fetches the chunks (w, then each vector) ahead, as above.  Points whose
 // own products and w all lie below 2^-U_NEAR of that largest product are done again with FP64
 // instructions, from the arrays: 59 bits leave them fewer than a double has.
-// 1023^2, 11 vectors: 90.1 us with FP64 multiply-adds, 50.0 us now (UU = 4; 58 with UU = 2, which
-// is the faster at 255^2: 7.6 against 11.4 us, few tiles a warp), 4.4 TB/s.
+// 1023^2, 11 random vectors: 90.1 us with FP64 multiply-adds, 50 before the look for low points (UU = 4;
+// 58 with UU = 2, which is the faster at 255^2: 7.6 against 11.4 us, few tiles a warp), 54 us now, 4.0 TB/s.
+// In a solve, where w is near its largest term and both are small at the same points, a quarter of the
+// tiles hold one, 81 against 59 us with cold L2.
 constexpr int U_NEAR = 6;
 constexpr int UF = 16;                                 // chunks in flight x points a lane
 

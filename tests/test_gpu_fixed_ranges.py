@@ -24,10 +24,8 @@ def _problem(nx, ny, E=0.5):
     return inputs.temkin_poet(nx, L=30.0, R0=20.0, theta=math.pi / 6, E=E, seed=3, ny=ny)
 
 
-def _solver(prob, levels, spike=0.0, **kw):
-    v12 = prob.v12.copy()
-    v12[prob.ny // 3, prob.nx // 5] += spike
-    return M.Solver(M.params_for(prob, levels=levels, **{"n_b": 0, **kw}), prob.v1, prob.v2, v12)
+def _solver(prob, levels, **kw):
+    return M.Solver(M.params_for(prob, levels=levels, **{"n_b": 0, **kw}), prob.v1, prob.v2, prob.v12)
 
 
 def _composed(sv, levels, f, u, nu1, nu2):
@@ -69,8 +67,9 @@ def test_updates_beyond_64_bits(E, omega):
     sv.close()
 
 
-# Cells of aspect 1 to 4: the coefficients spread over 3 to 6 powers of two.  A unit vector's image is a column of coefficients: to half a
-# unit of 2^-53 of its modulus in either part (the larger one exact), exact in the real box.
+# Cells of aspect 1 to 4: the coefficients spread over 3 to 6 powers of two.  A unit vector's image is a
+# column of coefficients: to half a unit of 2^-53 of its modulus in either part (the larger one exact),
+# exact in the real box.
 @pytest.mark.parametrize("nx,ny", [(256, 256), (512, 256), (768, 256), (1024, 256)])
 def test_coefficients_keep_their_bits(nx, ny):
     prob = _problem(nx, ny)
