@@ -420,16 +420,73 @@ __global__ void __launch_bounds__(NT, UU == 4 ? 2 : 3) k_multiaxpy_fx(long long 
 }
 constexpr int MULTIAXPY_SMEM = NT * UF * (int)sizeof(cplx);
 
-// out[i] = sum_b partial[i][b] (fixed order); acc_into[i] += out[i] when given.
+// A double in units of 2^(E - 1138) for the block's largest exponent E: below 2^116, and cut below 2^-116 of
+// the largest value only.
+__device__ __forceinline__ __int128 fixed_128(double x, int E) {
+  const int e = fx_exp(x), hi = __double2hiint(x);
+  const unsigned long long m =
+      (unsigned long long)(((unsigned)hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32 | (unsigned)__double2loint(x);
+  const __int128 v = ((__int128)m << 63) >> min(E - e, 127);
+  return hi < 0 ? -v : v;
+}
+__device__ __forceinline__ __int128 warp_sum_128(__int128 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)v, o);
+    const long long hi = __shfl_down_sync(0xffffffffu, (long long)(v >> 64), o);
+    v += (__int128)hi << 64 | lo;
+  }
+  return v;
+}
+
+// out[i] = sum_b partial[i][b]; acc_into[i] += out[i] when given.  At most 2^10 partials (krylov_blocks), added exactly as
+// 128-bit integers (FP64 additions out of the integer range): where a dot product of smooth vectors
+// cancels, rounding their sum was most of its error, 2 to 3 times that of all the products.
 __global__ void __launch_bounds__(NT) k_reduce_dots(int nblk, const cplx* __restrict__ partial,
                                                     cplx* __restrict__ out, cplx* __restrict__ acc_into) {
   mgc_pdl_enter();
   __shared__ double sh[2][NT / 32];
-  const int i = blockIdx.x;
-  cplx acc = cmk(0.0, 0.0);
-  for (int b = threadIdx.x; b < nblk; b += NT) acc = cadd(acc, partial[(size_t)i * nblk + b]);
-  cplx tot = block_sum_c<NT>(acc, sh);
-  if (threadIdx.x == 0) {
+  __shared__ __int128 part[2][NT / 32];
+  __shared__ int es;
+  const int i = blockIdx.x, t = threadIdx.x;
+  if (t == 0) es = 0;
+  __syncthreads();
+  int e = 0;
+  for (int b = t; b < nblk; b += NT) e = max(e, fx_exp(partial[(size_t)i * nblk + b]));
+  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if ((t & 31) == 0) atomicMax(&es, e);
+  __syncthreads();
+  cplx tot = cmk(0.0, 0.0);
+  const int E = es;
+  if (fx_ok(E)) {
+    __int128 x = 0, y = 0;
+    for (int b = t; b < nblk; b += NT) {
+      const cplx v = partial[(size_t)i * nblk + b];
+      x += fixed_128(v.x, E);
+      y += fixed_128(v.y, E);
+    }
+    x = warp_sum_128(x);
+    y = warp_sum_128(y);
+    if ((t & 31) == 0) { part[0][t >> 5] = x; part[1][t >> 5] = y; }
+    __syncthreads();
+    if (t == 0) {
+      const double sc = __hiloint2double((E - 1138 + 1023) << 20, 0);
+      double r[2];
+      for (int c = 0; c < 2; ++c) {
+        __int128 s = part[c][0];
+        for (int w = 1; w < NT / 32; ++w) s += part[c][w];
+        const unsigned __int128 m = s < 0 ? -s : s;
+        const double v = sc * fma((double)(unsigned long long)(m >> 64), 0x1p64, (double)(unsigned long long)m);
+        r[c] = s < 0 ? -v : v;
+      }
+      tot = cmk(r[0], r[1]);
+    }
+  } else {
+    cplx acc = cmk(0.0, 0.0);
+    for (int b = t; b < nblk; b += NT) acc = cadd(acc, partial[(size_t)i * nblk + b]);
+    tot = block_sum_c<NT>(acc, sh);
+  }
+  if (t == 0) {
     out[i] = tot;
     if (acc_into) acc_into[i] = cadd(acc_into[i], tot);
   }

@@ -273,6 +273,23 @@ def test_dots_term_by_term(nx, ny, k, kind):
     sv.close()
 
 
+
+def test_partial_sums_are_added_exactly():
+    """One product of 2^60, 1, -2^60 or 1 in each tile of 1024 points, a tile a block: the partial sums are
+    exact, and so is their sum."""
+    sv = _solver(_problem(320, 256), 5, krylov_restart=20)
+    V = np.zeros((2, sv.n), complex)
+    at = np.arange(0, sv.n, 1024)
+    V[0, at] = np.resize([2.0 ** 60, 1.0, 1.0, -2.0 ** 60], at.size)
+    V[1, at] = np.resize([1j, 2.0 ** 60, -2.0 ** 60, 3.0], at.size)
+    w = np.ones(sv.n, complex)
+    h = torch.empty(2, dtype=torch.complex128, device="cuda")
+    sv.gs_dots(torch.as_tensor(V).to("cuda"), 2, torch.as_tensor(w).to("cuda"), h)
+    assert at.size % 4 == 0
+    assert h.tolist() == [at.size / 2, at.size / 4 * (3.0 - 1j)]
+    sv.close()
+
+
 # An entry of the update is good to the roundings of its own 2 k multiply-adds a part, as FP64 instructions
 # give it, and as much again for k conversions at the guard.
 @pytest.mark.parametrize("nx,ny,k", [(32, 32, 5), (320, 256, 9), (1024, 512, 4)])
